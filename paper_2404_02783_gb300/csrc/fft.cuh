@@ -1,19 +1,25 @@
-// Register-resident FFT engine (Stockham autosort, radix 8 with one radix-4 or
-// radix-2 closing stage), compile-time length.
+// Register-resident FFT engine (Stockham autosort), compile-time length L and E elements a
+// thread.
 //
-// A length-L sequence is owned by Q = L/8 threads; thread t holds the eight
-// elements t + m Q (m = 0..7) in registers.  A stage of radix R performs 8/R
-// butterflies per thread: butterfly j = t + q Q reads elements j + r L/R,
-// multiplies by exp(-+2 pi i (j mod Ns) r / (Ns R)) and runs a register DFT of
-// size R; the result element (j / Ns) Ns R + (j mod Ns) + r Ns goes through
-// shared memory to whichever thread reads it in the next stage.  Loads of stage
-// one and stores after the last stage touch elements t + m Q, i.e. consecutive
-// threads touch consecutive elements, so callers stream them to and from global
-// memory directly.  Only the exchanges between stages use shared memory.
+// A length-L sequence is owned by Q = L/E threads; thread t holds the E elements t + m Q
+// (m = 0..E-1) in registers.  A stage of radix R <= E performs E/R butterflies per thread:
+// butterfly j = t + q Q reads elements j + r L/R, multiplies by exp(-+2 pi i (j mod Ns) r /
+// (Ns R)) and runs a register DFT of size R; the result element (j / Ns) Ns R + (j mod Ns) +
+// r Ns goes through shared memory to whichever thread reads it in the next stage.  Loads of
+// stage one and stores after the last stage touch elements t + m Q, i.e. consecutive threads
+// touch consecutive elements, so callers stream them to and from global memory directly.
 //
-// Twiddles come from a shared per-stage table (tw_stage_offset; values from the host
-// FP64 table exp(-2 pi i k / 1024), rounded once); INV conjugates them (unnormalised
-// inverse).
+// plan_e picks E so that every length up to 1024 takes two stages, i.e. one exchange: an
+// exchange costs 16 bytes of shared-memory traffic an element and a barrier, and the passes
+// are bound by that pipe and by issue, not by registers.  The threads of a row then fit in one
+// warp (Q <= 32) and its exchange needs only __syncwarp.  With eight elements a thread (three
+// stages at 512, CTA barriers) the passes of a 512^3 force evaluation took 432 (forward z + y),
+// 457 (x) and 1317 us (inverse y + z with the gradients); they take 324, 340 and 976 us, the
+// first and the last at the copy bandwidth over the bytes they move (2.15 and 6.46 GB).
+//
+// Twiddles come from a per-stage table (tw_stage_offset; values from the host FP64 table
+// exp(-2 pi i k / 1024), rounded once), in shared or global memory; INV conjugates them
+// (unnormalised inverse).
 #pragma once
 
 #include "pm_common.cuh"
@@ -67,31 +73,110 @@ __device__ __forceinline__ void dft8(C* v) {
     v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
 }
 
+// cos(2 pi j / 32), j = 0..16
+__host__ __device__ constexpr double cos32(int j) {
+    return j > 8 ? -cos32(16 - j)
+                 : (j == 0   ? 1.0
+                    : j == 1 ? 0.98078528040323044913
+                    : j == 2 ? 0.92387953251128675613
+                    : j == 3 ? 0.83146961230254523708
+                    : j == 4 ? 0.70710678118654752440
+                    : j == 5 ? 0.55557023301960222474
+                    : j == 6 ? 0.38268343236508977173
+                    : j == 7 ? 0.19509032201612826785
+                             : 0.0);
+}
+
+// a exp(-+2 pi i J / 32), J = 0..31
+template <int J, bool INV, typename C>
+__device__ __forceinline__ C mul_w32(C a) {
+    typedef decltype(a.x) T;
+    if constexpr (J >= 16) {
+        const C b = mul_w32<J - 16, INV>(a);
+        return cmake<C>(-b.x, -b.y);
+    } else if constexpr (J == 0) {
+        return a;
+    } else if constexpr (J == 4) {
+        return mul_w8_1<INV>(a);
+    } else if constexpr (J == 8) {
+        return cmul_mi<INV>(a);
+    } else if constexpr (J == 12) {
+        return mul_w8_3<INV>(a);
+    } else {
+        constexpr T c = T(cos32(J)), s = T(J <= 8 ? cos32(8 - J) : cos32(J - 8));
+        return INV ? cmake<C>(a.x * c - a.y * s, a.y * c + a.x * s) : cmake<C>(a.x * c + a.y * s, a.y * c - a.x * s);
+    }
+}
+
+// A DFT of size 4 R2 as 4 x R2: DFT4 over the stride-R2 elements, the twiddles
+// exp(-+2 pi i n2 k1 / (4 R2)), then DFT_R2 over n2 for each k1; X_{k1 + 4 k2}.
+template <int R2, int N2, int K1, bool INV, typename C>
+__device__ __forceinline__ void dft4xr_twiddle(C* v) {
+    if constexpr (K1 < 4) {
+        v[N2 + R2 * K1] = mul_w32<(N2 * K1 * (8 / R2)) % 32, INV>(v[N2 + R2 * K1]);
+        dft4xr_twiddle<R2, N2, K1 + 1, INV>(v);
+    } else if constexpr (N2 + 1 < R2) {
+        dft4xr_twiddle<R2, N2 + 1, 1, INV>(v);
+    }
+}
+
+template <int R2, bool INV, typename C>
+__device__ __forceinline__ void dft4xr(C* v) {
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) dft4<INV>(v[n2], v[n2 + R2], v[n2 + 2 * R2], v[n2 + 3 * R2]);
+    dft4xr_twiddle<R2, 1, 1, INV>(v);
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) {
+        if constexpr (R2 == 8) dft8<INV>(v + R2 * k1);
+        else dft4<INV>(v[R2 * k1], v[R2 * k1 + 1], v[R2 * k1 + 2], v[R2 * k1 + 3]);
+    }
+    C w[4 * R2];
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1)
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) w[k1 + 4 * k2] = v[R2 * k1 + k2];
+#pragma unroll
+    for (int k = 0; k < 4 * R2; ++k) v[k] = w[k];
+}
+
 template <int R, bool INV, typename C>
 __device__ __forceinline__ void dftR(C* v) {
-    if constexpr (R == 8) dft8<INV>(v);
+    if constexpr (R == 32) dft4xr<8, INV>(v);
+    else if constexpr (R == 16) dft4xr<4, INV>(v);
+    else if constexpr (R == 8) dft8<INV>(v);
     else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
     else if constexpr (R == 2) dft2<INV>(v[0], v[1]);
 }
 
-template <bool INV, typename C>
-__device__ __forceinline__ C twid(const C* tw, int e) {
-    C w = tw[e];
-    if (INV) w.y = -w.y;
-    return w;
-}
+// Elements a thread of the row and column passes.
+__host__ __device__ constexpr int plan_e(int L) { return L >= 512 ? 32 : L >= 128 ? 16 : L == 16 ? 4 : 8; }
 
-__host__ __device__ constexpr int radix_at(int L, int Ns) { return (L / Ns) >= 8 ? 8 : (L / Ns); }
-__host__ __device__ constexpr int last_radix(int L, int Ns = 1) { return (Ns * radix_at(L, Ns) >= L) ? radix_at(L, Ns) : last_radix(L, Ns * radix_at(L, Ns)); }
+__host__ __device__ constexpr int radix_at(int L, int Ns, int E) { return (L / Ns) >= E ? E : (L / Ns); }
+__host__ __device__ constexpr int last_radix(int L, int E, int Ns = 1) {
+    return (Ns * radix_at(L, Ns, E) >= L) ? radix_at(L, Ns, E) : last_radix(L, E, Ns * radix_at(L, Ns, E));
+}
 
 // Per-stage twiddle table: the stage with span Ns > 1 and radix R keeps
 // w(r, jm) = exp(-2 pi i jm r / (Ns R)) at [offset(Ns) + (r - 1) Ns + jm], r = 1..R-1,
 // jm = 0..Ns-1, so the lanes of a warp (consecutive jm) read consecutive entries.  The
-// table of a length-L transform holds L - radix_at(L, 1) < L entries.
-__host__ __device__ constexpr int tw_stage_offset(int L, int Ns, int s = 1, int off = 0) {
-    return (s >= Ns) ? off : tw_stage_offset(L, Ns, s * radix_at(L, s), off + (s > 1 ? (radix_at(L, s) - 1) * s : 0));
+// table of a length-L transform holds L - radix_at(L, 1, E) < L entries.
+__host__ __device__ constexpr int tw_stage_offset(int L, int E, int Ns, int s = 1, int off = 0) {
+    return (s >= Ns) ? off
+                     : tw_stage_offset(L, E, Ns, s * radix_at(L, s, E), off + (s > 1 ? (radix_at(L, s, E) - 1) * s : 0));
 }
-__host__ __device__ constexpr int tw_stage_entries(int L) { return tw_stage_offset(L, L); }
+__host__ __device__ constexpr int tw_stage_entries(int L, int E) { return tw_stage_offset(L, E, L); }
+
+// Reads of the table: from shared memory, or (the plan_e transforms) from the global one.
+template <typename C>
+struct TwShared {
+    const C* p;
+    __device__ __forceinline__ C operator[](int e) const { return p[e]; }
+};
+template <typename C>
+struct TwGlobal {
+    const C* p;
+    __device__ __forceinline__ C operator[](int e) const { return __ldg(p + e); }
+};
 
 // ---------------------------------------------------------------- exchangers
 // Shared-memory rows of the exchanges: element i of a row sits at slot
@@ -114,6 +199,7 @@ struct RowLayout {
 // buffers alternate (p) when PP, so one barrier per exchange suffices.
 template <typename C, int NSEQ, bool PP, class LAY>
 struct RowEx {
+    static constexpr bool kTwoStage = false;
     C* base;
     int RB, RS, b, p;
     __device__ __forceinline__ C& at(int s, int i) {
@@ -122,6 +208,7 @@ struct RowEx {
     __device__ __forceinline__ void begin() {
         if (!PP) __syncthreads();
     }
+    __device__ __forceinline__ void sync() { __syncthreads(); }
     __device__ __forceinline__ void end() {
         if (PP) p ^= 1;
     }
@@ -131,78 +218,139 @@ struct RowEx {
 // interleaved so that lanes of consecutive columns hit consecutive banks).
 template <typename C, int L>
 struct ColEx {
+    static constexpr bool kTwoStage = false;
     C* base;
     int CS, b;
     __device__ __forceinline__ C& at(int s, int i) { return base[(s * L + i) * CS + b]; }
     __device__ __forceinline__ void begin() { __syncthreads(); }
+    __device__ __forceinline__ void sync() { __syncthreads(); }
+    __device__ __forceinline__ void end() {}
+};
+
+// The plan_e transforms: element i of a sequence at slot i + i / E.  A writing thread holds E
+// consecutive elements and a reading one elements Q apart, so with one spare slot every E both
+// sides' lanes fall in distinct banks (E + 1 is odd).
+//
+// A row of Q <= 32 threads of one warp: only the warp synchronises.  Rows are row_stride slots
+// apart (1 modulo 16), and row_of spaces the rows of a half-warp Q apart, so that rows sharing a
+// half-warp use disjoint banks and a column of the rows can be walked without conflicts.
+__host__ __device__ constexpr int row_stride(int L) { return (L + L / plan_e(L) + 14) / 16 * 16 + 1; }
+template <int Q>
+__device__ __forceinline__ int row_of(int tid) {
+    if constexpr (Q == 32) return tid >> 5;
+    const int g = (tid & 31) / Q;                 // group of Q lanes in the warp
+    const int hg = g / (16 / (Q < 16 ? Q : 16));  // its half-warp
+    const int gi = g % (16 / (Q < 16 ? Q : 16));
+    const int idx = 2 * (tid >> 5) + hg;
+    return (idx / Q) * 16 + gi * Q + idx % Q;
+}
+template <typename C, int E>
+struct WarpRowEx {
+    static constexpr bool kTwoStage = true;
+    C* row;
+    // the two sides of the exchange: result r of thread t (element t E + r), and element
+    // j + r E of the reading butterfly j < E
+    __device__ __forceinline__ C& put(int t, int r) { return row[t * (E + 1) + r]; }
+    __device__ __forceinline__ C& get(int j, int r) { return row[j + r * (E + 1)]; }
+    __device__ __forceinline__ void begin() { __syncwarp(); }
+    __device__ __forceinline__ void sync() { __syncwarp(); }
+    __device__ __forceinline__ void end() {}
+};
+
+// Columns of a CTA, interleaved: slot s of column b at s CB + b.
+template <typename C, int E, int CB>
+struct CtaColEx {
+    static constexpr bool kTwoStage = true;
+    C* col;  // the CTA's buffer + column b
+    __device__ __forceinline__ C& put(int t, int r) { return col[(t * (E + 1) + r) * CB]; }
+    __device__ __forceinline__ C& get(int j, int r) { return col[(j + r * (E + 1)) * CB]; }
+    __device__ __forceinline__ void begin() { __syncthreads(); }
+    __device__ __forceinline__ void sync() { __syncthreads(); }
     __device__ __forceinline__ void end() {}
 };
 
 // ---------------------------------------------------------------- stages
-template <int L, int Ns, int NSEQ, bool INV, typename C, class X>
-__device__ __forceinline__ void fft_stages(C (*v)[8], int t, const C* __restrict__ tw, X& ex) {
-    constexpr int R = radix_at(L, Ns);
-    constexpr int NB = 8 / R;
-    constexpr int Q = L / 8;
+template <int L, int E, int Ns, int NSEQ, bool INV, typename C, class TW, class X>
+__device__ __forceinline__ void fft_stages(C (*v)[E], int t, const TW& tw, X& ex) {
+    constexpr int R = radix_at(L, Ns, E);
+    constexpr int NB = E / R;
+    constexpr int Q = L / E;
 #pragma unroll
     for (int s = 0; s < NSEQ; ++s)
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
             if constexpr (Ns > 1) {
-                const int jm = (t + q * Q) & (Ns - 1);
-                const C* tws = tw + tw_stage_offset(L, Ns) + jm;
+                const int e0 = tw_stage_offset(L, E, Ns) + ((t + q * Q) & (Ns - 1));
 #pragma unroll
-                for (int r = 1; r < R; ++r) v[s][q * R + r] = cmul(v[s][q * R + r], twid<INV>(tws, (r - 1) * Ns));
+                for (int r = 1; r < R; ++r) {
+                    const C w = tw[e0 + (r - 1) * Ns];
+                    v[s][q * R + r] = INV ? cmulc(v[s][q * R + r], w) : cmul(v[s][q * R + r], w);
+                }
             }
             dftR<R, INV>(&v[s][q * R]);
         }
     if constexpr (Ns * R < L) {
         constexpr int Ns2 = Ns * R;
-        constexpr int R2 = radix_at(L, Ns2);
-        constexpr int NB2 = 8 / R2;
+        constexpr int R2 = radix_at(L, Ns2, E);
+        constexpr int NB2 = E / R2;
         ex.begin();
+        if constexpr (X::kTwoStage) {
+            // two stages, one sequence at a time
+            static_assert(NSEQ == 1 && Ns == 1 && R == E && R2 == Q, "a plan_e transform takes two stages");
 #pragma unroll
-        for (int s = 0; s < NSEQ; ++s)
+            for (int r = 0; r < R; ++r) ex.put(t, r) = v[0][r];
+            ex.sync();
 #pragma unroll
-            for (int q = 0; q < NB; ++q) {
-                const int j = t + q * Q;
-                const int base = (j / Ns) * Ns2 + (j & (Ns - 1));
+            for (int q = 0; q < NB2; ++q)
 #pragma unroll
-                for (int r = 0; r < R; ++r) ex.at(s, base + r * Ns) = v[s][q * R + r];
-            }
-        __syncthreads();
+                for (int r = 0; r < R2; ++r) v[0][q * R2 + r] = ex.get(t + q * Q, r);
+            ex.end();
+            fft_stages<L, E, Ns2, NSEQ, INV>(v, t, tw, ex);
+            return;
+        } else {
 #pragma unroll
-        for (int s = 0; s < NSEQ; ++s)
+            for (int s = 0; s < NSEQ; ++s)
 #pragma unroll
-            for (int q = 0; q < NB2; ++q) {
-                const int j = t + q * Q;
+                for (int q = 0; q < NB; ++q) {
+                    const int j = t + q * Q;
+                    const int base = (j / Ns) * Ns2 + (j & (Ns - 1));
 #pragma unroll
-                for (int r = 0; r < R2; ++r) v[s][q * R2 + r] = ex.at(s, j + r * (L / R2));
-            }
-        ex.end();
-        fft_stages<L, Ns2, NSEQ, INV>(v, t, tw, ex);
+                    for (int r = 0; r < R; ++r) ex.at(s, base + r * Ns) = v[s][q * R + r];
+                }
+            ex.sync();
+#pragma unroll
+            for (int s = 0; s < NSEQ; ++s)
+#pragma unroll
+                for (int q = 0; q < NB2; ++q) {
+                    const int j = t + q * Q;
+#pragma unroll
+                    for (int r = 0; r < R2; ++r) v[s][q * R2 + r] = ex.at(s, j + r * (L / R2));
+                }
+            ex.end();
+            fft_stages<L, E, Ns2, NSEQ, INV>(v, t, tw, ex);
+        }
     }
 }
 
-// Transform NSEQ sequences of length L (8 <= L <= 1024, a power of two).  On entry
-// v[s][m] is element t + m L/8 of sequence s; on exit v[s][m] is transform element
-// t + m L/8.  Contains barriers: every thread of the CTA must call it.
-template <int L, int NSEQ, bool INV, typename C, class X>
-__device__ __forceinline__ void fft_regs(C (*v)[8], int t, const C* __restrict__ tw, X& ex) {
-    fft_stages<L, 1, NSEQ, INV>(v, t, tw, ex);
-    constexpr int RL = last_radix(L);
-    if constexpr (RL < 8) {
-        // after a closing radix-RL stage, slot q RL + r holds element t + (q + r 8/RL) L/8
-        constexpr int NB = 8 / RL;
+// Transform NSEQ sequences of length L (8 <= L <= 1024, a power of two), E elements a thread.
+// On entry v[s][m] is element t + m L/E of sequence s; on exit v[s][m] is transform element
+// t + m L/E.  Contains the exchanger's barriers: every thread of the CTA (or warp) must call it.
+template <int L, int NSEQ, bool INV, int E, typename C, class TW, class X>
+__device__ __forceinline__ void fft_regs(C (*v)[E], int t, const TW& tw, X& ex) {
+    fft_stages<L, E, 1, NSEQ, INV>(v, t, tw, ex);
+    constexpr int RL = last_radix(L, E);
+    if constexpr (RL < E) {
+        // after a closing radix-RL stage, slot q RL + r holds element t + (q + r E/RL) L/E
+        constexpr int NB = E / RL;
 #pragma unroll
         for (int s = 0; s < NSEQ; ++s) {
-            C w[8];
+            C w[E];
 #pragma unroll
             for (int q = 0; q < NB; ++q)
 #pragma unroll
                 for (int r = 0; r < RL; ++r) w[q + r * NB] = v[s][q * RL + r];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) v[s][m] = w[m];
+            for (int m = 0; m < E; ++m) v[s][m] = w[m];
         }
     }
 }

@@ -6,8 +6,14 @@ namespace pm {
 static __device__ float2 g_tw32[1024];
 template <> __device__ __forceinline__ float2 tw_global<float>(int k) { return g_tw32[k]; }
 
-cudaError_t upload_twiddles_f32(const float2* host) {
-    return cudaMemcpyToSymbol(g_tw32, host, sizeof(float2) * 1024);
+// per-stage tables of the plan_e transforms: length L at [L, 2 L)
+static __device__ __align__(256) float2 g_stages32[2048];
+template <> __device__ __forceinline__ const float2* tw_stages<float>() { return g_stages32; }
+
+cudaError_t upload_twiddles_f32(const float2* host, const float2* stages) {
+    cudaError_t e = cudaMemcpyToSymbol(g_tw32, host, sizeof(float2) * 1024);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyToSymbol(g_stages32, stages, sizeof(float2) * 2048);
 }
 
 PM_INST(float)

@@ -6,8 +6,14 @@ namespace pm {
 static __device__ double2 g_tw64[1024];
 template <> __device__ __forceinline__ double2 tw_global<double>(int k) { return g_tw64[k]; }
 
-cudaError_t upload_twiddles_f64(const double2* host) {
-    return cudaMemcpyToSymbol(g_tw64, host, sizeof(double2) * 1024);
+// per-stage tables of the plan_e transforms: length L at [L, 2 L)
+static __device__ __align__(256) double2 g_stages64[2048];
+template <> __device__ __forceinline__ const double2* tw_stages<double>() { return g_stages64; }
+
+cudaError_t upload_twiddles_f64(const double2* host, const double2* stages) {
+    cudaError_t e = cudaMemcpyToSymbol(g_tw64, host, sizeof(double2) * 1024);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyToSymbol(g_stages64, stages, sizeof(double2) * 2048);
 }
 
 PM_INST(double)

@@ -24,31 +24,31 @@
 namespace pm {
 
 template <typename T> __device__ __forceinline__ cplx<T> tw_global(int k);
+// The per-stage table (fft.cuh) of the length-L plan_e transform in global memory: a few KB
+// read by every CTA, so it stays in L1 and the passes need no set-up of their own.
+template <typename T> __device__ __forceinline__ const cplx<T>* tw_stages();
+template <typename T, int L>
+__device__ __forceinline__ TwGlobal<cplx<T>> tw_plan() {
+    return TwGlobal<cplx<T>>{tw_stages<T>() + L};
+}
 cudaError_t set_smem_once(const void* fn, size_t bytes);
 
-// The per-stage twiddle table of a length-L transform (layout: fft.cuh, tw_stage_offset).
+// The per-stage twiddle table of a length-L transform of eight elements a thread, into shared
+// memory (the persistent and whole-plane middle passes).
 template <typename T, int L>
 __device__ __forceinline__ void load_stage_twiddles(cplx<T>* tw) {
-    constexpr int TE = tw_stage_entries(L);
+    constexpr int TE = tw_stage_entries(L, 8);
     for (int k = threadIdx.x; k < TE; k += blockDim.x) {
-        int Ns = radix_at(L, 1), off = 0;  // stages with span Ns > 1, in order
-        while (k >= off + (radix_at(L, Ns) - 1) * Ns) {
-            off += (radix_at(L, Ns) - 1) * Ns;
-            Ns *= radix_at(L, Ns);
+        int Ns = radix_at(L, 1, 8), off = 0;  // stages with span Ns > 1, in order
+        while (k >= off + (radix_at(L, Ns, 8) - 1) * Ns) {
+            off += (radix_at(L, Ns, 8) - 1) * Ns;
+            Ns *= radix_at(L, Ns, 8);
         }
-        const int R = radix_at(L, Ns);
+        const int R = radix_at(L, Ns, 8);
         const int r = (k - off) / Ns + 1, jm = (k - off) % Ns;
         tw[k] = tw_global<T>(jm * r * (1024 / (Ns * R)));
     }
 }
-
-// First `count` entries of the length-L table.
-template <typename T>
-__device__ __forceinline__ void load_twiddles_head(cplx<T>* tw, int L, int count) {
-    const int stride = 1024 / L;
-    for (int k = threadIdx.x; k < count; k += blockDim.x) tw[k] = tw_global<T>(k * stride);
-}
-
 
 // a / d in the per-mode operators.  FP32 divides as written.  FP64 divides are slow on this
 // part, so FP64 computes the reciprocal of d by the Newton-Raphson iteration for 1/d,
@@ -71,19 +71,34 @@ static inline cudaError_t set_smem(const void* fn, size_t bytes) {
     return set_smem_once(fn, bytes);
 }
 
-// Launch shapes (compile time): sequences per CTA for each pass.
-template <typename T, int LOGN> struct Shape {
-    static constexpr int N = 1 << LOGN;
-    static constexpr int M = N / 2;
-    static constexpr int QN = N / 8;            // threads per length-N sequence
-    static constexpr int QM = (M >= 8) ? M / 8 : 1;
-    static constexpr int YB = (512 / QM < N) ? 512 / QM : N;     // z passes: rows per CTA
-    static constexpr int RB = (256 / QN > 0) ? 256 / QN : 1;     // y pass
-    static constexpr int RB3 = (sizeof(T) == 8) ? ((128 / QN > 0) ? 128 / QN : 1) : RB;  // y grad3
-    static constexpr int CB0 = (512 / QN < N) ? 512 / QN : N;
-    // x pass columns (FP64 halves them from n = 64 so that the exchange buffers and the
-    // prefetch stage stay within 227 KB of shared memory)
-    static constexpr int CB = (sizeof(T) == 8 && N >= 64) ? CB0 / 2 : CB0;
+// Launch shapes (compile time).
+// z passes: YB rows of one x slab a CTA, so that the transposed side moves segments of YB
+// complex values: 128 bytes at least in FP32.
+template <typename T, int LOGN> struct ZShape {
+    static constexpr int N = 1 << LOGN, M = N / 2, E = plan_e(M), Q = M / E, RS = row_stride(M);
+    static constexpr int YB = (N == 32 || N == 128 || N == 256) ? 32 : 16;
+    static constexpr int THREADS = YB * Q;
+    // the registers of E complex values and their temporaries decide the residency
+    static constexpr int MINB = (E == 32 ? 512 : 1024) / (sizeof(T) == 8 ? 2 : 1) / (THREADS < 64 ? 64 : THREADS);
+    static constexpr size_t SMEM = sizeof(cplx<T>) * (size_t)YB * RS;
+};
+// y passes: RB rows a CTA.
+template <typename T, int LOGN> struct YShape {
+    static constexpr int N = 1 << LOGN, E = plan_e(N), Q = N / E, RS = row_stride(N);
+    static constexpr int THREADS = 128, RB = THREADS / Q;
+    static constexpr int MINB = (E == 32 ? 512 : 1024) / (sizeof(T) == 8 ? 2 : 1) / THREADS;
+    static constexpr int MINB3 = (E == 32 ? 512 : E == 16 ? 768 : 1024) / (sizeof(T) == 8 ? 2 : 1) / THREADS;  // y grad3
+    static constexpr size_t SMEM = sizeof(cplx<T>) * (size_t)RB * RS;
+};
+// x passes: CB columns of one plane a CTA, CTAs of 64 to 256 threads with several an SM.  Eight
+// columns (64-byte row segments) beat sixteen where a thread holds 16 or 32 values: 340 against
+// 457 us for the Newtonian pass at 512^3 and 43 against 48 us at 256^3, since the wider CTA
+// halves the CTAs an SM that overlap one another's loads; below that sixteen are better.
+template <typename T, int LOGN> struct XShape {
+    static constexpr int N = 1 << LOGN, E = plan_e(N), Q = N / E;
+    static constexpr int CB = (sizeof(T) == 8) ? (E == 32 ? 4 : 8) : (E >= 16 ? 8 : 16);
+    static constexpr int THREADS = CB * Q;
+    static constexpr size_t COL = (size_t)(N + N / E) * CB;  // exchange slots
 };
 
 // Row of (slab row gl = field n + x, frequency kz) in the half spectra [field][kz][x][ky].
@@ -98,53 +113,47 @@ __device__ __forceinline__ size_t spec_row(int gl, int kz) {
 // with the fluctuations rather than with the mean.  With sub = 1, v - 1 is exact for v in
 // [0.5, 2^24] and below 0.5 within half the spacing of the values near 1 (2^-25 in FP32).
 template <typename T, int LOGN>
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 2) k_z_r2c(const T* __restrict__ in, cplx<T>* __restrict__ out,
-                                                                       T sub) {
+__global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MINB)
+    k_z_r2c(const T* __restrict__ in, cplx<T>* __restrict__ out, T sub) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, M = S::M, Q = S::QM, YB = S::YB;
-    typedef RowLayout<M, true> LAY;
-    constexpr int RS = LAY::RS;
-    constexpr int TWN = (M + 2) & ~1;
+    typedef ZShape<T, LOGN> S;
+    constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* twM = reinterpret_cast<C*>(smem_raw);
-    C* twN = twM + M;
-    C* buf = twN + TWN;
+    C* buf = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x;
     const int y0 = blockIdx.x * YB;
     const int gl = blockIdx.y;
-    const size_t g = gl;
-    load_stage_twiddles<T, M>(twM);
-    load_twiddles_head<T>(twN, N, M + 1);
-    const int b = tid / Q, t = tid % Q;
-    const C* row = reinterpret_cast<const C*>(in + (g * N + y0 + b) * N);
-    C v[1][8];
+    const int b = row_of<Q>(tid), t = tid % Q;
+    const C* row = reinterpret_cast<const C*>(in + ((size_t)gl * N + y0 + b) * N);
+    C v[1][E];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        v[0][m] = row[t + m * Q];
+    for (int m = 0; m < E; ++m) v[0][m] = row[t + m * Q];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
         v[0][m].x -= sub;
         v[0][m].y -= sub;
     }
-    __syncthreads();
-    RowEx<C, 1, false, LAY> ex{buf, YB, RS, b, 0};
-    fft_regs<M, 1, false>(v, t, twM, ex);
-    C* z = buf;
-    __syncthreads();  // every thread has read its last exchange before the buffer is reused
+    C* z = buf + b * RS;
+    WarpRowEx<C, E> ex{z};
+    fft_regs<M, 1, false>(v, t, tw_plan<T, M>(), ex);
+    ex.begin();  // the row's exchange has been read
 #pragma unroll
-    for (int m = 0; m < 8; ++m) z[b * RS + LAY::slot(t + m * Q)] = v[0][m];
+    for (int m = 0; m < E; ++m) z[t + m * Q] = v[0][m];
     __syncthreads();
-    constexpr int NT = YB * Q, ITERS = ((M + 1) * YB + NT - 1) / NT;
+    // the real transform from the packed one, the pair (k, M - k) at a time:
+    //   X_k = P + w^k O, X_{M-k} = conj(P - w^k O), P, O = (z_k +- z*_{M-k}) / 2 [* -i]
+    const int bb = tid % YB, k0 = tid / YB;
+    constexpr int TWS = 1024 / N;  // exp(-2 pi i k / N) = global table entry k TWS
+    auto pair = [&](int k) {
+        const C z1 = buf[bb * RS + k], z2 = cconj(buf[bb * RS + ((M - k) & (M - 1))]);
+        const C P = cscale(cadd(z1, z2), T(0.5));
+        const C O = cmul(cscale(cmul_mi<false>(csub(z1, z2)), T(0.5)), tw_global<T>(k * TWS));
+        out[spec_row<M, LOGN>(gl, k) * N + y0 + bb] = cadd(P, O);
+        if (2 * k != M) out[spec_row<M, LOGN>(gl, M - k) * N + y0 + bb] = cconj(csub(P, O));
+    };
 #pragma unroll
-    for (int it = 0; it < ITERS; ++it) {
-        const int e = tid + it * NT;
-        if (e >= (M + 1) * YB) break;
-        const int k = e / YB, bb = e % YB;
-        const C z1 = z[bb * RS + LAY::slot(k == M ? 0 : k)];
-        const C z2 = cconj(z[bb * RS + LAY::slot(k == 0 ? 0 : M - k)]);
-        const C E = cscale(cadd(z1, z2), T(0.5));
-        const C O = cscale(cmul_mi<false>(csub(z1, z2)), T(0.5));
-        out[spec_row<M, LOGN>(gl, k) * N + y0 + bb] = cadd(E, cmul(twN[k], O));
-    }
+    for (int it = 0; it < E / 2; ++it) pair(k0 + it * Q);
+    if (k0 == 0) pair(M / 2);
 }
 
 // =============================================================== z: c2r
@@ -155,199 +164,240 @@ template <typename T> struct Ptr3 {
 };
 
 template <typename T, int LOGN>
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 4 : 2) k_z_c2r(Ptr3<T> P, unsigned gradz_mask, T kf0,
-                                                                       const double* __restrict__ kf_arr) {
+__global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MINB)
+    k_z_c2r(Ptr3<T> P, unsigned gradz_mask, T kf0, const double* __restrict__ kf_arr) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, M = S::M, Q = S::QM, YB = S::YB;
-    typedef RowLayout<M, true> LAY;
-    constexpr int RS = LAY::RS;
+    typedef ZShape<T, LOGN> S;
+    constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* twM = reinterpret_cast<C*>(smem_raw);
-    C* buf = twM + M;
+    C* buf = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x;
     const int comp = blockIdx.z;
     const bool grad = (gradz_mask >> comp) & 1u;
     const int y0 = blockIdx.x * YB;
     const int gl = blockIdx.y;
-    const size_t g = gl;
-    load_stage_twiddles<T, M>(twM);
     const T kf = kf_arr ? T(kf_arr[gl >> LOGN]) : kf0;
     const C* inp = comp == 0 ? P.in[0] : (comp == 1 ? P.in[1] : P.in[2]);
     T* pout = comp == 0 ? P.out[0] : (comp == 1 ? P.out[1] : P.out[2]);
-    C* xb = buf;  // the pre-processed half spectrum; the FFT exchanges reuse the buffer afterwards
-    // Each thread loads the pairs (X_k, X_{M-k}), k = 0..M/2, of its columns -- all of its
-    // strided row segments in flight together -- and forms in registers
-    //   Y_k = (X_k + X*_{M-k}) + i (X_k - X*_{M-k}) exp(+2 pi i k / N)   (and Y_{M-k} likewise),
+    // Each thread loads the pairs (X_k, X_{M-k}) of its column -- all of its strided row
+    // segments in flight together -- and forms in registers
+    //   Y_k = s + i d, Y_{M-k} = conj(s) + i conj(d), s = X_k + X*_{M-k},
+    //   d = (X_k - X*_{M-k}) exp(+2 pi i k / N),
     // the M-point sequence whose inverse transform interleaves the real output.
-    constexpr int NT = YB * Q, NP = (M / 2 + 1) * YB, ITERS = (NP + NT - 1) / NT;
-    C X1[ITERS], X2[ITERS];
+    const int bb = tid % YB, k0 = tid / YB;
+    const C* col = inp + spec_row<M, LOGN>(gl, 0) * N + y0 + bb;
+    constexpr size_t KZ = (size_t)N * N;  // elements from one kz to the next
+    C X1[E / 2], X2[E / 2], Xm;
 #pragma unroll
-    for (int it = 0; it < ITERS; ++it) {
-        const int e = tid + it * NT;
-        if (e < NP) {
-            const int k = e / YB, col = y0 + e % YB;
-            X1[it] = inp[spec_row<M, LOGN>(gl, k) * N + col];
-            X2[it] = inp[spec_row<M, LOGN>(gl, M - k) * N + col];
-        }
+    for (int it = 0; it < E / 2; ++it) {
+        X1[it] = col[(k0 + it * Q) * KZ];
+        X2[it] = col[(M - k0 - it * Q) * KZ];
     }
+    if (k0 == 0) Xm = col[(M / 2) * KZ];
     constexpr int TWS = 1024 / N;  // exp(-2 pi i k / N) = global table entry k TWS
-#pragma unroll
-    for (int it = 0; it < ITERS; ++it) {
-        const int e = tid + it * NT;
-        if (e < NP) {
-            const int k = e / YB, bb = e % YB;
-            C a = X1[it], c = X2[it];
-            if (grad) {  // (-i kz) X, Nyquist kz -> 0
-                const T kza = kf * T(k), kzc = (k == 0) ? T(0) : kf * T(M - k);
-                a = cmake<C>(a.y * kza, -a.x * kza);
-                c = cmake<C>(c.y * kzc, -c.x * kzc);
-            }
-            if (k == 0) {
-                a.y = T(0);
-                c.y = T(0);
-            }
-            C* r = xb + bb * RS;
-            const C bconj = cconj(c);
-            const C d = cmul(csub(a, bconj), cconj(tw_global<T>(k * TWS)));
-            r[LAY::slot(k)] = cadd(cadd(a, bconj), cmake<C>(-d.y, d.x));
-            if (k > 0 && k < M - k) {
-                const C aconj = cconj(a);
-                const C d2 = cmul(csub(c, aconj), cconj(tw_global<T>((M - k) * TWS)));
-                r[LAY::slot(M - k)] = cadd(cadd(c, aconj), cmake<C>(-d2.y, d2.x));
-            }
+    C* r = buf + bb * RS;          // the FFT exchanges reuse the rows afterwards
+    auto pair = [&](int k, C a, C c) {
+        if (grad) {  // (-i kz) X, Nyquist kz -> 0
+            const T kza = kf * T(k), kzc = (k == 0) ? T(0) : kf * T(M - k);
+            a = cmake<C>(a.y * kza, -a.x * kza);
+            c = cmake<C>(c.y * kzc, -c.x * kzc);
         }
-    }
+        if (k == 0) {
+            a.y = T(0);
+            c.y = T(0);
+        }
+        const C s = cadd(a, cconj(c));
+        const C d = cmulc(csub(a, cconj(c)), tw_global<T>(k * TWS));
+        r[k] = cmake<C>(s.x - d.y, s.y + d.x);
+        if (k > 0 && 2 * k != M) r[M - k] = cmake<C>(s.x + d.y, d.x - s.y);
+    };
+#pragma unroll
+    for (int it = 0; it < E / 2; ++it) pair(k0 + it * Q, X1[it], X2[it]);
+    if (k0 == 0) pair(M / 2, Xm, Xm);
     __syncthreads();
-    const int b = tid / Q, t = tid % Q;
-    C v[1][8];
+    const int b = row_of<Q>(tid), t = tid % Q;
+    C* z = buf + b * RS;
+    C v[1][E];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) v[0][m] = xb[b * RS + LAY::slot(t + m * Q)];
-    RowEx<C, 1, false, LAY> ex{buf, YB, RS, b, 0};
-    fft_regs<M, 1, true>(v, t, twM, ex);
-    C* orow = reinterpret_cast<C*>(pout + (g * N + y0 + b) * N);
+    for (int m = 0; m < E; ++m) v[0][m] = z[t + m * Q];
+    WarpRowEx<C, E> ex{z};
+    fft_regs<M, 1, true>(v, t, tw_plan<T, M>(), ex);
+    C* orow = reinterpret_cast<C*>(pout + ((size_t)gl * N + y0 + b) * N);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) orow[t + m * Q] = v[0][m];
+    for (int m = 0; m < E; ++m) orow[t + m * Q] = v[0][m];
     if (P.zero && comp == 0) {  // the same rows of the mesh the caller clears for its next use
-        C* zrow = reinterpret_cast<C*>(P.zero + (g * N + y0 + b) * N);
+        C* zrow = reinterpret_cast<C*>(P.zero + ((size_t)gl * N + y0 + b) * N);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) zrow[t + m * Q] = cmake<C>(T(0), T(0));
+        for (int m = 0; m < E; ++m) zrow[t + m * Q] = cmake<C>(T(0), T(0));
     }
 }
 
 // =============================================================== y: contiguous rows
-// In place when in == out.
+// In place when in == out.  Each row is one warp's (or part of one), so no CTA barriers.
 template <typename T, int LOGN, bool INV>
-__global__ void __launch_bounds__(512) k_y_rows(const cplx<T>* in, cplx<T>* out, int64_t nrows) {
+__global__ void __launch_bounds__(YShape<T, LOGN>::THREADS, YShape<T, LOGN>::MINB)
+    k_y_rows(const cplx<T>* in, cplx<T>* out, int64_t nrows) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, Q = S::QN, RB = S::RB;
-    typedef RowLayout<N, false> LAY;
-    constexpr int RS = LAY::RS;
+    typedef YShape<T, LOGN> S;
+    constexpr int N = S::N, E = S::E, Q = S::Q;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
-    const int tid = threadIdx.x;
-    const int b = tid / Q, t = tid % Q;
-    const int64_t r = (int64_t)blockIdx.x * RB + b;
+    const int b = row_of<Q>(threadIdx.x), t = threadIdx.x % Q;
+    const int64_t r = (int64_t)blockIdx.x * S::RB + b;
     const bool ok = r < nrows;
-    load_stage_twiddles<T, N>(tw);
-    C v[1][8];
+    C v[1][E];
     const C* irow = in + r * N;
     if (ok) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) v[0][m] = irow[t + m * Q];
+        for (int m = 0; m < E; ++m) v[0][m] = irow[t + m * Q];
     }
-    __syncthreads();
-    RowEx<C, 1, true, LAY> ex{buf, RB, RS, b, 0};
-    fft_regs<N, 1, INV>(v, t, tw, ex);
+    WarpRowEx<C, E> ex{reinterpret_cast<C*>(smem_raw) + b * S::RS};
+    fft_regs<N, 1, INV>(v, t, tw_plan<T, N>(), ex);
     C* orow = out + r * N;
     if (ok) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) orow[t + m * Q] = v[0][m];
+        for (int m = 0; m < E; ++m) orow[t + m * Q] = v[0][m];
     }
 }
 
 // A' = IFFT_y(A), B' = IFFT_y(B), C' = IFFT_y(-i ky A) (in place when Aout == A, Bout == B).
+// The three transforms run one after the other in the same registers; A is read twice (the
+// second time from L2) rather than held beside its transform, which would halve the warps.
 template <typename T, int LOGN>
-__global__ void __launch_bounds__(512) k_y_grad3(const cplx<T>* A, const cplx<T>* B, cplx<T>* Aout, cplx<T>* Bout,
-                                                 cplx<T>* __restrict__ Cout, int64_t nrows, T kf0,
-                                                 const double* __restrict__ kf_arr, int64_t rows_per_field) {
+__global__ void __launch_bounds__(YShape<T, LOGN>::THREADS, YShape<T, LOGN>::MINB3)
+    k_y_grad3(const cplx<T>* A, const cplx<T>* B, cplx<T>* Aout, cplx<T>* Bout, cplx<T>* __restrict__ Cout,
+              int64_t nrows, T kf0, const double* __restrict__ kf_arr, int64_t rows_per_field) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, Q = S::QN, RB = S::RB3;
-    typedef RowLayout<N, false> LAY;
-    constexpr int RS = LAY::RS;
+    typedef YShape<T, LOGN> S;
+    constexpr int N = S::N, E = S::E, Q = S::Q;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
-    const int tid = threadIdx.x;
-    const int b = tid / Q, t = tid % Q;
-    const int64_t r = (int64_t)blockIdx.x * RB + b;
+    const int b = row_of<Q>(threadIdx.x), t = threadIdx.x % Q;
+    const int64_t r = (int64_t)blockIdx.x * S::RB + b;
     const bool ok = r < nrows;
-    const int64_t ri = r;
     const T kf = (kf_arr && ok) ? T(kf_arr[r / rows_per_field]) : kf0;
-    load_stage_twiddles<T, N>(tw);
-    // two rounds keep two sequences live at a time: (A, -i ky A), then B
-    C v[2][8];
+    WarpRowEx<C, E> ex{reinterpret_cast<C*>(smem_raw) + b * S::RS};
+    const int64_t o = r * N + t;
+    C v[1][E];
     if (ok) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int i = t + m * Q;
-            const C a = A[ri * N + i];
-            v[0][m] = a;
-            const int ny = (i < N / 2) ? i : i - N;
-            const T ky = (2 * ny == -N) ? T(0) : kf * T(ny);
-            v[1][m] = cmake<C>(a.y * ky, -a.x * ky);
-        }
+        for (int m = 0; m < E; ++m) v[0][m] = A[o + m * Q];
     }
-    __syncthreads();
-    RowEx<C, 2, false, LAY> ex{buf, RB, RS, b, 0};
-    fft_regs<N, 2, true>(v, t, tw, ex);
-    if (ok) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int i = t + m * Q;
-            Aout[r * N + i] = v[0][m];
-            Cout[r * N + i] = v[1][m];
-        }
-        // Bout may alias B, never A: the rows of A written above are not read again
-#pragma unroll
-        for (int m = 0; m < 8; ++m) v[0][m] = B[ri * N + t + m * Q];
+    for (int m = 0; m < E; ++m) {
+        const int i = t + m * Q;
+        const T ky = (2 * m == E && t == 0) ? T(0) : kf * T(2 * m < E ? i : i - N);
+        v[0][m] = cmake<C>(v[0][m].y * ky, -v[0][m].x * ky);
     }
-    RowEx<C, 1, false, LAY> ex1{buf, RB, RS, b, 0};
-    fft_regs<N, 1, true>(v, t, tw, ex1);
+    fft_regs<N, 1, true>(v, t, tw_plan<T, N>(), ex);
     if (ok) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) Bout[r * N + t + m * Q] = v[0][m];
+        for (int m = 0; m < E; ++m) Cout[o + m * Q] = v[0][m];
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[0][m] = A[o + m * Q];
+    }
+    fft_regs<N, 1, true>(v, t, tw_plan<T, N>(), ex);
+    if (ok) {
+        // a thread's own elements of A, which no other thread reads
+#pragma unroll
+        for (int m = 0; m < E; ++m) Aout[o + m * Q] = v[0][m];
+        // Bout may alias B, never A
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[0][m] = B[o + m * Q];
+    }
+    fft_regs<N, 1, true>(v, t, tw_plan<T, N>(), ex);
+    if (ok) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) Bout[o + m * Q] = v[0][m];
     }
 }
 
 // =============================================================== x: strided columns + spectral operators
-// 16-byte asynchronous copy global -> shared (cp.async, completion by wait_group).
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // A hint that brings the 128-byte line holding p into L2 (no register, no wait).
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Persistent: each CTA walks blocks blk = blockIdx.x, + gridDim.x, ... of CB columns of one
-// plane (plane = blk / (N / CB)).  The next block's columns are copied into a shared
-// stage with cp.async while the current block is transformed, so the loads of one block
-// overlap the butterflies and stores of the previous one.
-// Column groups of the x pass: FP32 meshes of 256 and more take 1024-thread CTAs of twice
-// the columns (full 128-byte row segments; the binning pass keeps 512 threads, its
-// cross-spectrum stage would not fit).
-template <typename T, int LOGN, int KIND> struct XShape {
-    typedef Shape<T, LOGN> S;
-    static constexpr bool WIDE = sizeof(T) == 4 && S::N >= 256 && KIND != OP_BIN;
-    static constexpr int CB = WIDE ? 1024 / S::QN : S::CB;
-    static constexpr int THREADS = CB * S::QN;
-    static constexpr int MINB = WIDE ? 1 : (sizeof(T) == 4 ? 2 : 1);
+// The linearised Poisson-gauge constraint on one mode in the working precision:
+// Phi = (num delta + cc Phi_old) / (k^2 + base), cc = 0 at the first force evaluation.
+template <typename T> struct GrOp {
+    T kf2, num, base, cc;
+    __device__ __forceinline__ GrOp(const SpecOp& op, T kf2T) {
+        const T H = T(op.calH), om = T(op.omm_a);
+        kf2 = kf2T;
+        num = T(-1.5) * H * H * om;
+        cc = op.first ? T(0) : T(3) * H * T(op.inv_dtau);
+        base = T(3) * H * H + T(4.5) * H * H * om + cc;
+    }
+    __device__ __forceinline__ cplx<T> solve(cplx<T> delta, cplx<T> old, int n2) const {
+        const T r = div_mode(T(1), kf2 * T(n2) + base);
+        return cmake<cplx<T>>((num * delta.x + cc * old.x) * r, (num * delta.y + cc * old.y) * r);
+    }
 };
+
+// The modes |n|^2 <= n_lo^2 of the constraint, solved and kept in FP64 in the island
+// ((n_lo + 1) (2 n_lo + 1)^2 modes a field); the zero mode is 0.
+template <typename T>
+__device__ __noinline__ cplx<T> gr_island_mode(const SpecOp& op, cplx<T> vv, int nx, int ny, int nz, int n2, int field,
+                                               double kf) {
+    const int L = op.n_lo, W2 = 2 * L + 1;
+    const size_t id = (((size_t)field * (L + 1) + nz) * W2 + (nx + L)) * W2 + (ny + L);
+    if (n2 == 0) {
+        if (L > 0) op.island[id] = make_double2(0.0, 0.0);
+        return cmake<cplx<T>>(T(0), T(0));
+    }
+    const double k2 = kf * kf * (double)n2;
+    const double H = op.calH;
+    const double num_s = -1.5 * H * H * op.omm_a;
+    double den = k2 + 3.0 * H * H + 4.5 * H * H * op.omm_a;
+    double2 P = make_double2(num_s * (double)vv.x, num_s * (double)vv.y);
+    if (!op.first) {
+        const double2 old = op.island[id];
+        const double cc = 3.0 * H * op.inv_dtau;
+        P.x += cc * old.x;
+        P.y += cc * old.y;
+        den += cc;
+    }
+    P.x /= den;
+    P.y /= den;
+    op.island[id] = P;
+    return cmake<cplx<T>>(T(P.x * op.ac2_over_n3), T(P.y * op.ac2_over_n3));
+}
+
+// The constraint on a thread's E modes kx = t + m Q of the x pass, in place (phi), Phi_old at
+// old[i N].  The island's modes take the few columns near the origin out of line; the others'
+// Phi_old are loaded eight at a time ahead of the arithmetic, since each store that follows
+// keeps the next load from moving above it (one mode at a time made a chain of E L2 latencies).
+template <typename T, int N, int E, int Q>
+__device__ __forceinline__ void gr_modes(const SpecOp& op, cplx<T>* v, int t, int ny, int nz, int field, double kf,
+                                         T kf2T, cplx<T>* old) {
+    typedef cplx<T> C;
+    const int nyz2 = ny * ny + nz * nz, nlo2 = op.n_lo * op.n_lo;
+    const GrOp<T> g(op, kf2T);
+    const T out = T(op.ac2_over_n3);
+    if (nyz2 <= nlo2) {
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int nx = (2 * m < E) ? t + m * Q : t + m * Q - N;
+            const int n2 = nx * nx + nyz2;
+            if (n2 <= nlo2) v[m] = gr_island_mode<T>(op, v[m], nx, ny, nz, n2, field, kf);
+        }
+    }
+    constexpr int G = E < 8 ? E : 8;
+#pragma unroll
+    for (int m0 = 0; m0 < E; m0 += G) {
+        C o[G];
+#pragma unroll
+        for (int m = 0; m < G; ++m)
+            o[m] = op.first ? cmake<C>(T(0), T(0)) : old[(size_t)(t + (m0 + m) * Q) * N];
+#pragma unroll
+        for (int m = m0; m < m0 + G; ++m) {
+            const int nx = (2 * m < E) ? t + m * Q : t + m * Q - N;
+            const int n2 = nx * nx + nyz2;
+            if (n2 > nlo2) {
+                const C P = g.solve(v[m], o[m - m0], n2);
+                old[(size_t)(t + m * Q) * N] = P;
+                v[m] = cscale(P, out);
+            }
+        }
+    }
+}
 
 // The per-mode operator of the x pass on mode (nx, ny, nz), |n|^2 = n2, of field `field`:
 // the Newtonian Green's function (or the potential alone), the Zel'dovich filter, or the
@@ -374,46 +424,11 @@ __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx,
                                                              : op.coef / (kf * kf) * amp[n2] / (double)n2;
         phi = (n2 == 0 || nyq) ? cmake<C>(T(0), T(0)) : cscale(g, T(filt));
     } else {  // OP_GR
-        // the FP64 island of field `field` ((n_lo + 1) (2 n_lo + 1)^2 modes a field)
-        if (n2 == 0) {
-            phi = cmake<C>(T(0), T(0));
-            if (op.n_lo > 0) {
-                const int L = op.n_lo, W2 = 2 * L + 1;
-                op.island[(((size_t)field * (L + 1) + nz) * W2 + L) * W2 + L] = make_double2(0.0, 0.0);
-            }
-        } else if (n2 <= op.n_lo * op.n_lo) {
-            const int L = op.n_lo, W2 = 2 * L + 1;
-            const size_t id = (((size_t)field * (L + 1) + nz) * W2 + (nx + L)) * W2 + (ny + L);
-            const double k2 = kf * kf * (double)n2;
-            const double H = op.calH;
-            const double num_s = -1.5 * H * H * op.omm_a;
-            double den = k2 + 3.0 * H * H + 4.5 * H * H * op.omm_a;
-            double2 P = make_double2(num_s * (double)vv.x, num_s * (double)vv.y);
-            if (!op.first) {
-                const double2 old = op.island[id];
-                const double cc = 3.0 * H * op.inv_dtau;
-                P.x += cc * old.x;
-                P.y += cc * old.y;
-                den += cc;
-            }
-            P.x /= den;
-            P.y /= den;
-            op.island[id] = P;
-            phi = cmake<C>(T(P.x * op.ac2_over_n3), T(P.y * op.ac2_over_n3));
+        if (n2 <= op.n_lo * op.n_lo) {
+            phi = gr_island_mode<T>(op, vv, nx, ny, nz, n2, field, kf);
         } else {
-            const T k2 = kf2T * T(n2);
-            const T H = T(op.calH), om = T(op.omm_a);
-            const T num_s = T(-1.5) * H * H * om;
-            T den = k2 + T(3) * H * H + T(4.5) * H * H * om;
-            C Pc = cscale(vv, num_s);
-            if (!op.first) {
-                const T cc = T(3) * H * T(op.inv_dtau);
-                const C o = *old;
-                Pc.x += cc * o.x;
-                Pc.y += cc * o.y;
-                den += cc;
-            }
-            Pc = cscale(Pc, div_mode(T(1), den));
+            const C o = op.first ? cmake<C>(T(0), T(0)) : *old;
+            const C Pc = GrOp<T>(op, kf2T).solve(vv, o, n2);
             *old = Pc;
             phi = cscale(Pc, T(op.ac2_over_n3));
         }
@@ -421,60 +436,43 @@ __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx,
     return phi;
 }
 
+// Registers of the x passes: kinds that hold a second sequence (phi beside its transform, or
+// the second field of a cross spectrum) take twice the data registers.
+template <typename T, int LOGN, int KIND> struct XRes {
+    static constexpr bool TWO = KIND != OP_FWD_STORE && KIND != OP_INV && KIND != OP_POTENTIAL;
+    static constexpr int DATA = plan_e(1 << LOGN) * 2 * (int)sizeof(T) / 4 * (TWO ? 2 : 1);  // registers
+    static constexpr int REGS = DATA <= 32 ? 64 : DATA <= 64 ? 104 : DATA <= 128 ? 168 : 255;
+    static constexpr int MINB = 65536 / (REGS * XShape<T, LOGN>::THREADS);
+};
+
+// CTAs walk blocks blk = blockIdx.x, + gridDim.x, ... of CB columns of one plane (plane =
+// blk / (N / CB)); several CTAs an SM overlap one another's loads, butterflies and stores.  The
+// binning pass runs one CTA for each row of bin sums, the others one for each block.
 template <typename T, int LOGN, int KIND>
-__global__ void __launch_bounds__(XShape<T, LOGN, KIND>::THREADS, XShape<T, LOGN, KIND>::MINB)
+__global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>::MINB)
     k_x_cols(cplx<T>* __restrict__ data, cplx<T>* __restrict__ out2, SpecOp op, int nplanes) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, M = S::M, Q = S::QN, CB = XShape<T, LOGN, KIND>::CB;
-    constexpr int CS = CB + 1;
-    constexpr int NCG = N / CB;                              // column groups per plane
-    constexpr int CHUNKS_ROW = CB * (int)sizeof(C) / 16;     // 16-byte chunks per row of a group
-    static_assert(CB * sizeof(C) % 16 == 0, "column groups of whole 16-byte chunks");
+    typedef XShape<T, LOGN> S;
+    constexpr int N = S::N, M = N / 2, E = S::E, Q = S::Q, CB = S::CB;
+    constexpr int NCG = N / CB;  // column groups per plane
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
-    const bool cross = (KIND == OP_BIN) && op.in2 != nullptr;
-    C* stage = buf + (size_t)2 * N * CS;                     // [1 + cross][N][CB]: field (and in2)
+    C* buf = reinterpret_cast<C*>(smem_raw);
     // OP_BIN: 1 / W^2 of the CIC window per |n_j| (W per axis from the FP64 table), in T
-    T* iw2 = reinterpret_cast<T*>(stage + (size_t)(cross ? 2 : 1) * N * CB);
+    T* iw2 = reinterpret_cast<T*>(buf + S::COL);
+    const bool cross = (KIND == OP_BIN) && op.in2 != nullptr;
     const int tid = threadIdx.x;
     const int b = tid % CB, t = tid / CB;
     const int64_t nblk = (int64_t)nplanes * NCG;
-    load_stage_twiddles<T, N>(tw);
-    if (KIND == OP_BIN)
-        for (int e = tid; e <= M; e += blockDim.x) iw2[e] = op.deconv ? T(1.0 / (op.wtab[e] * op.wtab[e])) : T(1);
+    const auto tw = tw_plan<T, N>();
+    CtaColEx<C, E, CB> ex{buf + b};
+    if constexpr (KIND == OP_BIN) {
+        for (int e = tid; e <= M; e += S::THREADS) iw2[e] = op.deconv ? T(1.0 / (op.wtab[e] * op.wtab[e])) : T(1);
+        __syncthreads();
+    }
     // OP_BIN: this CTA's row of per-bin sums in global memory (zeroed by the caller)
     double* acc_row = (KIND == OP_BIN) ? op.acc + (size_t)blockIdx.x * op.nbins : nullptr;
     // with a cross spectrum, optionally the auto spectrum of the second field in the same pass
     double* acc2_row = (KIND == OP_BIN && cross && op.acc2) ? op.acc2 + (size_t)blockIdx.x * op.nbins : nullptr;
-    auto issue = [&](int64_t blk) {
-        const size_t pb = (size_t)(blk / NCG) * N * N + (size_t)(blk % NCG) * CB;
-        if constexpr (KIND == OP_GR) {
-            // the Poisson-gauge constraint reads this block's Phi_old after the forward
-            // transform: its lines are brought into L2 now, one block ahead, with the data
-            constexpr int LINES = CB * (int)sizeof(C) >= 128 ? CB * (int)sizeof(C) / 128 : 1;
-            constexpr int THREADS = XShape<T, LOGN, KIND>::THREADS;  // the launch's block size
-            const C* ph = reinterpret_cast<const C*>(op.phi_old) + pb;
-#pragma unroll
-            for (int q0 = 0; q0 < N * LINES; q0 += THREADS) {
-                const int q = q0 + tid;
-                if (q < N * LINES)
-                    prefetch_l2(reinterpret_cast<const char*>(ph + (size_t)(q / LINES) * N) + 128 * (q % LINES));
-            }
-        }
-        for (int q = tid; q < N * CHUNKS_ROW; q += blockDim.x) {
-            const int r = q / CHUNKS_ROW, h = q % CHUNKS_ROW;
-            cp_async16(reinterpret_cast<char*>(stage + (size_t)r * CB) + 16 * h,
-                       reinterpret_cast<const char*>(data + pb + (size_t)r * N) + 16 * h);
-            if (cross)
-                cp_async16(reinterpret_cast<char*>(stage + (size_t)(N + r) * CB) + 16 * h,
-                           reinterpret_cast<const char*>(reinterpret_cast<const C*>(op.in2) + pb + (size_t)r * N) +
-                               16 * h);
-        }
-        cp_async_commit();
-    };
-    if ((int64_t)blockIdx.x < nblk) issue(blockIdx.x);
 #pragma unroll 1
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int plane = (int)(blk / NCG);
@@ -483,131 +481,143 @@ __global__ void __launch_bounds__(XShape<T, LOGN, KIND>::THREADS, XShape<T, LOGN
         const double kf = op.kf_arr ? op.kf_arr[field] : op.kf;
         const int c = (int)(blk % NCG) * CB + b;
         const size_t pbase = (size_t)plane * N * N;
-        C* base = data + pbase;
-        cp_async_wait_all();
-        __syncthreads();
-        C v[2][8];
+        C* base = data + pbase + c;
+        C v[1][E];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) v[0][m] = stage[(size_t)(t + m * Q) * CB + b];
-        if (cross) {
-#pragma unroll
-            for (int m = 0; m < 8; ++m) v[1][m] = stage[(size_t)(N + t + m * Q) * CB + b];
+        for (int m = 0; m < E; ++m) v[0][m] = base[(size_t)(t + m * Q) * N];
+        if constexpr (KIND == OP_GR) {
+            // the Poisson-gauge constraint reads the block's Phi_old after the forward transform:
+            // its lines are brought into L2 beside the data
+            constexpr int LINES = CB * (int)sizeof(C) >= 128 ? CB * (int)sizeof(C) / 128 : 1;
+            const C* ph = reinterpret_cast<const C*>(op.phi_old) + pbase + (c - b);
+            if (!op.first)
+                for (int q = tid; q < N * LINES; q += S::THREADS)
+                    prefetch_l2(reinterpret_cast<const char*>(ph + (size_t)(q / LINES) * N) + 128 * (q % LINES));
         }
-        __syncthreads();  // the stage is free: fetch the next block while this one is transformed
-        if (blk + gridDim.x < nblk) issue(blk + gridDim.x);
-        ColEx<C, N> ex{buf, CS, b};
-        if (op.fwd) {
-            if (cross) fft_regs<N, 2, false>(v, t, tw, ex);
-            else fft_regs<N, 1, false>(v, t, tw, ex);
-        }
+        if (op.fwd) fft_regs<N, 1, false>(v, t, tw, ex);
         if constexpr (KIND == OP_FWD_STORE) {
 #pragma unroll
-            for (int m = 0; m < 8; ++m) base[(size_t)(t + m * Q) * N + c] = v[0][m];
+            for (int m = 0; m < E; ++m) base[(size_t)(t + m * Q) * N] = v[0][m];
             continue;
         }
         if constexpr (KIND == OP_INV) {
             fft_regs<N, 1, true>(v, t, tw, ex);
 #pragma unroll
-            for (int m = 0; m < 8; ++m) base[(size_t)(t + m * Q) * N + c] = v[0][m];
+            for (int m = 0; m < E; ++m) base[(size_t)(t + m * Q) * N] = v[0][m];
             continue;
         }
-        if constexpr (KIND == OP_BIN) {
-            // regroup through the exchange buffer so that the thread holds kx = 8 t + m
-            // (m = 0..7): neighbouring kx mostly share a |k| bin, so runs merge in registers
-            __syncthreads();  // the transform's last exchange has been read
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                buf[(size_t)(t + m * Q) * CS + b] = v[0][m];
-                if (cross) buf[(size_t)(N + t + m * Q) * CS + b] = v[1][m];
-            }
-            __syncthreads();
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                v[0][m] = buf[(size_t)(8 * t + m) * CS + b];
-                if (cross) v[1][m] = buf[(size_t)(N + 8 * t + m) * CS + b];
-            }
-        }
-        // ---- per-mode operator on modes (kx = t + m Q, or 8 t + m when binning; ky = c, kz)
         const int ny = (c < M) ? c : c - N;
-        const int nz = kz;
-        // per-CTA constants, formed once in the working precision (no FP64 work per mode in FP32)
-        const T kfT = T(kf);
-        const T coefT = T(op.coef) / (kfT * kfT);
-        const T kf2T = T(kf * kf);
-        // OP_BIN: consecutive modes of a thread that fall in the same bin are summed in
-        // registers, each run added once to the CTA's row (native FP64 reduction in L2)
-        int run_bin = -1;
-        T run_sum = T(0), run_sum2 = T(0);
-        const T wyz = (KIND == OP_BIN) ? iw2[ny < 0 ? -ny : ny] * iw2[nz] * T((nz == 0 || nz == M) ? 1 : 2) : T(1);
-        // OP_BIN: the thread's modes kx = 8 t .. 8 t + 7 lie on one side of the Nyquist index, so
-        // |n|^2 is monotone over them, and a bin is a contiguous range of |n|^2: when the first
-        // and the last mode fall in the same bin (neither the zero mode nor beyond (n/2)^2), so
-        // do all eight, and two table lookups replace eight
-        int bin_all = -1;
+        const int nyz2 = ny * ny + kz * kz;
         if constexpr (KIND == OP_BIN) {
-            const int ia = 8 * t, ib = 8 * t + 7;
-            const int nxa = (ia < M) ? ia : ia - N, nxb = (ib < M) ? ib : ib - N;
-            const int n2a = nxa * nxa + ny * ny + nz * nz, n2b = nxb * nxb + ny * ny + nz * nz;
-            if (n2a > 0 && n2b > 0 && n2a <= M * M && n2b <= M * M) {
-                const int ba = op.bin_of[n2a], bb = op.bin_of[n2b];
-                if (ba == bb) bin_all = ba;
+            C u[1][E];
+            if (cross) {
+                const C* in2 = reinterpret_cast<const C*>(op.in2) + pbase + c;
+#pragma unroll
+                for (int m = 0; m < E; ++m) u[0][m] = in2[(size_t)(t + m * Q) * N];
+                fft_regs<N, 1, false>(u, t, tw, ex);
             }
-        }
-    #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int i = (KIND == OP_BIN) ? 8 * t + m : t + m * Q;
-            const int nx = (i < M) ? i : i - N;
-            const int n2 = nx * nx + ny * ny + nz * nz;
-            const C vv = v[0][m];
-            if constexpr (KIND == OP_BIN) {
-                if (n2 == 0 || n2 > M * M) continue;
-                const int bin = (bin_all >= 0) ? bin_all : op.bin_of[n2];
-                if (bin < 0) continue;
-                const C u = cross ? v[1][m] : vv;
-                // w |delta_n|^2 / W^2 (or the cross product), w = 1 on the kz = 0, n/2 planes, 2 elsewhere
-                const T wgt = iw2[nx < 0 ? -nx : nx] * wyz;
-                const T val = (vv.x * u.x + vv.y * u.y) * wgt;
-                const T val2 = acc2_row ? (u.x * u.x + u.y * u.y) * wgt : T(0);
-                if (bin != run_bin) {
-                    if (run_bin >= 0) {
-                        atomicAdd(acc_row + run_bin, (double)run_sum);
-                        if (acc2_row) atomicAdd(acc2_row + run_bin, (double)run_sum2);
+            // regroup through the exchange buffer so that the thread holds kx = E t + m
+            // (m = 0..E-1): neighbouring kx mostly share a |k| bin, so runs merge in registers
+            auto regroup = [&](C* w) {
+                __syncthreads();  // the buffer's last reads
+#pragma unroll
+                for (int m = 0; m < E; ++m) {
+                    const int i = t + m * Q;
+                    ex.col[(i + i / E) * CB] = w[m];
+                }
+                __syncthreads();
+#pragma unroll
+                for (int m = 0; m < E; ++m) w[m] = ex.put(t, m);
+            };
+            regroup(v[0]);
+            if (cross) regroup(u[0]);
+            // The thread's modes kx = E t .. E t + E - 1 lie on one side of the Nyquist index, so
+            // |n|^2 is monotone over them, and a bin is a contiguous range of |n|^2: when the first
+            // and the last mode of a group of eight fall in the same bin (neither the zero mode nor
+            // beyond (n/2)^2), so do all eight, and two table lookups replace eight.  Consecutive
+            // modes of a bin are summed in registers, each run added once to the CTA's row (native
+            // FP64 reduction in L2).
+            int run_bin = -1;
+            T run_sum = T(0), run_sum2 = T(0);
+            const T wyz = iw2[ny < 0 ? -ny : ny] * iw2[kz] * T((kz == 0 || kz == M) ? 1 : 2);
+            constexpr int G = E < 8 ? E : 8;
+#pragma unroll
+            for (int g = 0; g < E; g += G) {
+                const int ia = E * t + g, ib = ia + G - 1;
+                const int nxa = (ia < M) ? ia : ia - N, nxb = (ib < M) ? ib : ib - N;
+                const int n2a = nxa * nxa + nyz2, n2b = nxb * nxb + nyz2;
+                int bin_all = -1;
+                if (n2a > 0 && n2b > 0 && n2a <= M * M && n2b <= M * M) {
+                    const int ba = op.bin_of[n2a], bb = op.bin_of[n2b];
+                    if (ba == bb) bin_all = ba;
+                } else if (n2a > M * M && n2b > M * M) {
+                    continue;
+                }
+#pragma unroll
+                for (int m = g; m < g + G; ++m) {
+                    const int nx = nxa + (m - g);
+                    const int n2 = nx * nx + nyz2;
+                    if (n2 == 0 || n2 > M * M) continue;
+                    const int bin = (bin_all >= 0) ? bin_all : op.bin_of[n2];
+                    if (bin < 0) continue;
+                    const C vv = v[0][m], uu = cross ? u[0][m] : vv;
+                    // w |delta_n|^2 / W^2 (or the cross product), w = 1 on the kz = 0, n/2 planes, 2 elsewhere
+                    const T wgt = iw2[nx < 0 ? -nx : nx] * wyz;
+                    const T val = (vv.x * uu.x + vv.y * uu.y) * wgt;
+                    const T val2 = acc2_row ? (uu.x * uu.x + uu.y * uu.y) * wgt : T(0);
+                    if (bin != run_bin) {
+                        if (run_bin >= 0) {
+                            atomicAdd(acc_row + run_bin, (double)run_sum);
+                            if (acc2_row) atomicAdd(acc2_row + run_bin, (double)run_sum2);
+                        }
+                        run_bin = bin;
+                        run_sum = val;
+                        run_sum2 = val2;
+                    } else {
+                        run_sum += val;
+                        run_sum2 += val2;
                     }
-                    run_bin = bin;
-                    run_sum = val;
-                    run_sum2 = val2;
-                } else {
-                    run_sum += val;
-                    run_sum2 += val2;
-                }
-            } else {
-                const C phi = mode_op<T, KIND, N>(op, vv, nx, ny, nz, n2, field, kf, kfT, coefT, kf2T,
-                                                  reinterpret_cast<C*>(op.phi_old) + pbase + (size_t)i * N + c);
-                v[0][m] = phi;
-                if constexpr (KIND != OP_POTENTIAL) {
-                    const T kx = (2 * nx == -N) ? T(0) : kfT * T(nx);
-                    v[1][m] = cmake<C>(phi.y * kx, -phi.x * kx);  // -i kx phi
                 }
             }
-        }
-        if constexpr (KIND == OP_BIN) {
             if (run_bin >= 0) {
                 atomicAdd(acc_row + run_bin, (double)run_sum);
                 if (acc2_row) atomicAdd(acc2_row + run_bin, (double)run_sum2);
             }
             continue;
-        }
-        if constexpr (KIND == OP_POTENTIAL) {
-            fft_regs<N, 1, true>(v, t, tw, ex);
-    #pragma unroll
-            for (int m = 0; m < 8; ++m) base[(size_t)(t + m * Q) * N + c] = v[0][m];
         } else {
-            fft_regs<N, 2, true>(v, t, tw, ex);
-    #pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                base[(size_t)(t + m * Q) * N + c] = v[0][m];
-                out2[pbase + (size_t)(t + m * Q) * N + c] = v[1][m];
+            // ---- per-mode operator on modes (kx = t + m Q, ky = c, kz)
+            // per-thread constants, formed once in the working precision (no FP64 work per mode in FP32)
+            const T kfT = T(kf);
+            const T coefT = T(op.coef) / (kfT * kfT);
+            const T kf2T = T(kf * kf);
+            if constexpr (KIND == OP_GR) {
+                gr_modes<T, N, E, Q>(op, v[0], t, ny, kz, field, kf, kf2T,
+                                     reinterpret_cast<C*>(op.phi_old) + pbase + c);
+            } else {
+#pragma unroll
+                for (int m = 0; m < E; ++m) {
+                    const int i = t + m * Q;
+                    const int nx = (2 * m < E) ? i : i - N;
+                    v[0][m] = mode_op<T, KIND, N>(op, v[0][m], nx, ny, kz, nx * nx + nyz2, field, kf, kfT, coefT, kf2T,
+                                                  nullptr);
+                }
             }
+            if constexpr (KIND != OP_POTENTIAL) {
+                C u[1][E];
+#pragma unroll
+                for (int m = 0; m < E; ++m) {
+                    const int i = t + m * Q;
+                    const T kx = (2 * m == E && t == 0) ? T(0) : kfT * T(2 * m < E ? i : i - N);
+                    u[0][m] = cmake<C>(v[0][m].y * kx, -v[0][m].x * kx);  // -i kx phi
+                }
+                fft_regs<N, 1, true>(u, t, tw, ex);
+                C* o2 = out2 + pbase + c;
+#pragma unroll
+                for (int m = 0; m < E; ++m) o2[(size_t)(t + m * Q) * N] = u[0][m];
+            }
+            fft_regs<N, 1, true>(v, t, tw, ex);
+#pragma unroll
+            for (int m = 0; m < E; ++m) base[(size_t)(t + m * Q) * N] = v[0][m];
         }
     }
 }
@@ -681,11 +691,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     typedef typename SH::LAY LAY;
     constexpr int RS = LAY::RS, CS = CB + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
+    C* tws = reinterpret_cast<C*>(smem_raw);
+    const TwShared<C> tw{tws};
+    C* buf = tws + N;
     __shared__ unsigned s_item;
     const int tid = threadIdx.x;
-    load_stage_twiddles<T, N>(tw);
+    load_stage_twiddles<T, N>(tws);
     const unsigned rounds = (unsigned)(nplanes + 2 * lag);
     const unsigned total = rounds * 3 * ITEMS;
 #pragma unroll 1
@@ -813,10 +824,11 @@ __global__ void __launch_bounds__(PlaneShape<T, LOGN>::THREADS, PlaneShape<T, LO
     constexpr int N = SH::N, M = SH::M, Q = SH::Q, SEQ = SH::SEQ, ROUNDS = SH::ROUNDS;
     typedef RowLayout<N, false> LAY;  // a permutation within each row's N slots
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* P = tw + N;
+    C* tws = reinterpret_cast<C*>(smem_raw);
+    const TwShared<C> tw{tws};
+    C* P = tws + N;
     const int tid = threadIdx.x;
-    load_stage_twiddles<T, N>(tw);
+    load_stage_twiddles<T, N>(tws);
 #pragma unroll 1
     for (int plane = blockIdx.x; plane < nplanes; plane += gridDim.x) {
         const size_t pbase = (size_t)plane * N * N;
@@ -919,24 +931,20 @@ __global__ void __launch_bounds__(PlaneShape<T, LOGN>::THREADS, PlaneShape<T, LO
 // Poisson-gauge operator of AdjGrOp instead of c(k), with the carried spectrum gr.Z.  FD (the
 // first-order gradient): V is one scalar field and W = FFT_x V, without the i k_j factors.
 template <typename T, int LOGN, bool GR, bool FD>
-__global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_x_adj(const cplx<T>* V,
-                                                                      cplx<T>* out, double kf,
-                                                                      double coef, float4* __restrict__ zero,
-                                                                      int64_t nzero4, AdjGrOp gr) {
+__global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, OP_NEWTON>::MINB)
+    k_x_adj(const cplx<T>* V, cplx<T>* out, double kf, double coef, float4* __restrict__ zero, int64_t nzero4,
+            AdjGrOp gr) {
     typedef cplx<T> C;
-    typedef Shape<T, LOGN> S;
-    constexpr int N = S::N, M = S::M, Q = S::QN, CB = S::CB;
-    constexpr int CS = CB + 1;
+    typedef XShape<T, LOGN> S;
+    constexpr int N = S::N, M = N / 2, E = S::E, Q = S::Q, CB = S::CB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* tw = reinterpret_cast<C*>(smem_raw);
-    C* buf = tw + N;
     const int tid = threadIdx.x;
     const int b = tid % CB, t = tid / CB;
     const int kz = blockIdx.y;
     const int c = blockIdx.x * CB + b;
     const size_t pbase = (size_t)kz * N * N;
     const size_t field = (size_t)(M + 1) * N * N;
-    load_stage_twiddles<T, N>(tw);
+    const auto tw = tw_plan<T, N>();
     {  // side job: clear `zero` (a buffer the caller has finished with), grid-stride
         const int64_t nthr = (int64_t)gridDim.x * gridDim.y * blockDim.x;
         for (int64_t e = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + tid; e < nzero4; e += nthr)
@@ -947,109 +955,102 @@ __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) k_x_adj(const cpl
     const int ny = (c < M) ? c : c - N;
     const T kyT = (2 * ny == -N) ? T(0) : kfT * T(ny);
     const T kzT = (kz == M) ? T(0) : kfT * T(kz);
-    C acc[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) acc[m] = cmake<C>(T(0), T(0));
-    ColEx<C, N> ex{buf, CS, b};
+    C acc[1][E];
+    CtaColEx<C, E, CB> ex{reinterpret_cast<C*>(smem_raw) + b};
 #pragma unroll 1
     for (int j = 0; j < (FD ? 1 : 3); ++j) {
-        C v[1][8];
+        C v[1][E];
         const C* col = V + j * field + pbase + c;
 #pragma unroll
-        for (int m = 0; m < 8; ++m) v[0][m] = col[(size_t)(t + m * Q) * N];
-        if (j == 0) __syncthreads();  // twiddles loaded
+        for (int m = 0; m < E; ++m) v[0][m] = col[(size_t)(t + m * Q) * N];
         fft_regs<N, 1, false>(v, t, tw, ex);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
+        for (int m = 0; m < E; ++m) {
             const int i = t + m * Q;
-            const int nx = (i < M) ? i : i - N;
+            const int nx = (2 * m < E) ? i : i - N;
             const T kj = FD ? T(1) : (j == 0) ? ((2 * nx == -N) ? T(0) : kfT * T(nx)) : (j == 1 ? kyT : kzT);
-            acc[m].x += kj * v[0][m].x;
-            acc[m].y += kj * v[0][m].y;
+            const C a = j == 0 ? cmake<C>(T(0), T(0)) : acc[0][m];
+            acc[0][m] = cmake<C>(a.x + kj * v[0][m].x, a.y + kj * v[0][m].y);
         }
     }
-    C w[1][8];
     if constexpr (GR) {
         // per-evaluation constants in the working precision; den and src / carry per mode
         const T kf2 = kfT * kfT, H = T(gr.H), H1 = T(gr.H1);
         const T base = T(3) * H * H + T(4.5) * H * H * T(gr.om) + T(gr.cc);
         const T base1 = T(3) * H1 * H1 + T(4.5) * H1 * H1 * T(gr.om1) + T(gr.cc1);
         const T num = T(-1.5) * H * H * T(gr.om), cc1 = T(gr.cc1), KA = T(gr.K_ac2_n3);
-        C* Zc = reinterpret_cast<C*>(gr.Z);
+        C* Zc = reinterpret_cast<C*>(gr.Z) + pbase + c;
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
+        for (int m = 0; m < E; ++m) {
             const int i = t + m * Q;
-            const int nx = (i < M) ? i : i - N;
+            const int nx = (2 * m < E) ? i : i - N;
             const int n2 = nx * nx + ny * ny + kz * kz;
             const T k2 = kf2 * T(n2);
             const T src = (n2 == 0) ? T(0) : div_mode(num, k2 + base);
             const T carry = (n2 == 0) ? T(0) : div_mode(cc1, k2 + base1);
-            const size_t zi = pbase + (size_t)i * N + c;
-            const C zo = Zc[zi];
+            C* zi = Zc + (size_t)i * N;
+            const C zo = *zi, a = acc[0][m];
             // K a c^2 W + carry Z, W = i acc (spectral gradient) or acc (first order)
-            const C Z = FD ? cmake<C>(KA * acc[m].x + carry * zo.x, KA * acc[m].y + carry * zo.y)
-                           : cmake<C>(-KA * acc[m].y + carry * zo.x, KA * acc[m].x + carry * zo.y);
-            Zc[zi] = Z;
-            w[0][m] = cscale(Z, src);
+            const C Z = FD ? cmake<C>(KA * a.x + carry * zo.x, KA * a.y + carry * zo.y)
+                           : cmake<C>(-KA * a.y + carry * zo.x, KA * a.x + carry * zo.y);
+            *zi = Z;
+            acc[0][m] = cscale(Z, src);
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
+        for (int m = 0; m < E; ++m) {
             const int i = t + m * Q;
-            const int nx = (i < M) ? i : i - N;
+            const int nx = (2 * m < E) ? i : i - N;
             const int n2 = nx * nx + ny * ny + kz * kz;
             const T cc = (n2 == 0) ? T(0) : coefT / T(n2);
-            w[0][m] = FD ? cscale(acc[m], cc) : cmake<C>(-cc * acc[m].y, cc * acc[m].x);  // (i) c sum_j k_j V_j
+            const C a = acc[0][m];
+            acc[0][m] = FD ? cscale(a, cc) : cmake<C>(-cc * a.y, cc * a.x);  // (i) c sum_j k_j V_j
         }
     }
-    fft_regs<N, 1, true>(w, t, tw, ex);
+    fft_regs<N, 1, true>(acc, t, tw, ex);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) out[pbase + (size_t)(t + m * Q) * N + c] = w[0][m];
+    for (int m = 0; m < E; ++m) out[pbase + (size_t)(t + m * Q) * N + c] = acc[0][m];
 }
 
 // =============================================================== launchers
 template <typename T, int LOGN>
 cudaError_t z_r2c_n(const T* in, cplx<T>* out, int rows, cudaStream_t st, double sub = 0.0) {
-    typedef Shape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * (S::M + ((S::M + 2) & ~1) + (size_t)S::YB * RowLayout<S::M, true>::RS);
-    cudaError_t e = set_smem((const void*)k_z_r2c<T, LOGN>, smem);
+    typedef ZShape<T, LOGN> S;
+    cudaError_t e = set_smem((const void*)k_z_r2c<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    k_z_r2c<T, LOGN><<<dim3(S::N / S::YB, rows), S::YB * S::QM, smem, st>>>(in, out, (T)sub);
+    k_z_r2c<T, LOGN><<<dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st>>>(in, out, (T)sub);
     return cudaGetLastError();
 }
 
 template <typename T, int LOGN>
 cudaError_t z_c2r_n(const Ptr3<T>& P, int ncomp, int rows, unsigned mask, double kf, cudaStream_t st,
                     const double* kf_arr) {
-    typedef Shape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * (S::M + (size_t)S::YB * RowLayout<S::M, true>::RS);
-    cudaError_t e = set_smem((const void*)k_z_c2r<T, LOGN>, smem);
+    typedef ZShape<T, LOGN> S;
+    cudaError_t e = set_smem((const void*)k_z_c2r<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    k_z_c2r<T, LOGN><<<dim3(S::N / S::YB, rows, ncomp), S::YB * S::QM, smem, st>>>(P, mask, (T)kf, kf_arr);
+    k_z_c2r<T, LOGN><<<dim3(S::N / S::YB, rows, ncomp), S::THREADS, S::SMEM, st>>>(P, mask, (T)kf, kf_arr);
     return cudaGetLastError();
 }
 
 template <typename T, int LOGN, bool INV>
 cudaError_t y_rows_n(const cplx<T>* in, cplx<T>* out, int64_t nrows, cudaStream_t st) {
-    typedef Shape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * (S::N + 2 * (size_t)S::RB * RowLayout<S::N, false>::RS);
-    cudaError_t e = set_smem((const void*)k_y_rows<T, LOGN, INV>, smem);
+    typedef YShape<T, LOGN> S;
+    cudaError_t e = set_smem((const void*)k_y_rows<T, LOGN, INV>, S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t nblk = (nrows + S::RB - 1) / S::RB;
-    k_y_rows<T, LOGN, INV><<<(unsigned)nblk, S::RB * S::QN, smem, st>>>(in, out, nrows);
+    k_y_rows<T, LOGN, INV><<<(unsigned)nblk, S::THREADS, S::SMEM, st>>>(in, out, nrows);
     return cudaGetLastError();
 }
 
 template <typename T, int LOGN>
 cudaError_t y_grad3_n(const cplx<T>* A, const cplx<T>* B, cplx<T>* Ao, cplx<T>* Bo, cplx<T>* Co, int64_t nrows, double kf,
                       cudaStream_t st, const double* kf_arr, int64_t rows_per_field) {
-    typedef Shape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * (S::N + 2 * (size_t)S::RB3 * RowLayout<S::N, false>::RS);
-    cudaError_t e = set_smem((const void*)k_y_grad3<T, LOGN>, smem);
+    typedef YShape<T, LOGN> S;
+    cudaError_t e = set_smem((const void*)k_y_grad3<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    const int64_t nblk = (nrows + S::RB3 - 1) / S::RB3;
-    k_y_grad3<T, LOGN><<<(unsigned)nblk, S::RB3 * S::QN, smem, st>>>(A, B, Ao, Bo, Co, nrows, (T)kf, kf_arr,
-                                                                       rows_per_field);
+    const int64_t nblk = (nrows + S::RB - 1) / S::RB;
+    k_y_grad3<T, LOGN><<<(unsigned)nblk, S::THREADS, S::SMEM, st>>>(A, B, Ao, Bo, Co, nrows, (T)kf, kf_arr,
+                                                                    rows_per_field);
     return cudaGetLastError();
 }
 
@@ -1081,24 +1082,21 @@ cudaError_t inverse_yz_grad_n(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const
 
 template <typename T, int LOGN, int KIND>
 cudaError_t x_cols_n(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp& op, cudaStream_t st) {
-    typedef Shape<T, LOGN> S;
-    typedef XShape<T, LOGN, KIND> X;
-    const int nstage = (KIND == OP_BIN && op.in2 != nullptr) ? 2 : 1;
-    const size_t smem = sizeof(cplx<T>) * (S::N + 2 * (size_t)S::N * (X::CB + 1) + nstage * (size_t)S::N * X::CB) +
-                        (KIND == OP_BIN ? sizeof(T) * (S::M + 1) : 0);
+    typedef XShape<T, LOGN> S;
+    const size_t smem = sizeof(cplx<T>) * S::COL + (KIND == OP_BIN ? sizeof(T) * (S::N / 2 + 1) : 0);
     const void* fn = (const void*)k_x_cols<T, LOGN, KIND>;
     cudaError_t e = set_smem(fn, smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 1;
-    e = resident_ctas(fn, X::THREADS, smem, &per_sm);
-    if (e != cudaSuccess) return e;
-    const int64_t nblk = (int64_t)nplanes * (S::N / X::CB);
-    int64_t grid = std::min<int64_t>(nblk, (int64_t)per_sm * num_sms());
-    if (KIND == OP_BIN) grid = std::min<int64_t>(grid, op.acc_rows);  // one row of bin sums per CTA
-    k_x_cols<T, LOGN, KIND><<<(unsigned)grid, X::THREADS, smem, st>>>(data, out2, op, nplanes);
+    int64_t grid = (int64_t)nplanes * (S::N / S::CB);
+    if (KIND == OP_BIN) {  // one row of bin sums per CTA
+        int per_sm = 1;
+        e = resident_ctas(fn, S::THREADS, smem, &per_sm);
+        if (e != cudaSuccess) return e;
+        grid = std::min<int64_t>(grid, std::min<int64_t>((int64_t)per_sm * num_sms(), op.acc_rows));
+    }
+    k_x_cols<T, LOGN, KIND><<<(unsigned)grid, S::THREADS, smem, st>>>(data, out2, op, nplanes);
     return cudaGetLastError();
 }
-
 
 template <typename T, int LOGN, int THREADS>
 cudaError_t middle_n(cplx<T>* A, cplx<T>* B, cplx<T>* Cs, int nplanes, const SpecOp& op, unsigned* sync_words,
@@ -1155,11 +1153,11 @@ cudaError_t plane_n(cplx<T>* A, cplx<T>* GX, cplx<T>* GY, int nplanes, const Spe
 template <typename T, int LOGN, bool GR, bool FD>
 cudaError_t x_adj_k(const cplx<T>* V, cplx<T>* out, double kf, double coef, float* zero, int64_t nzero, cudaStream_t st,
                     const AdjGrOp& gr) {
-    typedef Shape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * (S::N + 2 * (size_t)S::N * (S::CB + 1));
+    typedef XShape<T, LOGN> S;
+    const size_t smem = sizeof(cplx<T>) * S::COL;
     cudaError_t e = set_smem((const void*)k_x_adj<T, LOGN, GR, FD>, smem);
     if (e != cudaSuccess) return e;
-    k_x_adj<T, LOGN, GR, FD><<<dim3(S::N / S::CB, S::M + 1), S::CB * S::QN, smem, st>>>(
+    k_x_adj<T, LOGN, GR, FD><<<dim3(S::N / S::CB, S::N / 2 + 1), S::THREADS, smem, st>>>(
         V, out, kf, coef, (float4*)zero, zero ? nzero / 4 : 0, gr);
     return cudaGetLastError();
 }

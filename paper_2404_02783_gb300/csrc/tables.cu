@@ -8,12 +8,13 @@
 #include <tuple>
 #include <utility>
 
+#include "fft.cuh"
 #include "internal.h"
 
 namespace pm {
 
-cudaError_t upload_twiddles_f32(const float2* host);
-cudaError_t upload_twiddles_f64(const double2* host);
+cudaError_t upload_twiddles_f32(const float2* host, const float2* stages);
+cudaError_t upload_twiddles_f64(const double2* host, const double2* stages);
 
 static std::mutex g_tab_mutex;
 static bool g_tab_ready[128];
@@ -40,9 +41,25 @@ cudaError_t ensure_device_tables() {
         h64[k] = make_double2(c, s);
         h32[k] = make_float2((float)c, (float)s);
     }
-    e = upload_twiddles_f32(h32);
+    // per-stage tables of the plan_e transforms (fft.cuh: tw_stage_offset), length L at [L, 2 L)
+    static float2 s32[2048];
+    static double2 s64[2048];
+    for (int L = 8; L <= 1024; L *= 2) {
+        const int E = plan_e(L);
+        for (int Ns = radix_at(L, 1, E); Ns < L; Ns *= radix_at(L, Ns, E)) {
+            const int R = radix_at(L, Ns, E);
+            for (int r = 1; r < R; ++r)
+                for (int jm = 0; jm < Ns; ++jm) {
+                    const int at = L + tw_stage_offset(L, E, Ns) + (r - 1) * Ns + jm;
+                    const int k = (jm * r * (1024 / (Ns * R))) % 1024;
+                    s32[at] = h32[k];
+                    s64[at] = h64[k];
+                }
+        }
+    }
+    e = upload_twiddles_f32(h32, s32);
     if (e != cudaSuccess) return e;
-    e = upload_twiddles_f64(h64);
+    e = upload_twiddles_f64(h64, s64);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 128) g_tab_ready[dev] = true;
     return cudaSuccess;
