@@ -66,24 +66,6 @@ __global__ void k_adj_gather(const uint32_t* __restrict__ x, int64_t count, int 
     }
 }
 
-// lam_u += K sum_j v_j grad_u interp(G_j)  (the direct part of the transposed kick)
-__global__ void k_adj_direct(const uint32_t* __restrict__ x, int64_t count, int logn, float inv_cell_ticks,
-                             const float* __restrict__ v, const float* __restrict__ G0, const float* __restrict__ G1,
-                             const float* __restrict__ G2, float K, float* __restrict__ lam_u) {
-    const size_t n = (size_t)1 << logn;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const Cic1 cx = decode(x[i], logn, inv_cell_ticks), cy = decode(x[count + i], logn, inv_cell_ticks),
-                   cz = decode(x[2 * count + i], logn, inv_cell_ticks);
-        const float v0 = v[i], v1 = v[count + i], v2 = v[2 * count + i];
-        float g0[3], g1[3], g2[3];
-        grad_gather(G0, n, cx, cy, cz, g0);
-        grad_gather(G1, n, cx, cy, cz, g1);
-        grad_gather(G2, n, cx, cy, cz, g2);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) lam_u[j * count + i] += K * (v0 * g0[j] + v1 * g1[j] + v2 * g2[j]);
-    }
-}
-
 // The particle side of the transposed kick at positions x (one pass, the next particle's
 // inputs loaded one iteration ahead):
 //   lam_u += K sum_j v_j grad_u interp(G_j) + K mass grad_u interp(rho_bar)
@@ -91,10 +73,10 @@ __global__ void k_adj_direct(const uint32_t* __restrict__ x, int64_t count, int 
 //   v += drift_next lam_u   (v = lam_p, updated in place).
 __global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* __restrict__ x, int64_t count, int logn,
                                                   float inv_cell_ticks, float* __restrict__ v,
-                                                  const float* __restrict__ G0, const float* __restrict__ G1,
-                                                  const float* __restrict__ G2, const float* __restrict__ rho_bar,
+                                                  const float* __restrict__ G, const float* __restrict__ rho_bar,
                                                   float K, float Km, float drift_next, float* __restrict__ lam_u) {
-    const float nf = (float)(1 << logn);
+    const int n = 1 << logn;
+    const float nf = (float)n;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t nx0 = 0, nx1 = 0, nx2 = 0;
@@ -124,9 +106,10 @@ __global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* __restrict__ x
             for (int b = 0; b < 2; ++b)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    const uint32_t o = (((ix[a] << logn) + iy[b]) << logn) + iz[c];
+                    const uint32_t row = ((ix[a] << logn) + iy[b]) << logn, o = row + iz[c];
+                    const float* Go = G + (kForceRows * row + iz[c]);
                     // K sum_j v_j G_j + K mass rho_bar at the corner
-                    const float s = K * (v0 * __ldg(G0 + o) + v1 * __ldg(G1 + o) + v2 * __ldg(G2 + o)) +
+                    const float s = K * (v0 * __ldg(Go) + v1 * __ldg(Go + n) + v2 * __ldg(Go + 2 * n)) +
                                     Km * __ldg(rho_bar + o);
                     g0 = fmaf(dw[a] * wy[b] * wz[c], s, g0);
                     g1 = fmaf(wx[a] * dw[b] * wz[c], s, g1);
@@ -363,19 +346,11 @@ cudaError_t adj_gather(const uint32_t* x, int64_t count, int n, const float* F, 
     return cudaGetLastError();
 }
 
-cudaError_t adj_direct(const uint32_t* x, int64_t count, int n, const float* v, const float* const* G, float K,
-                       float* lam_u, cudaStream_t st) {
-    const int logn = ilog2(n);
-    k_adj_direct<<<blocks_for(count), 256, 0, st>>>(x, count, logn, (float)ldexp(1.0, -(32 - logn)), v, G[0], G[1],
-                                                    G[2], K, lam_u);
-    return cudaGetLastError();
-}
-
-cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v, const float* const* G,
+cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v, const float* G,
                                const float* rho_bar, float K, float Km, float drift_next, float* lam_u,
                                cudaStream_t st) {
     const int logn = ilog2(n);
-    k_adj_kick<<<blocks_for(count), 256, 0, st>>>(x, count, logn, (float)ldexp(1.0, -(32 - logn)), v, G[0], G[1], G[2],
+    k_adj_kick<<<blocks_for(count), 256, 0, st>>>(x, count, logn, (float)ldexp(1.0, -(32 - logn)), v, G,
                                                   rho_bar, K, Km, drift_next, lam_u);
     return cudaGetLastError();
 }

@@ -149,7 +149,8 @@ struct pm_ctx {
     // when set, the force meshes of the step (three n^3 meshes back to back) live here
     // instead of L.force (the gradient's forward re-run writes them straight into its record)
     void* force_at = nullptr;
-    void* force(int j) { return force_at ? (void*)((char*)force_at + (size_t)j * n * n * n * sT()) : at(L.force[j]); }
+    // the three force meshes (layout kForceRows), or the potential of the first-order gradient
+    void* force() { return force_at ? force_at : at(L.force[0]); }
     // when set, the positions of the step are read from x_at and the fused update writes the
     // drifted ones to x_out (the gradient's re-run records each step's positions this way)
     void* x_at = nullptr;
@@ -373,7 +374,7 @@ pm_status compute_forces_t(pm_ctx* c, double a) {
         op.island = c->L.has_island ? (double2*)c->at(c->L.island) : nullptr;
     }
     if (c->cfg.gradient == PM_GRAD_FD1) {
-        // the potential alone goes back to real space (force(0)); the update differentiates
+        // the potential alone goes back to real space (force()); the update differentiates
         // its CIC interpolant (the Poisson-gauge pass still writes its x gradient, unused)
         if (op.kind == OP_NEWTON) op.kind = OP_POTENTIAL;
         {
@@ -383,7 +384,7 @@ pm_status compute_forces_t(pm_ctx* c, double a) {
         Phase ph(c, PM_PHASE_FFT_YZ_INV);
         PM_CK((y_rows<T, true>(s0, (int64_t)(n / 2 + 1) * n, n, c->st)));
         const cplx<T>* in[1] = {s0};
-        T* out[1] = {(T*)c->force(0)};
+        T* out[1] = {(T*)c->force()};
         PM_CK(z_c2r<T>(in, out, 1, n, 1, 0u, 0.0, c->st, nullptr, clear));
     } else if (plane_middle(c)) {
         {
@@ -392,8 +393,9 @@ pm_status compute_forces_t(pm_ctx* c, double a) {
         }
         Phase ph(c, PM_PHASE_FFT_YZ_INV);
         const cplx<T>* in[3] = {s1, s2, s0};  // -i k_j phi back along x and y, j = x, y, z
-        T* out[3] = {(T*)c->force(0), (T*)c->force(1), (T*)c->force(2)};
-        PM_CK(z_c2r<T>(in, out, 3, n, 1, 0u, c->kf, c->st, nullptr, clear));
+        T* f = (T*)c->force();
+        T* out[3] = {f, f + n, f + 2 * n};
+        PM_CK(z_c2r<T>(in, out, 3, n, 1, 0u, c->kf, c->st, nullptr, clear, kForceRows));
     } else if (fused_middle(c)) {
         // z r2c above left the half spectrum in s0 before its forward y pass (see forward_to_y)
         {
@@ -402,16 +404,18 @@ pm_status compute_forces_t(pm_ctx* c, double a) {
         }
         Phase ph(c, PM_PHASE_FFT_YZ_INV);
         const cplx<T>* in[3] = {s1, s2, s0};  // IFFT_y(-i kx phi), IFFT_y(-i ky phi), IFFT_y(phi) (-i kz)
-        T* out[3] = {(T*)c->force(0), (T*)c->force(1), (T*)c->force(2)};
-        PM_CK(z_c2r<T>(in, out, 3, n, 1, 4u, c->kf, c->st, nullptr, clear));
+        T* f = (T*)c->force();
+        T* out[3] = {f, f + n, f + 2 * n};
+        PM_CK(z_c2r<T>(in, out, 3, n, 1, 4u, c->kf, c->st, nullptr, clear, kForceRows));
     } else {
         {
             Phase ph(c, PM_PHASE_FFT_X_GREEN);
             PM_CK(x_cols<T>(s0, s1, n / 2 + 1, n, op, c->st));
         }
         Phase ph(c, PM_PHASE_FFT_YZ_INV);
-        T* out[3] = {(T*)c->force(0), (T*)c->force(1), (T*)c->force(2)};
-        PM_CK(inverse_yz_grad<T>(s0, s1, s2, out, n, 1, c->kf, c->st, nullptr, clear));
+        T* f = (T*)c->force();
+        T* out[3] = {f, f + n, f + 2 * n};
+        PM_CK(inverse_yz_grad<T>(s0, s1, s2, out, n, 1, c->kf, c->st, nullptr, clear, kForceRows));
     }
     if (c->cfg.mode == PM_GR_POISSON) {
         c->have_phi = true;
@@ -426,8 +430,8 @@ pm_status compute_forces(pm_ctx* c, double a) {
 
 pm_status kick_drift(pm_ctx* c, double kick, double drift) {
     Phase ph(c, PM_PHASE_KICK_DRIFT);
-    void* g[3] = {c->force(0), c->force(1), c->force(2)};
-    // first-order gradient: force(0) holds the potential, differentiated across the cell of spacing L/n
+    const void* g = c->force();
+    // first-order gradient: force() holds the potential, differentiated across the cell of spacing L/n
     const double fd_inv_d = c->cfg.gradient == PM_GRAD_FD1 ? c->n / c->cfg.box : 0.0;
     if (fused_update(c)) {
         PM_CK(interp_kick_drift_deposit(c->xpos(), c->at(c->L.p), c->np, c->cfg.precision, c->n, g, kick, drift,
@@ -1365,7 +1369,6 @@ pm_status adj_kick(pm_ctx* c, const uint32_t* xs, const float* gs, double K, flo
                    double drift_next, const AdjGrOp* gr = nullptr) {
     const int n = c->n;
     const size_t n3 = (size_t)n * n * n;
-    const float* G[3] = {gs, gs + n3, gs + 2 * n3};
     // V_j and the spectra are three meshes back to back (256-byte multiples): one batched transform
     float* V[3] = {(float*)c->at(c->L.force[0]), (float*)c->at(c->L.force[1]), (float*)c->at(c->L.force[2])};
     const double mass = std::pow((double)n / c->np, 3);
@@ -1402,7 +1405,7 @@ pm_status adj_kick(pm_ctx* c, const uint32_t* xs, const float* gs, double K, flo
     float* zout[1] = {rho_bar};
     PM_CK(z_c2r<float>(zin, zout, 1, n, 1, 0u, 0.0, c->st));
     // Newtonian: rho_bar lacks this evaluation's K; Poisson gauge: Z carries every K already
-    PM_CK(adj_kick_particles(xs, c->np3, n, lam_p, G, rho_bar, (float)K, (float)(gr ? mass : K * mass),
+    PM_CK(adj_kick_particles(xs, c->np3, n, lam_p, gs, rho_bar, (float)K, (float)(gr ? mass : K * mass),
                              (float)drift_next, lam_u, c->st));
     return PM_OK;
 }
@@ -1867,25 +1870,25 @@ pm_status batch_forces(pm_batch* b, cudaStream_t s, int r0, int c) {
         op.phi_old = (float2*)b->at(b->PHI) + r0 * nspec;
         op.island = b->isl ? (double2*)((unsigned char*)b->at(b->ISL) + r0 * b->isl) : nullptr;
     }
-    float* out[3] = {(float*)b->at(b->FORCE[0]) + r0 * n3, (float*)b->at(b->FORCE[1]) + r0 * n3,
-                     (float*)b->at(b->FORCE[2]) + r0 * n3};
+    // realisation r's force meshes at 3 r n^3 of the three arrays, which lie back to back
+    float* f = (float*)b->at(b->FORCE[0]) + 3 * r0 * n3;
+    float* out[3] = {f, f + n, f + 2 * n};
     if (plane) {
         // whole kz planes in shared memory: the three gradient spectra, then the z pass
         PM_CK(fft_plane<float>(s0, s1, s2, c * (M + 1), n, op, s));
         const float2* in[3] = {s1, s2, s0};
-        PM_CK(z_c2r<float>(in, out, 3, n, c, 0u, 0.0, s, nullptr, rho));
+        PM_CK(z_c2r<float>(in, out, 3, n, c, 0u, 0.0, s, nullptr, rho, kForceRows));
         return PM_OK;
     }
     PM_CK(x_cols<float>(s0, s1, c * (M + 1), n, op, s));
-    PM_CK(inverse_yz_grad<float>(s0, s1, s2, out, n, c, 0.0, s, kf, rho));
+    PM_CK(inverse_yz_grad<float>(s0, s1, s2, out, n, c, 0.0, s, kf, rho, kForceRows));
     return PM_OK;
 }
 
 pm_status batch_update(pm_batch* b, double kick, double drift, cudaStream_t s, int r0, int c) {
     const size_t n3 = (size_t)b->cfg.nmesh * b->cfg.nmesh * b->cfg.nmesh;
     const size_t np3 = (size_t)b->cfg.np * b->cfg.np * b->cfg.np;
-    void* g[3] = {(float*)b->at(b->FORCE[0]) + r0 * n3, (float*)b->at(b->FORCE[1]) + r0 * n3,
-                  (float*)b->at(b->FORCE[2]) + r0 * n3};
+    const void* g = (const float*)b->at(b->FORCE[0]) + 3 * r0 * n3;
     const double mass = std::pow((double)b->cfg.nmesh / b->cfg.np, 3);
     PM_CK(interp_kick_drift_deposit((uint32_t*)b->at(b->X) + r0 * 3 * np3, (float*)b->at(b->P) + r0 * 3 * np3,
                                     b->cfg.np, PM_FP32_FIXED, b->cfg.nmesh, g, kick, drift, 1.0, mass,

@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MIN
 template <typename T> struct Ptr3 {
     const cplx<T>* in[3];
     T* out[3];
-    T* zero = nullptr;  // optional mesh of the same shape as out, set to 0 by the component-0 CTAs
+    T* zero = nullptr;  // optional plain mesh, set to 0 by the component-0 CTAs
+    int rows = 1;       // row r of out[j] at out[j] + r rows n
 };
 
 template <typename T, int LOGN>
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MIN
     for (int m = 0; m < E; ++m) v[0][m] = z[t + m * Q];
     WarpRowEx<C, E> ex{z};
     fft_regs<M, 1, true>(v, t, tw_plan<T, M>(), ex);
-    C* orow = reinterpret_cast<C*>(pout + ((size_t)gl * N + y0 + b) * N);
+    C* orow = reinterpret_cast<C*>(pout + ((size_t)gl * N + y0 + b) * N * P.rows);
 #pragma unroll
     for (int m = 0; m < E; ++m) orow[t + m * Q] = v[0][m];
     if (P.zero && comp == 0) {  // the same rows of the mesh the caller clears for its next use
@@ -1066,7 +1067,7 @@ cudaError_t forward_zy_n(const T* in, cplx<T>* spec, int batch, cudaStream_t st,
 // one half spectrum for IFFT_y(-i ky A).
 template <typename T, int LOGN>
 cudaError_t inverse_yz_grad_n(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const* out, int batch, double kf,
-                              const double* kf_arr, cudaStream_t st, T* zero) {
+                              const double* kf_arr, cudaStream_t st, T* zero, int rows_out) {
     constexpr int N = 1 << LOGN, M = N / 2;
     const int64_t rows = (int64_t)batch * (M + 1) * N;
     cudaError_t e = y_grad3_n<T, LOGN>(A, B, A, B, scratch, rows, kf, st, kf_arr, (int64_t)(M + 1) * N);
@@ -1077,6 +1078,7 @@ cudaError_t inverse_yz_grad_n(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const
     P.in[2] = A;        // IFFT_y(phi), -i kz  -> g_z
     for (int j = 0; j < 3; ++j) P.out[j] = out[j];
     P.zero = zero;
+    P.rows = rows_out;
     return z_c2r_n<T, LOGN>(P, 3, N * batch, 4u, kf, st, kf_arr);
 }
 
@@ -1207,8 +1209,9 @@ cudaError_t z_r2c(const T* in, cplx<T>* out, int n, int batch, cudaStream_t st, 
 
 template <typename T>
 cudaError_t z_c2r(const cplx<T>* const* in, T* const* out, int ncomp, int n, int batch, unsigned gradz_mask,
-                  double kf, cudaStream_t st, const double* kf_arr, T* zero) {
+                  double kf, cudaStream_t st, const double* kf_arr, T* zero, int rows) {
     Ptr3<T> P;
+    P.rows = rows;
     for (int j = 0; j < 3; ++j) {
         P.in[j] = in[j < ncomp ? j : 0];
         P.out[j] = out[j < ncomp ? j : 0];
@@ -1271,8 +1274,8 @@ cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_
 
 template <typename T>
 cudaError_t inverse_yz_grad(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const* out, int n, int batch, double kf,
-                            cudaStream_t st, const double* kf_arr, T* zero) {
-    PM_DISPATCH_LOGN(n, (inverse_yz_grad_n<T, LG>(A, B, scratch, out, batch, kf, kf_arr, st, zero)))
+                            cudaStream_t st, const double* kf_arr, T* zero, int rows) {
+    PM_DISPATCH_LOGN(n, (inverse_yz_grad_n<T, LG>(A, B, scratch, out, batch, kf, kf_arr, st, zero, rows)))
 }
 
 template <typename T>
@@ -1283,7 +1286,7 @@ cudaError_t x_cols(cplx<T>* data, cplx<T>* out2, int nplanes, int n, const SpecO
 #define PM_INST(T)                                                                                     \
     template cudaError_t z_r2c<T>(const T*, cplx<T>*, int, int, cudaStream_t, double);                 \
     template cudaError_t z_c2r<T>(const cplx<T>* const*, T* const*, int, int, int, unsigned, double,  \
-                                  cudaStream_t, const double*, T*);                                    \
+                                  cudaStream_t, const double*, T*, int);                               \
     template cudaError_t y_rows<T, false>(cplx<T>*, int64_t, int, cudaStream_t);                      \
     template cudaError_t y_rows<T, true>(cplx<T>*, int64_t, int, cudaStream_t);                       \
     template cudaError_t y_rows_grad3<T>(cplx<T>*, cplx<T>*, cplx<T>*, int64_t, int, double,           \
@@ -1293,6 +1296,6 @@ cudaError_t x_cols(cplx<T>* data, cplx<T>* out2, int nplanes, int n, const SpecO
     template cudaError_t x_adj<T>(const cplx<T>*, cplx<T>*, int, double, double, cudaStream_t, float*, \
                                   int64_t, const AdjGrOp*, bool);                                       \
     template cudaError_t inverse_yz_grad<T>(cplx<T>*, cplx<T>*, cplx<T>*, T* const*, int, int, double,   \
-                                            cudaStream_t, const double*, T*);
+                                            cudaStream_t, const double*, T*, int);
 
 }  // namespace pm

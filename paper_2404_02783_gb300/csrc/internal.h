@@ -71,12 +71,17 @@ cudaError_t div_mode_check(const double* a, const double* d, int64_t count, doub
 // input value (a density's mean: only the zero mode changes).
 template <typename T>
 cudaError_t z_r2c(const T* in, cplx<T>* out, int n, int batch, cudaStream_t st, double sub = 0.0);
+// Layout of the force meshes: the three components' z rows side by side, [x][y][3][z], so that
+// the particle kernels reach all three with one address (component j of cell (x, y, z) at
+// ((x n + y) 3 + j) n + z).  The transforms write component j's row r at out[j] + r rows n with
+// rows = kForceRows and out[j] = out[0] + j n.
+constexpr int kForceRows = 3;
 // out_j = c2r(in_j [* -i kf kz when gradz_mask bit j is set]) for the ncomp fields; zero (if
 // given, a mesh of the outputs' shape that the caller has finished with) is cleared beside them
 template <typename T>
 cudaError_t z_c2r(const cplx<T>* const* in, T* const* out, int ncomp, int n, int batch,
                   unsigned gradz_mask, double kf, cudaStream_t st, const double* kf_arr = nullptr,
-                  T* zero = nullptr);
+                  T* zero = nullptr, int rows = 1);
 template <typename T, bool INV>
 cudaError_t y_rows(cplx<T>* data, int64_t nrows, int n, cudaStream_t st);
 // A <- IFFT_y(A), B <- IFFT_y(B), C <- IFFT_y(-i ky A); kf_arr (optional) gives the kf of
@@ -140,6 +145,6 @@ cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_
 // zero (optional): a mesh set to 0 in the same pass (rows written beside the force rows).
 template <typename T>
 cudaError_t inverse_yz_grad(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const* out, int n, int batch, double kf,
-                            cudaStream_t st, const double* kf_arr = nullptr, T* zero = nullptr);
+                            cudaStream_t st, const double* kf_arr = nullptr, T* zero = nullptr, int rows = 1);
 
 }  // namespace pm

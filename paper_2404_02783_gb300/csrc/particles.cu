@@ -59,10 +59,10 @@ __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restric
     }
 }
 
-template <int R>
+template <int R, int XC>
 __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restrict__ x, int lognp, int logn,
                                                        float inv_cell_ticks, float mass, float* __restrict__ rho) {
-    typedef DepTile<R> D;
+    typedef DepTile<R, XC> D;
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
     uint32_t* carry = tile_words + D::CELLS;
@@ -70,15 +70,18 @@ __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restric
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
     const int64_t count = (int64_t)1 << (3 * lognp);
-    tile_zero<D>(tile_words);
+    tile_zero<D::CELLS>(lo);
     __syncthreads();
     auto pid = [&](int e) -> int64_t {
         const int lz = e % D::TZ, ly = (e / D::TZ) % D::TY, lx = e / (D::TZ * D::TY);
         return ((((int64_t)(bx * D::TX + lx) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
     };
+    const float quanta = mass * kTileQuanta;
+    uint32_t sum = 0;
     // positions are loaded one iteration ahead (their latency overlaps the deposit)
     int64_t idn = pid(threadIdx.x);
-    uint32_t nu0 = x[idn], nu1 = x[count + idn], nu2 = x[2 * count + idn];
+    uint32_t nu0 = 0, nu1 = 0, nu2 = 0;
+    if (D::PER >= 512 || threadIdx.x < D::PER) nu0 = x[idn], nu1 = x[count + idn], nu2 = x[2 * count + idn];
 #pragma unroll 1
     for (int e = threadIdx.x; e < D::PER; e += 512) {
         const uint32_t u0 = nu0, u1 = nu1, u2 = nu2;
@@ -88,17 +91,23 @@ __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restric
             nu1 = x[count + idn];
             nu2 = x[2 * count + idn];
         }
-        tile_deposit<D>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, mass);
+        tile_deposit<D, false>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
     }
-    __syncthreads();
-    tile_flush<D>(lo, carry, rho, ox, oy, oz, logn);
+    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sum, [&] {
+        for (int e = threadIdx.x; e < D::PER; e += 512) {
+            const int64_t id = pid(e);
+            tile_deposit<D, true>(lo, carry, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+                                  oz, quanta, sum);
+        }
+    });
 }
 
 // R = 1: each thread walks one lattice row of the CTA's block along x and carries the upper-x
 // plane of its CIC stencil to the next particle (the deposit half of the fused update kernel).
+template <int XC>
 __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __restrict__ x, int lognp, int logn,
                                                           float inv_cell_ticks, float mass, float* __restrict__ rho) {
-    typedef DepTile<1> D;
+    typedef DepTile<1, XC> D;
     static_assert(D::TY * D::TZ == 512, "one thread per (ly, lz); lx runs over the loop");
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
@@ -108,11 +117,12 @@ __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __rest
     const int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX - D::H, oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
-    tile_zero<D>(tile_words);
+    tile_zero<D::CELLS>(lo);
     __syncthreads();
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
     const int64_t id0 = ((((int64_t)(bx * D::TX) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
     const int64_t xstride = (int64_t)1 << (2 * lognp);
+    const float quanta = mass * kTileQuanta;
     SweepCarry sc;
     uint32_t nu0 = x[id0], nu1 = x[count + id0], nu2 = x[2 * count + id0];
 #pragma unroll 1
@@ -124,11 +134,16 @@ __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __rest
             nu1 = x[count + idn];
             nu2 = x[2 * count + idn];
         }
-        sweep_deposit<D>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, mass, sc);
+        sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
-    sweep_finish<D>(lo, carry, sc);
-    __syncthreads();
-    tile_flush<D>(lo, carry, rho, ox, oy, oz, logn);
+    if (sc.dnext >= 0) sweep_carried<D>(lo, sc);
+    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sc.sum, [&] {
+        for (int lx = 0; lx < D::TX; ++lx) {
+            const int64_t id = id0 + lx * xstride;
+            tile_deposit<D, true>(lo, carry, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+                                  oz, quanta, sc.sum);
+        }
+    });
 }
 
 __global__ void k_deposit_frac(const double* __restrict__ x, int64_t count, int n, double mass,
@@ -158,23 +173,28 @@ static unsigned grid_for(int64_t count, int threads) {
     return (unsigned)b;
 }
 
-template <int R>
+template <int R, int XC>
 static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, void* rho, cudaStream_t st) {
-    typedef DepTile<R> D;
+    typedef DepTile<R, XC> D;
     const int lognp = ilog2(np), logn = ilog2(n);
     const unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
     const float inv = (float)ldexp(1.0, -(32 - logn));
     const size_t smem = sizeof(uint32_t) * D::WORDS;
-    if constexpr (R == 1) {
-        cudaError_t e = set_smem_once((const void*)k_deposit_sweep, smem);
-        if (e != cudaSuccess) return e;
-        k_deposit_sweep<<<blocks, 512, smem, st>>>((const uint32_t*)x, lognp, logn, inv, (float)mass, (float*)rho);
-        return cudaGetLastError();
-    } else {
-        cudaError_t e = set_smem_once((const void*)k_deposit_tiled<R>, smem);
-        if (e != cudaSuccess) return e;
-        k_deposit_tiled<R><<<blocks, 512, smem, st>>>((const uint32_t*)x, lognp, logn, inv, (float)mass, (float*)rho);
-        return cudaGetLastError();
+    const auto fn = [] {
+        if constexpr (R == 1) return k_deposit_sweep<XC>;
+        else return k_deposit_tiled<R, XC>;
+    }();
+    cudaError_t e = set_smem_once((const void*)fn, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<blocks, 512, smem, st>>>((const uint32_t*)x, lognp, logn, inv, (float)mass, (float*)rho);
+    return cudaGetLastError();
+}
+template <int R>
+static cudaError_t deposit_tiled(const void* x, int np, int n, double mass, void* rho, cudaStream_t st) {
+    switch (tile_depth(R, np, 1)) {
+        case 4: return deposit_tiled_r<R, 4>(x, np, n, mass, rho, st);
+        case 8: return deposit_tiled_r<R, 8>(x, np, n, mass, rho, st);
+        default: return deposit_tiled_r<R, 16>(x, np, n, mass, rho, st);
     }
 }
 
@@ -184,9 +204,9 @@ cudaError_t deposit_lattice(const void* x, int np, int precision, int n, double 
     // the tile box (16 + 4) x (16 + 4) x (32 + 8) cells must fit in the mesh without overlapping itself
     const bool tiled = precision == PM_FP32_FIXED && n >= 64 && (R == 1 || R == 2 || R == 4) && np >= 32 / R;
     if (!tiled) return deposit(x, (int64_t)np * np * np, precision, n, mass, rho, st);
-    if (R == 1) return deposit_tiled_r<1>(x, np, n, mass, rho, st);
-    if (R == 2) return deposit_tiled_r<2>(x, np, n, mass, rho, st);
-    return deposit_tiled_r<4>(x, np, n, mass, rho, st);
+    if (R == 1) return deposit_tiled<1>(x, np, n, mass, rho, st);
+    if (R == 2) return deposit_tiled<2>(x, np, n, mass, rho, st);
+    return deposit_tiled<4>(x, np, n, mass, rho, st);
 }
 
 cudaError_t deposit(const void* x, int64_t count, int precision, int n, double mass, void* rho,
@@ -204,7 +224,7 @@ cudaError_t deposit(const void* x, int64_t count, int precision, int n, double m
 }
 
 // ---------------------------------------------------------------- interpolation
-template <typename T, typename X>
+template <typename T, typename X, int ROWS = 1>
 __device__ __forceinline__ T gather8(const T* __restrict__ f, size_t n, const int* ix, const int* iy,
                                      const int* iz, const T* wx, const T* wy, const T* wz) {
     T acc = T(0);
@@ -212,7 +232,7 @@ __device__ __forceinline__ T gather8(const T* __restrict__ f, size_t n, const in
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const T* row = f + ((size_t)ix[a] * n + iy[b]) * n;
+            const T* row = f + ((size_t)ix[a] * n + iy[b]) * n * ROWS;
             acc += wx[a] * wy[b] * (wz[0] * __ldg(row + iz[0]) + wz[1] * __ldg(row + iz[1]));
         }
     return acc;
@@ -261,14 +281,13 @@ cudaError_t interp(const void* field, int n, const void* x, int64_t count, int p
 // ---------------------------------------------------------------- interp + kick + drift
 template <bool FD>
 __global__ void __launch_bounds__(256) k_ikd_ticks(uint32_t* __restrict__ x, float* __restrict__ p, int64_t count,
-                                                   int logn, float inv_cell_ticks, const float* __restrict__ gx,
-                                                   const float* __restrict__ gy, const float* __restrict__ gz,
+                                                   int logn, float inv_cell_ticks, const float* __restrict__ g,
                                                    float kick, float drift_ticks, float inv_d) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
         uint32_t u0 = x[i], u1 = x[count + i], u2 = x[2 * count + i];
         float p0 = p[i], p1 = p[count + i], p2 = p[2 * count + i];
-        ikd_particle<FD>(u0, u1, u2, p0, p1, p2, logn, inv_cell_ticks, gx, gy, gz, kick, drift_ticks, inv_d);
+        ikd_particle<FD>(u0, u1, u2, p0, p1, p2, logn, inv_cell_ticks, g, kick, drift_ticks, inv_d);
         p[i] = p0;
         p[count + i] = p1;
         p[2 * count + i] = p2;
@@ -283,8 +302,7 @@ __global__ void __launch_bounds__(256) k_ikd_ticks(uint32_t* __restrict__ x, flo
 // second particle's gathers mostly hit L1.
 template <bool FD>
 __global__ void __launch_bounds__(256) k_ikd_ticks2(uint32_t* __restrict__ x, float* __restrict__ p, int64_t count,
-                                                    int logn, float inv_cell_ticks, const float* __restrict__ gx,
-                                                    const float* __restrict__ gy, const float* __restrict__ gz,
+                                                    int logn, float inv_cell_ticks, const float* __restrict__ g,
                                                     float kick, float drift_ticks, float inv_d) {
     const int64_t pairs = count >> 1;
     uint2* x0 = reinterpret_cast<uint2*>(x);
@@ -297,8 +315,8 @@ __global__ void __launch_bounds__(256) k_ikd_ticks2(uint32_t* __restrict__ x, fl
          i += (int64_t)gridDim.x * blockDim.x) {
         uint2 a = x0[i], b = x1[i], c = x2[i];
         float2 pa = p0[i], pb = p1[i], pc = p2[i];
-        ikd_particle<FD>(a.x, b.x, c.x, pa.x, pb.x, pc.x, logn, inv_cell_ticks, gx, gy, gz, kick, drift_ticks, inv_d);
-        ikd_particle<FD>(a.y, b.y, c.y, pa.y, pb.y, pc.y, logn, inv_cell_ticks, gx, gy, gz, kick, drift_ticks, inv_d);
+        ikd_particle<FD>(a.x, b.x, c.x, pa.x, pb.x, pc.x, logn, inv_cell_ticks, g, kick, drift_ticks, inv_d);
+        ikd_particle<FD>(a.y, b.y, c.y, pa.y, pb.y, pc.y, logn, inv_cell_ticks, g, kick, drift_ticks, inv_d);
         p0[i] = pa;
         p1[i] = pb;
         p2[i] = pc;
@@ -310,8 +328,7 @@ __global__ void __launch_bounds__(256) k_ikd_ticks2(uint32_t* __restrict__ x, fl
 
 template <bool FD>
 __global__ void __launch_bounds__(256) k_ikd_frac(double* __restrict__ x, double* __restrict__ p, int64_t count,
-                                                  int n, const double* __restrict__ gx, const double* __restrict__ gy,
-                                                  const double* __restrict__ gz, double kick, double drift_box,
+                                                  int n, const double* __restrict__ g, double kick, double drift_box,
                                                   double inv_d) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -327,12 +344,12 @@ __global__ void __launch_bounds__(256) k_ikd_frac(double* __restrict__ x, double
 #pragma unroll
                 for (int b = 0; b < 2; ++b)
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) P[a][2 * b + c] = gx[((size_t)ix[a] * n + iy[b]) * n + iz[c]];
+                    for (int c = 0; c < 2; ++c) P[a][2 * b + c] = g[((size_t)ix[a] * n + iy[b]) * n + iz[c]];
             fd1_force<double>(P[0], P[1], wx[0], wx[1], wy, wz, inv_d, f[0], f[1], f[2]);
         } else {
-            f[0] = gather8<double, double>(gx, (size_t)n, ix, iy, iz, wx, wy, wz);
-            f[1] = gather8<double, double>(gy, (size_t)n, ix, iy, iz, wx, wy, wz);
-            f[2] = gather8<double, double>(gz, (size_t)n, ix, iy, iz, wx, wy, wz);
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                f[j] = gather8<double, double, kForceRows>(g + j * n, (size_t)n, ix, iy, iz, wx, wy, wz);
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
@@ -346,7 +363,7 @@ __global__ void __launch_bounds__(256) k_ikd_frac(double* __restrict__ x, double
 }
 
 template <bool FD>
-static cudaError_t interp_kick_drift_t(void* x, void* p, int64_t count, int precision, int n, void* const* g,
+static cudaError_t interp_kick_drift_t(void* x, void* p, int64_t count, int precision, int n, const void* g,
                                        double kick, double drift, double box, double inv_d, cudaStream_t st) {
     const int logn = ilog2(n);
     if (precision == PM_FP32_FIXED) {
@@ -355,22 +372,19 @@ static cudaError_t interp_kick_drift_t(void* x, void* p, int64_t count, int prec
         const bool pairs = (count % 2 == 0) && ((uintptr_t)x % 8 == 0) && ((uintptr_t)p % 8 == 0);
         if (pairs)
             k_ikd_ticks2<FD><<<grid_for(count / 2, 256), 256, 0, st>>>((uint32_t*)x, (float*)p, count, logn, inv,
-                                                                       (const float*)g[0], (const float*)g[1],
-                                                                       (const float*)g[2], (float)kick, dt,
+                                                                       (const float*)g, (float)kick, dt,
                                                                        (float)inv_d);
         else
             k_ikd_ticks<FD><<<grid_for(count, 256), 256, 0, st>>>((uint32_t*)x, (float*)p, count, logn, inv,
-                                                                  (const float*)g[0], (const float*)g[1],
-                                                                  (const float*)g[2], (float)kick, dt, (float)inv_d);
+                                                                  (const float*)g, (float)kick, dt, (float)inv_d);
     } else {
-        k_ikd_frac<FD><<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, count, n, (const double*)g[0],
-                                                             (const double*)g[1], (const double*)g[2], kick,
+        k_ikd_frac<FD><<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, count, n, (const double*)g, kick,
                                                              drift / box, inv_d);
     }
     return cudaGetLastError();
 }
 
-cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, int n, void* const* g,
+cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, int n, const void* g,
                               double kick, double drift, double box, cudaStream_t st, double fd_inv_d) {
     if (count == 0) return cudaSuccess;
     if (fd_inv_d > 0.0) return interp_kick_drift_t<true>(x, p, count, precision, n, g, kick, drift, box, fd_inv_d, st);

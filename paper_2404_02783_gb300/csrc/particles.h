@@ -14,17 +14,19 @@ cudaError_t deposit(const void* x, int64_t count, int precision, int n, double m
 cudaError_t deposit_lattice(const void* x, int np, int precision, int n, double mass, void* rho, cudaStream_t st);
 cudaError_t interp(const void* field, int n, const void* x, int64_t count, int precision, void* out,
                    cudaStream_t st);
-// g: three force meshes; kick = K(a, b); drift = D(a, b) in Mpc/h per unit p
-// fd_inv_d > 0: first-order gradient (g[0] is the potential, g[1], g[2] unused), inv_d = n / L.
-cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, int n, void* const* g, double kick,
+// g: the three force meshes (layout kForceRows); kick = K(a, b); drift = D(a, b) in Mpc/h per unit p
+// fd_inv_d > 0: first-order gradient (g is the potential, a plain mesh), inv_d = n / L.
+cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, int n, const void* g, double kick,
                               double drift, double box, cudaStream_t st, double fd_inv_d = 0.0);
+// x extent in mesh cells (16, 8 or 4) of the Lagrangian deposit tiles of nfields lattices.
+int tile_depth(int R, int np, int nfields);
 // Kick + drift of the np^3 lattice-ordered particles fused with the deposit of the
 // drifted positions into rho (which must be zero on entry); FP32 ticks, n / np in {1,2,4}.
 bool ikd_deposit_supported(int np, int precision, int n);
 // nfields > 1: a batch of runs stored back to back, box given per field as
 // scale_arr[f] = 2^32 / L_f (box is then ignored).  x_out: where the drifted positions go
 // (null: back into x); p is always updated in place.
-cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, int n, void* const* g, double kick,
+cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, int n, const void* g, double kick,
                                       double drift, double box, double mass, void* rho, cudaStream_t st,
                                       int nfields = 1, const double* scale_arr = nullptr, void* x_out = nullptr,
                                       double fd_inv_d = 0.0);
@@ -66,10 +68,8 @@ size_t halo_proxy_scratch_bytes(int64_t count);
 // Reverse sweep of the FP32 step (adjoint.cu).
 cudaError_t adj_gather(const uint32_t* x, int64_t count, int n, const float* F, float scale, int accumulate,
                        float* lam_u, cudaStream_t st);
-cudaError_t adj_direct(const uint32_t* x, int64_t count, int n, const float* v, const float* const* G, float K,
-                       float* lam_u, cudaStream_t st);
-// lam_u += K sum_j v_j grad interp(G_j) + Km grad interp(rho_bar); then v += drift_next lam_u.
-cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v, const float* const* G,
+// lam_u += K sum_j v_j grad interp(G_j) (G: layout kForceRows) + Km grad interp(rho_bar); then v += drift_next lam_u.
+cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v, const float* G,
                                const float* rho_bar, float K, float Km, float drift_next, float* lam_u,
                                cudaStream_t st);
 // First-order gradient: V += -sum_j v_j dW/dx_j (inv_d = n / L; V zeroed by the caller), and the

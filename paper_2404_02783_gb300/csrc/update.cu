@@ -14,47 +14,51 @@ namespace pm {
 // density mesh through the tile's shared-memory accumulator, exactly as
 // k_deposit_tiled would have done from the drifted positions.
 // blockIdx.y selects the field of a batch of independent runs stored back to back
-// (particles [field][3][np^3], meshes [field][n^3]); scale = 2^32 / L of that field.
-template <int R, bool FD>
-__global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo, float* __restrict__ p, int lognp,
-                                                     int logn, float inv_cell_ticks, const float* __restrict__ gx,
-                                                     const float* __restrict__ gy, const float* __restrict__ gz,
-                                                     float kick, double drift, double scale0,
-                                                     const double* __restrict__ scale_arr, float mass,
-                                                     float* __restrict__ rho, float inv_d) {
-    typedef DepTile<R> D;
+// (particles [field][3][np^3], force meshes [field][n][n][3][n], density [field][n^3]); scale =
+// 2^32 / L of that field.  The mesh side 2^LOGN is a compile-time constant: the kernels are
+// bound by issue, and its shifts, masks and row strides are then immediates.
+template <int R, int XC, int LOGN, bool FD>
+__global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
+                                                        float* __restrict__ p, const float* __restrict__ g, float kick,
+                                                        double drift, double scale0,
+                                                        const double* __restrict__ scale_arr, float mass,
+                                                        float* __restrict__ rho, float inv_d) {
+    typedef DepTile<R, XC> D;
+    constexpr int logn = LOGN, lognp = LOGN - (R == 4 ? 2 : R == 2 ? 1 : 0), np = 1 << lognp;
+    constexpr int64_t count = (int64_t)1 << (3 * lognp);
+    constexpr float inv_cell_ticks = 1.0f / (float)(1u << (32 - LOGN));
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
     uint32_t* carry = tile_words + D::CELLS;
-    const int np = 1 << lognp;
-    const int64_t count = (int64_t)1 << (3 * lognp);
     {
         const int64_t fb = blockIdx.y;
-        const int64_t n3 = (int64_t)1 << (3 * logn);
+        constexpr int64_t n3 = (int64_t)1 << (3 * LOGN);
         x += fb * 3 * count;
         xo += fb * 3 * count;
         p += fb * 3 * count;
-        gx += fb * n3;
-        if (!FD) {
-            gy += fb * n3;
-            gz += fb * n3;
-        }
+        g += fb * (FD ? 1 : kForceRows) * n3;
         rho += fb * n3;
     }
     const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
-    const int ntz = np / D::TZ, nty = np / D::TY;
+    constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
-    tile_zero<D>(tile_words);
+    tile_zero<D::CELLS>(lo);
     __syncthreads();
     auto pid = [&](int e) -> int64_t {
         const int lz = e % D::TZ, ly = (e / D::TZ) % D::TY, lx = e / (D::TZ * D::TY);
         return ((((int64_t)(bx * D::TX + lx) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
     };
+    const float quanta = mass * kTileQuanta;
+    uint32_t sum = 0;
     // the next particle is loaded one iteration ahead (its latency overlaps this one's work)
     int64_t idn = pid(threadIdx.x);
-    uint32_t nu0 = x[idn], nu1 = x[count + idn], nu2 = x[2 * count + idn];
-    float np0 = p[idn], np1 = p[count + idn], np2 = p[2 * count + idn];
+    uint32_t nu0 = 0, nu1 = 0, nu2 = 0;
+    float np0 = 0.f, np1 = 0.f, np2 = 0.f;
+    if (D::PER >= 512 || threadIdx.x < D::PER) {
+        nu0 = x[idn], nu1 = x[count + idn], nu2 = x[2 * count + idn];
+        np0 = p[idn], np1 = p[count + idn], np2 = p[2 * count + idn];
+    }
 #pragma unroll 1
     for (int e = threadIdx.x; e < D::PER; e += 512) {
         const int64_t id = idn;
@@ -69,67 +73,72 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restri
             np1 = p[count + idn];
             np2 = p[2 * count + idn];
         }
-        ikd_particle<FD>(u0, u1, u2, p0, p1, p2, logn, inv_cell_ticks, gx, gy, gz, kick, drift_ticks, inv_d);
+        ikd_particle<FD>(u0, u1, u2, p0, p1, p2, logn, inv_cell_ticks, g, kick, drift_ticks, inv_d);
         p[id] = p0;
         p[count + id] = p1;
         p[2 * count + id] = p2;
         xo[id] = u0;
         xo[count + id] = u1;
         xo[2 * count + id] = u2;
-        tile_deposit<D>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, mass);
+        tile_deposit<D, false>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
     }
-    __syncthreads();
-    tile_flush<D>(lo, carry, rho, ox, oy, oz, logn);
+    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sum, [&] {
+        for (int e = threadIdx.x; e < D::PER; e += 512) {
+            const int64_t id = pid(e);
+            tile_deposit<D, true>(lo, carry, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
+                                  oy, oz, quanta, sum);
+        }
+    });
 }
 
 // x and xo may be the same array (in-place update): every particle's position is read once,
 // one iteration before its own thread writes it, and no thread touches another's particles.
-// R = 1: each thread walks its lattice row along x (lx = 0..15 at fixed ly, lz), so the
+// R = 1: each thread walks its lattice row along x (lx = 0..XC-1 at fixed ly, lz), so the
 // next particle usually sits one cell further in x with the same y and z cells.  Then
 // its lower-x CIC corners are this particle's upper-x corners: the gather keeps the 12
 // upper-plane force values in registers and loads only the new plane, and the deposit
 // carries the upper-plane weights in registers, adds them to the next particle's
 // lower-plane weights and issues 4 tile atomics a particle instead of 8.  Any other
 // particle takes the full path, so the result is the same CIC gather and deposit.
-template <bool FD>
-__global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo, float* __restrict__ p,
-                                                              int lognp, int logn, float inv_cell_ticks,
-                                                              const float* __restrict__ gx,
-                                                              const float* __restrict__ gy,
-                                                              const float* __restrict__ gz, float kick, double drift,
-                                                              double scale0, const double* __restrict__ scale_arr,
-                                                              float mass, float* __restrict__ rho, float inv_d) {
-    typedef DepTile<1> D;
+// Bound by issue (about 70% busy) and by the latency of the gather: the upper plane's loads, which
+// every particle needs, are issued before the branch that reloads the lower plane (512^3, early
+// and clustered steps: 1742 and 1953 us; after it 1826 and 2020).  Holding the gather in flight
+// across the previous particle's deposit spills at two 512-thread CTAs an SM (2293 us) and gains
+// nothing at three 256-thread CTAs (1798 and 1958).
+template <int XC, int LOGN, bool FD>
+__global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
+                                                              float* __restrict__ p, const float* __restrict__ g,
+                                                              float kick, double drift, double scale0,
+                                                              const double* __restrict__ scale_arr, float mass,
+                                                              float* __restrict__ rho, float inv_d) {
+    typedef DepTile<1, XC> D;
     static_assert(D::TY * D::TZ == 512, "one thread per (ly, lz); lx runs over the loop");
+    constexpr int logn = LOGN, np = 1 << LOGN, NC = FD ? 1 : 3, ROWS = FD ? 1 : kForceRows;
+    constexpr int64_t count = (int64_t)1 << (3 * LOGN);
+    constexpr float inv_cell_ticks = 1.0f / (float)(1u << (32 - LOGN));
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
     uint32_t* carry = tile_words + D::CELLS;
-    const int np = 1 << lognp, nm = (1 << logn) - 1;
-    const int64_t count = (int64_t)1 << (3 * lognp);
     {
         const int64_t fb = blockIdx.y;
-        const int64_t n3 = (int64_t)1 << (3 * logn);
         x += fb * 3 * count;
         xo += fb * 3 * count;
         p += fb * 3 * count;
-        gx += fb * n3;
-        if (!FD) {
-            gy += fb * n3;
-            gz += fb * n3;
-        }
-        rho += fb * n3;
+        g += fb * ROWS * count;
+        rho += fb * count;
     }
     const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
-    const int ntz = np / D::TZ, nty = np / D::TY;
+    constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX - D::H, oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
-    tile_zero<D>(tile_words);
+    tile_zero<D::CELLS>(lo);
     __syncthreads();
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
-    const int64_t id0 = ((((int64_t)(bx * D::TX) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
-    const int64_t xstride = (int64_t)1 << (2 * lognp);
+    const int64_t id0 = ((((int64_t)(bx * D::TX) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
+    constexpr int64_t xstride = (int64_t)1 << (2 * LOGN);
     uint32_t next_cell = 0xffffffffu;  // packed (ix, iy, iz) whose lower plane the registers hold
-    float U[4][FD ? 1 : 3];             // force (FD: potential) at the carried plane, corner (b, c) = 2 b + c
+    float U[4][NC];                     // force (FD: potential) at the carried plane, corner (b, c) = 2 b + c
+    const float quanta = mass * kTileQuanta;
     SweepCarry sc;                      // deposit weights carried to the next particle's plane
     // the next particle's position and momentum are loaded one iteration ahead, so their
     // memory latency overlaps the current particle's gather, update and deposit
@@ -154,35 +163,26 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
             const CicF cx = cic_ticks(u0, logn, inv_cell_ticks);
             const CicF cy = cic_ticks(u1, logn, inv_cell_ticks);
             const CicF cz = cic_ticks(u2, logn, inv_cell_ticks);
-            const uint32_t cell = ((((uint32_t)cx.i0 << logn) | (uint32_t)cy.i0) << logn) | (uint32_t)cz.i0;
-            const uint32_t iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1}, iz[2] = {(uint32_t)cz.i0, (uint32_t)cz.i1};
-            constexpr int NC = FD ? 1 : 3;
-            const float* g3[3] = {gx, gy, gz};
+            const uint32_t yz = ((uint32_t)cy.i0 << LOGN) | (uint32_t)cz.i0;
             float L[4][NC];
-            if (cell == next_cell) {
+            const bool same = (((uint32_t)cx.i0 << (2 * LOGN)) | yz) == next_cell;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < NC; ++j) L[q][j] = U[q][j];
+            const PlaneCorners<ROWS> ku(cx.i1, cy, cz, logn);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < NC; ++j) U[q][j] = __ldg(g + ku[q] + j * np);
+            if (!same) {
+                const PlaneCorners<ROWS> k(cx.i0, cy, cz, logn);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
-                    for (int j = 0; j < NC; ++j) L[q][j] = U[q][j];
-            } else {
-#pragma unroll
-                for (int b = 0; b < 2; ++b)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const uint32_t o = ((((uint32_t)cx.i0 << logn) + iy[b]) << logn) + iz[c];
-#pragma unroll
-                        for (int j = 0; j < NC; ++j) L[2 * b + c][j] = __ldg(g3[j] + o);
-                    }
+                    for (int j = 0; j < NC; ++j) L[q][j] = __ldg(g + k[q] + j * np);
             }
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const uint32_t o = ((((uint32_t)cx.i1 << logn) + iy[b]) << logn) + iz[c];
-#pragma unroll
-                    for (int j = 0; j < NC; ++j) U[2 * b + c][j] = __ldg(g3[j] + o);
-                }
-            next_cell = ((((uint32_t)cx.i1 << logn) | (uint32_t)cy.i0) << logn) | (uint32_t)cz.i0;
+            next_cell = ((uint32_t)cx.i1 << (2 * LOGN)) | yz;
             const float wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};
             const float wx0 = 1.0f - cx.w1, wx1 = cx.w1;
             float f0 = 0.f, f1 = 0.f, f2 = 0.f;
@@ -216,38 +216,89 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
         xo[count + id] = u1;
         xo[2 * count + id] = u2;
         // ---- deposit at the new position
-        sweep_deposit<D>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, mass, sc);
+        sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
-    sweep_finish<D>(lo, carry, sc);
-    __syncthreads();
-    tile_flush<D>(lo, carry, rho, ox, oy, oz, logn);
+    if (sc.dnext >= 0) sweep_carried<D>(lo, sc);  // the carried plane of the row's last particle
+    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sc.sum, [&] {
+        for (int lx = 0; lx < D::TX; ++lx) {
+            const int64_t id = id0 + lx * xstride;
+            tile_deposit<D, true>(lo, carry, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
+                                  oy, oz, quanta, sc.sum);
+        }
+    });
 }
 
-template <int R, bool FD>
-static cudaError_t ikd_deposit_r(void* x, void* p, int np, int n, void* const* g, double kick, double drift,
-                                 double box, double mass, void* rho, cudaStream_t st, int nfields,
-                                 const double* scale_arr, void* x_out, double inv_d) {
-    typedef DepTile<R> D;
-    const int lognp = ilog2(np), logn = ilog2(n);
-    const unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
-    const float inv = (float)ldexp(1.0, -(32 - logn));
+namespace {
+
+struct UpdateArgs {
+    void* x;
+    void* xo;
+    void* p;
+    const void* g;
+    double kick, drift, scale0;
+    const double* scale_arr;
+    double mass;
+    void* rho;
+    double inv_d;
+    int nfields;
+    cudaStream_t st;
+};
+
+template <int R, int XC, int LOGN, bool FD>
+cudaError_t ikd_launch(const UpdateArgs& a) {
+    typedef DepTile<R, XC> D;
+    constexpr int np = (1 << LOGN) / R;
+    constexpr unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
     const size_t smem = sizeof(uint32_t) * D::WORDS;
-    if constexpr (R == 1) {
-        cudaError_t e = set_smem_once((const void*)k_ikd_deposit_sweep<FD>, smem);
-        if (e != cudaSuccess) return e;
-        k_ikd_deposit_sweep<FD><<<dim3(blocks, nfields), 512, smem, st>>>(
-            (const uint32_t*)x, (uint32_t*)(x_out ? x_out : x), (float*)p, lognp, logn, inv, (const float*)g[0],
-            (const float*)g[1], (const float*)g[2],
-            (float)kick, drift, 4294967296.0 / box, scale_arr, (float)mass, (float*)rho, (float)inv_d);
-    } else {
-        cudaError_t e = set_smem_once((const void*)k_ikd_deposit<R, FD>, smem);
-        if (e != cudaSuccess) return e;
-        k_ikd_deposit<R, FD><<<dim3(blocks, nfields), 512, smem, st>>>(
-            (const uint32_t*)x, (uint32_t*)(x_out ? x_out : x), (float*)p, lognp, logn, inv, (const float*)g[0],
-            (const float*)g[1], (const float*)g[2],
-            (float)kick, drift, 4294967296.0 / box, scale_arr, (float)mass, (float*)rho, (float)inv_d);
-    }
+    const auto fn = [] {
+        if constexpr (R == 1) return k_ikd_deposit_sweep<XC, LOGN, FD>;
+        else return k_ikd_deposit<R, XC, LOGN, FD>;
+    }();
+    cudaError_t e = set_smem_once((const void*)fn, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<dim3(blocks, a.nfields), 512, smem, a.st>>>((const uint32_t*)a.x, (uint32_t*)a.xo, (float*)a.p,
+                                                     (const float*)a.g, (float)a.kick, a.drift, a.scale0, a.scale_arr,
+                                                     (float)a.mass, (float*)a.rho, (float)a.inv_d);
     return cudaGetLastError();
+}
+
+// Meshes of 128^3 and up always fill the SMs with tiles of depth 16.
+template <int R, bool FD>
+cudaError_t ikd_sized(int n, int np, const UpdateArgs& a) {
+    switch (n) {
+        case 64:
+            switch (tile_depth(R, np, a.nfields)) {
+                case 4: return ikd_launch<R, 4, 6, FD>(a);
+                case 8: return ikd_launch<R, 8, 6, FD>(a);
+                default: return ikd_launch<R, 16, 6, FD>(a);
+            }
+        case 128: return ikd_launch<R, 16, 7, FD>(a);
+        case 256: return ikd_launch<R, 16, 8, FD>(a);
+        case 512: return ikd_launch<R, 16, 9, FD>(a);
+        case 1024: return ikd_launch<R, 16, 10, FD>(a);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <bool FD>
+cudaError_t ikd_any(int n, int np, const UpdateArgs& a) {
+    switch (n / np) {
+        case 1: return ikd_sized<1, FD>(n, np, a);
+        case 2: return ikd_sized<2, FD>(n, np, a);
+        case 4: return ikd_sized<4, FD>(n, np, a);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+// A tile of XC cells in x brings 4 of its own in halo cells, so the deepest tile is used that
+// still gives every SM one: 64^3 particles on 64^3 cells are 32 tiles of depth 16 and the update
+// takes 25.4 us, 15.5 at depth 8, 11.9 at depth 4; from 152 tiles on depth 16 is as good or
+// better (64^3 on 128^3, 256 tiles: 15.0 us against 16.1 and 18.5; 256^3: 237, 247, 269 us).
+int tile_depth(int R, int np, int nfields) {
+    const int64_t tiles = (int64_t)nfields * (np * R / 16) * (np * R / 16) * (np * R / 32);  // of depth 16
+    return tiles >= num_sms() ? 16 : 2 * tiles >= num_sms() ? 8 : 4;
 }
 
 bool ikd_deposit_supported(int np, int precision, int n) {
@@ -255,27 +306,15 @@ bool ikd_deposit_supported(int np, int precision, int n) {
     return precision == PM_FP32_FIXED && n >= 64 && (R == 1 || R == 2 || R == 4) && np >= 32 / R;
 }
 
-template <bool FD>
-static cudaError_t ikd_deposit_any(void* x, void* p, int np, int n, void* const* g, double kick, double drift,
-                                   double box, double mass, void* rho, cudaStream_t st, int nfields,
-                                   const double* scale_arr, void* x_out, double inv_d) {
-    const int R = n / np;
-    if (R == 1)
-        return ikd_deposit_r<1, FD>(x, p, np, n, g, kick, drift, box, mass, rho, st, nfields, scale_arr, x_out, inv_d);
-    if (R == 2)
-        return ikd_deposit_r<2, FD>(x, p, np, n, g, kick, drift, box, mass, rho, st, nfields, scale_arr, x_out, inv_d);
-    return ikd_deposit_r<4, FD>(x, p, np, n, g, kick, drift, box, mass, rho, st, nfields, scale_arr, x_out, inv_d);
-}
-
-cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, int n, void* const* g, double kick,
+cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, int n, const void* g, double kick,
                                       double drift, double box, double mass, void* rho, cudaStream_t st, int nfields,
                                       const double* scale_arr, void* x_out, double fd_inv_d) {
     if (!ikd_deposit_supported(np, precision, n) || nfields < 1 || (uintptr_t)rho % 16 != 0)
         return cudaErrorInvalidValue;
-    if (fd_inv_d > 0.0)
-        return ikd_deposit_any<true>(x, p, np, n, g, kick, drift, box, mass, rho, st, nfields, scale_arr, x_out,
-                                     fd_inv_d);
-    return ikd_deposit_any<false>(x, p, np, n, g, kick, drift, box, mass, rho, st, nfields, scale_arr, x_out, 0.0);
+    const bool fd = fd_inv_d > 0.0;
+    const UpdateArgs a{x, x_out ? x_out : x, p, g, kick, drift, 4294967296.0 / box, scale_arr, mass, rho,
+                       fd ? fd_inv_d : 0.0, nfields, st};
+    return fd ? ikd_any<true>(n, np, a) : ikd_any<false>(n, np, a);
 }
 
 }  // namespace pm

@@ -5,6 +5,7 @@
 
 #include <stdint.h>
 
+#include "internal.h"
 #include "pm_common.cuh"
 
 namespace pm {
@@ -24,32 +25,39 @@ __device__ __forceinline__ CicF cic_ticks(uint32_t u, int logn, float inv_cell_t
     return c;
 }
 // Deposit of lattice-ordered particles (count = np^3, id = (ix np + iy) np + iz) by
-// Lagrangian tiles.  A CTA owns a TX x TY x TZ block of lattice sites (16 x 16 x 32
-// mesh cells' worth, R = n / np cells per lattice step); particles that have not
-// travelled far land in that mesh box widened by H cells on every side, which the CTA
-// accumulates in shared memory and then adds to the global mesh once per cell.  A
-// particle whose CIC stencil leaves the box adds its weights to global memory directly,
-// so the result is the same CIC density for any displacement.
+// Lagrangian tiles.  A CTA owns a TX x TY x TZ block of lattice sites (XC x 16 x 32 mesh
+// cells' worth, R = n / np cells per lattice step); particles that have not travelled far land
+// in that mesh box widened by H cells on every side, which the CTA accumulates in shared memory
+// and then adds to the global mesh once per cell.  A particle whose CIC stencil leaves the box
+// adds its weights to global memory directly, so the result is the same CIC density for any
+// displacement.  XC is 16, or less where 16 would leave SMs without a tile (tile_depth).
 //
 // The tile accumulates in fixed point: each weight is rounded to a multiple of 2^-24
 // (half a quantum at most, 3e-8, below the FP32 rounding of a sum near 1) and added
 // with a native 32-bit integer atomic (shared-memory float atomics are a compare-and-
-// swap loop on this part).  A wrap of the 32-bit word is seen in the atomic's return
-// value and counted in an 8-bit carry per cell.  A tile holds at most 8192 mass units
-// (TX TY TZ R^3 = 8192 for every R), i.e. 2^37 quanta, so a cell's carry stays below 32
-// and the tile sum is exact and independent of the order of the additions.
+// swap loop on this part), so the tile sum is exact and independent of the order of the
+// additions as long as no cell reaches 256 mass units.  The additions return nothing and test
+// nothing; instead the sum of all cells is compared with the sum of all additions, both in 64
+// bits, before the tile is flushed: each wrap of a 32-bit cell takes exactly 2^32 from the
+// former.  A tile that fails the comparison (a cell of 256 times the mean density) is
+// accumulated again from the positions just written, with an 8-bit carry per cell caught from
+// the atomics' return values (a tile holds at most 8192 mass units, i.e. 2^37 quanta, so a
+// carry stays below 32).
 // The box starts HZ = 4 cells below the tile in z so that its rows are made of 16-byte
 // chunks aligned in the mesh: the flush adds four cells per vector reduction.
-template <int R>
+template <int R, int XC = 16>
 struct DepTile {
-    static constexpr int TX = 16 / R, TY = 16 / R, TZ = 32 / R, H = 2, HZ = 4;
+    static constexpr int THREADS = 512;
+    static constexpr int TX = XC / R, TY = 16 / R, TZ = 32 / R, H = 2, HZ = 4;
     static constexpr int DX = TX * R + 2 * H, DY = TY * R + 2 * H, DZ = TZ * R + 2 * HZ;
-    static constexpr int CELLS = DX * DY * DZ, CHUNKS = CELLS / 4;
-    static constexpr int CARRY_WORDS = CHUNKS;  // one word of four 8-bit carries per chunk
+    static constexpr int CELLS = DX * DY * DZ, CZ = DZ / 4, PLANE = DY * CZ;  // 16-byte chunks a row, an x plane
+    static constexpr int CARRY_WORDS = CELLS / 4;      // one word of four 8-bit carries per chunk
     static constexpr int WORDS = CELLS + CARRY_WORDS;  // shared memory: lo[CELLS], carry[CARRY_WORDS]
     static constexpr int PER = TX * TY * TZ;
-    static_assert(PER * R * R * R == 8192, "tile mass bound");
+    static constexpr int PLANES = THREADS / PLANE;     // x planes a pass over the chunks takes at once
+    static_assert(TX >= 1 && PER * R * R * R <= 8192, "tile mass bound");
     static_assert(DZ % 4 == 0 && (TZ * R) % 4 == 0 && HZ % 4 == 0, "z box made of aligned 16-byte chunks");
+    static_assert(CELLS % 4 == 0 && CARRY_WORDS % 4 == 0 && PLANES >= 1, "whole vectors");
 };
 
 __device__ __forceinline__ void red_add_v4(float* dst, float4 v) {
@@ -61,22 +69,31 @@ __device__ __forceinline__ void red_add_v4(float* dst, float4 v) {
 constexpr float kTileQuanta = 16777216.0f;  // 2^24 quanta per unit mass
 constexpr float kTileQuantum = 5.9604644775390625e-08f;  // 2^-24
 
-__device__ __forceinline__ void tile_add(uint32_t* lo, uint32_t* carry, int c, float w) {
-    const uint32_t v = __float2uint_rn(w * kTileQuanta);
+// Adds w quanta to a cell and to the thread's sum of additions (at most 16 mass units, 2^28).
+__device__ __forceinline__ void tile_add(uint32_t* lo, int c, float w, uint32_t& sum) {
+    const uint32_t v = __float2uint_rn(w);
+    atomicAdd(lo + c, v);
+    sum += v;
+}
+__device__ __forceinline__ void tile_add_carry(uint32_t* lo, uint32_t* carry, int c, float w) {
+    const uint32_t v = __float2uint_rn(w);
     const uint32_t old = atomicAdd(lo + c, v);
     if (old + v < old) atomicAdd(carry + (c >> 2), 1u << (8 * (c & 3)));
 }
 
-template <class D>
+template <int WORDS>
 __device__ __forceinline__ void tile_zero(uint32_t* words) {
-    for (int c = threadIdx.x; c < D::WORDS; c += blockDim.x) words[c] = 0u;
+    for (int c = threadIdx.x; c < WORDS / 4; c += blockDim.x)
+        reinterpret_cast<uint4*>(words)[c] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// One particle's CIC weights into the tile (box origin o*) or, outside it, into rho.
-template <class D>
+// One particle's CIC weights into the tile (box origin o*) or, outside it, into rho.  quanta =
+// mass 2^24 (a power of two times the mass: the weights are the same numbers, scaled).
+// CARRY: the second accumulation of a tile, of the particles inside the box alone.
+template <class D, bool CARRY>
 __device__ __forceinline__ void tile_deposit(uint32_t* lo, uint32_t* carry, float* __restrict__ rho, uint32_t u0,
                                              uint32_t u1, uint32_t u2, int logn, float inv_cell_ticks, int ox,
-                                             int oy, int oz, float mass) {
+                                             int oy, int oz, float quanta, uint32_t& sum) {
     const int nm = (1 << logn) - 1;
     const CicF cx = cic_ticks(u0, logn, inv_cell_ticks);
     const CicF cy = cic_ticks(u1, logn, inv_cell_ticks);
@@ -89,18 +106,23 @@ __device__ __forceinline__ void tile_deposit(uint32_t* lo, uint32_t* carry, floa
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const float wab = mass * wx[a] * wy[b];
+                const float wab = quanta * wx[a] * wy[b];
                 const int c = c0 + (a * D::DY + b) * D::DZ;
-                tile_add(lo, carry, c, wab * wz[0]);
-                tile_add(lo, carry, c + 1, wab * wz[1]);
+                if (CARRY) {
+                    tile_add_carry(lo, carry, c, wab * wz[0]);
+                    tile_add_carry(lo, carry, c + 1, wab * wz[1]);
+                } else {
+                    tile_add(lo, c, wab * wz[0], sum);
+                    tile_add(lo, c + 1, wab * wz[1], sum);
+                }
             }
-    } else {
+    } else if (!CARRY) {
         const uint32_t ix[2] = {(uint32_t)cx.i0, (uint32_t)cx.i1}, iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const float wab = mass * wx[a] * wy[b];
+                const float wab = quanta * kTileQuantum * wx[a] * wy[b];
                 float* row = rho + (((ix[a] << logn) + iy[b]) << logn);
                 atomicAdd(row + cz.i0, wab * wz[0]);
                 atomicAdd(row + cz.i1, wab * wz[1]);
@@ -108,26 +130,72 @@ __device__ __forceinline__ void tile_deposit(uint32_t* lo, uint32_t* carry, floa
     }
 }
 
+// f(chunk, lx, ly, lz4) for every 16-byte chunk of the tile: a thread keeps its place in the x
+// plane and walks the planes, so nothing is divided per chunk.
+template <class D, class F>
+__device__ __forceinline__ void for_chunks(F f) {
+    const int lz4 = threadIdx.x % D::CZ, ly = (threadIdx.x / D::CZ) % D::DY, l0 = threadIdx.x / D::PLANE;
+    if (l0 >= D::PLANES) return;
+#pragma unroll 2
+    for (int lx = l0; lx < D::DX; lx += D::PLANES) f((lx * D::DY + ly) * D::CZ + lz4, lx, ly, lz4);
+}
+
 // Adds the tile's cells (box origin o*, oz a multiple of 4, rho 16-byte aligned) to rho,
 // four z-cells per reduction.
-template <class D>
+template <class D, bool CARRY>
 __device__ __forceinline__ void tile_flush(const uint32_t* lo, const uint32_t* carry, float* __restrict__ rho, int ox,
                                            int oy, int oz, int logn) {
     const int nm = (1 << logn) - 1;
-    for (int c = threadIdx.x; c < D::CHUNKS; c += blockDim.x) {
+    for_chunks<D>([&](int c, int lx, int ly, int lz4) {
         const uint4 l = reinterpret_cast<const uint4*>(lo)[c];
-        const uint32_t h = carry[c];
+        const uint32_t h = CARRY ? carry[c] : 0u;
         if (l.x | l.y | l.z | l.w | h) {
-            const int lz4 = c % (D::DZ / 4), ly = (c / (D::DZ / 4)) % D::DY, lx = c / ((D::DZ / 4) * D::DY);
-            const float4 v = make_float4(__uint2float_rn(l.x) * kTileQuantum + (float)(h & 255u) * 256.0f,
-                                         __uint2float_rn(l.y) * kTileQuantum + (float)((h >> 8) & 255u) * 256.0f,
-                                         __uint2float_rn(l.z) * kTileQuantum + (float)((h >> 16) & 255u) * 256.0f,
-                                         __uint2float_rn(l.w) * kTileQuantum + (float)(h >> 24) * 256.0f);
+            float4 v = make_float4(__uint2float_rn(l.x) * kTileQuantum, __uint2float_rn(l.y) * kTileQuantum,
+                                   __uint2float_rn(l.z) * kTileQuantum, __uint2float_rn(l.w) * kTileQuantum);
+            if (CARRY) {
+                v.x += (float)(h & 255u) * 256.0f;
+                v.y += (float)((h >> 8) & 255u) * 256.0f;
+                v.z += (float)((h >> 16) & 255u) * 256.0f;
+                v.w += (float)(h >> 24) * 256.0f;
+            }
             red_add_v4(rho + ((((uint32_t)((ox + lx) & nm) << logn) + (uint32_t)((oy + ly) & nm)) << logn) +
                            ((oz + 4 * lz4) & nm),
                        v);
         }
+    });
+}
+
+// Ends a tile: compares the sum of its cells with the sum of all additions (`sum` of every
+// thread) and flushes it, after accumulating it again with carries when they differ (redo()
+// deposits the thread's particles from their written positions with CARRY).  Every thread of
+// the CTA calls it.
+template <class D, class F>
+__device__ __forceinline__ void tile_close(uint32_t* lo, uint32_t* carry, float* __restrict__ rho, int ox, int oy,
+                                           int oz, int logn, uint32_t sum, F redo) {
+    __shared__ unsigned long long missing;
+    if (threadIdx.x == 0) missing = 0;
+    __syncthreads();
+    unsigned long long d = sum;
+    for_chunks<D>([&](int c, int, int, int) {
+        const uint4 l = reinterpret_cast<const uint4*>(lo)[c];
+        d -= (unsigned long long)l.x + l.y + l.z + l.w;
+    });
+    // the warp's sum of d modulo 2^64 in three limbs
+    const uint32_t l0 = __reduce_add_sync(0xffffffffu, (uint32_t)d & 0xffffu);
+    const uint32_t l1 = __reduce_add_sync(0xffffffffu, (uint32_t)d >> 16);
+    const uint32_t l2 = __reduce_add_sync(0xffffffffu, (uint32_t)(d >> 32));
+    if ((threadIdx.x & 31) == 0)
+        atomicAdd(&missing, (unsigned long long)l0 + ((unsigned long long)l1 << 16) + ((unsigned long long)l2 << 32));
+    __syncthreads();
+    if (missing == 0) {
+        tile_flush<D, false>(lo, carry, rho, ox, oy, oz, logn);
+        return;
     }
+    tile_zero<D::WORDS>(lo);  // the carries follow the cells
+    __syncthreads();
+    redo();
+    __syncthreads();
+    tile_flush<D, true>(lo, carry, rho, ox, oy, oz, logn);
 }
 
 // Deposit of a thread walking its lattice row along x (R = 1).  The next particle usually
@@ -136,20 +204,29 @@ __device__ __forceinline__ void tile_flush(const uint32_t* lo, const uint32_t* c
 // dnext) and added with the next particle's lower plane: 4 tile atomics a particle instead
 // of 8.  A particle whose stencil leaves the box adds to rho directly.
 struct SweepCarry {
-    int dnext = -1;  // tile cell of the carried plane's (b, c) = (0, 0) corner, -1: none
-    float W[4];      // carried weights, corner (b, c) = 2 b + c
+    int dnext = -1;    // tile cell of the carried plane's (b, c) = (0, 0) corner, -1: none
+    float W[4];        // carried weights, corner (b, c) = 2 b + c
+    uint32_t sum = 0;  // quanta added to the tile by this thread
 };
 
 template <class D>
-__device__ __forceinline__ void sweep_deposit(uint32_t* lo, uint32_t* carry, float* __restrict__ rho, uint32_t u0,
-                                              uint32_t u1, uint32_t u2, int logn, float inv_cell_ticks, int ox,
-                                              int oy, int oz, float mass, SweepCarry& sc) {
+__device__ __forceinline__ void sweep_carried(uint32_t* lo, SweepCarry& sc) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) tile_add(lo, sc.dnext + b * D::DZ + c, sc.W[2 * b + c], sc.sum);
+}
+
+template <class D>
+__device__ __forceinline__ void sweep_deposit(uint32_t* lo, float* __restrict__ rho, uint32_t u0, uint32_t u1,
+                                              uint32_t u2, int logn, float inv_cell_ticks, int ox, int oy, int oz,
+                                              float quanta, SweepCarry& sc) {
     const int nm = (1 << logn) - 1;
     const CicF cx = cic_ticks(u0, logn, inv_cell_ticks);
     const CicF cy = cic_ticks(u1, logn, inv_cell_ticks);
     const CicF cz = cic_ticks(u2, logn, inv_cell_ticks);
     const float wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};
-    const float m0 = mass * (1.0f - cx.w1), m1 = mass * cx.w1;
+    const float m0 = quanta * (1.0f - cx.w1), m1 = quanta * cx.w1;
     const int dx = (cx.i0 - ox) & nm, dy = (cy.i0 - oy) & nm, dz = (cz.i0 - oz) & nm;
     if (dx < D::DX - 1 && dy < D::DY - 1 && dz < D::DZ - 1) {
         const int c0 = (dx * D::DY + dy) * D::DZ + dz;
@@ -162,29 +239,21 @@ __device__ __forceinline__ void sweep_deposit(uint32_t* lo, uint32_t* carry, flo
 #pragma unroll
             for (int q = 0; q < 4; ++q) w0[q] += sc.W[q];
         } else if (sc.dnext >= 0) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) tile_add(lo, carry, sc.dnext + b * D::DZ + c, sc.W[2 * b + c]);
+            sweep_carried<D>(lo, sc);
         }
 #pragma unroll
         for (int b = 0; b < 2; ++b)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                tile_add(lo, carry, c0 + b * D::DZ + c, w0[2 * b + c]);
+                tile_add(lo, c0 + b * D::DZ + c, w0[2 * b + c], sc.sum);
                 sc.W[2 * b + c] = m1 * wy[b] * wz[c];
             }
         sc.dnext = c0 + D::DY * D::DZ;
     } else {
-        if (sc.dnext >= 0) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) tile_add(lo, carry, sc.dnext + b * D::DZ + c, sc.W[2 * b + c]);
-        }
+        if (sc.dnext >= 0) sweep_carried<D>(lo, sc);
         sc.dnext = -1;
         const uint32_t ix[2] = {(uint32_t)cx.i0, (uint32_t)cx.i1}, iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1};
-        const float mx[2] = {m0, m1};
+        const float mx[2] = {m0 * kTileQuantum, m1 * kTileQuantum};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -193,17 +262,6 @@ __device__ __forceinline__ void sweep_deposit(uint32_t* lo, uint32_t* carry, flo
                 atomicAdd(row + cz.i0, mx[a] * wy[b] * wz[0]);
                 atomicAdd(row + cz.i1, mx[a] * wy[b] * wz[1]);
             }
-    }
-}
-
-// The carried plane of the row's last particle.
-template <class D>
-__device__ __forceinline__ void sweep_finish(uint32_t* lo, uint32_t* carry, const SweepCarry& sc) {
-    if (sc.dnext >= 0) {
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) tile_add(lo, carry, sc.dnext + b * D::DZ + c, sc.W[2 * b + c]);
     }
 }
 
@@ -231,42 +289,54 @@ __device__ __forceinline__ void fd1_force(const T* L, const T* U, T wx0, T wx1, 
     f2 = inv_d * gz;
 }
 
-// p += kick * g(x);  x += drift * p   (g = -grad phi gathered with the deposit's weights).
-// The eight corner offsets are formed once in 32 bits (n^3 <= 2^30) and serve the
-// three force meshes.  FD: gx is the potential and g its first-order gradient (fd1_force).
+// The CIC corners of one x plane of a mesh of ROWS z rows a cell row: 32-bit element offsets
+// (3 n^3 < 2^32) of (y, z) corner q = 2 b + c, the periodic wrap included.  One offset serves
+// the three components of the force meshes (kForceRows), a row apart.
+template <int ROWS>
+struct PlaneCorners {
+    uint32_t o00;
+    int dy, dz;
+    __device__ __forceinline__ PlaneCorners(int ix, const CicF& cy, const CicF& cz, int logn)
+        : o00((uint32_t)((((ix << logn) + cy.i0) * ROWS) << logn) + (uint32_t)cz.i0),
+          dy((cy.i1 - cy.i0) * (ROWS << logn)), dz(cz.i1 - cz.i0) {}
+    __device__ __forceinline__ uint32_t operator[](int q) const {
+        return o00 + (uint32_t)((q & 2 ? dy : 0) + (q & 1 ? dz : 0));
+    }
+};
+
+// p += kick * g(x);  x += drift * p   (g = -grad phi gathered with the deposit's weights; the
+// force meshes in the layout kForceRows).  FD: g is the potential, a plain mesh, differentiated
+// to first order (fd1_force).
 template <bool FD>
 __device__ __forceinline__ void ikd_particle(uint32_t& u0, uint32_t& u1, uint32_t& u2, float& p0, float& p1,
-                                             float& p2, int logn, float inv_cell_ticks, const float* __restrict__ gx,
-                                             const float* __restrict__ gy, const float* __restrict__ gz, float kick,
-                                             float drift_ticks, float inv_d) {
+                                             float& p2, int logn, float inv_cell_ticks, const float* __restrict__ g,
+                                             float kick, float drift_ticks, float inv_d) {
+    constexpr int ROWS = FD ? 1 : kForceRows;
     const CicF cx = cic_ticks(u0, logn, inv_cell_ticks);
     const CicF cy = cic_ticks(u1, logn, inv_cell_ticks);
     const CicF cz = cic_ticks(u2, logn, inv_cell_ticks);
     const float wx[2] = {1.0f - cx.w1, cx.w1}, wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};
-    const uint32_t ix[2] = {(uint32_t)cx.i0, (uint32_t)cx.i1}, iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1};
+    const PlaneCorners<ROWS> k[2] = {{cx.i0, cy, cz, logn}, {cx.i1, cy, cz, logn}};
     float f0 = 0.f, f1 = 0.f, f2 = 0.f;
     if constexpr (FD) {
         float P[2][4];
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const uint32_t row = ((ix[a] << logn) + iy[b]) << logn;
-                P[a][2 * b] = __ldg(gx + row + (uint32_t)cz.i0);
-                P[a][2 * b + 1] = __ldg(gx + row + (uint32_t)cz.i1);
-            }
+            for (int q = 0; q < 4; ++q) P[a][q] = __ldg(g + k[a][q]);
         fd1_force<float>(P[0], P[1], wx[0], wx[1], wy, wz, inv_d, f0, f1, f2);
     } else {
+        const int n = 1 << logn;
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const uint32_t row = ((ix[a] << logn) + iy[b]) << logn;
-                const uint32_t o0 = row + (uint32_t)cz.i0, o1 = row + (uint32_t)cz.i1;
+                const float* c0 = g + k[a][2 * b];
+                const float* c1 = g + k[a][2 * b + 1];
                 const float w0 = wx[a] * wy[b] * wz[0], w1 = wx[a] * wy[b] * wz[1];
-                f0 = fmaf(w0, __ldg(gx + o0), fmaf(w1, __ldg(gx + o1), f0));
-                f1 = fmaf(w0, __ldg(gy + o0), fmaf(w1, __ldg(gy + o1), f1));
-                f2 = fmaf(w0, __ldg(gz + o0), fmaf(w1, __ldg(gz + o1), f2));
+                f0 = fmaf(w0, __ldg(c0), fmaf(w1, __ldg(c1), f0));
+                f1 = fmaf(w0, __ldg(c0 + n), fmaf(w1, __ldg(c1 + n), f1));
+                f2 = fmaf(w0, __ldg(c0 + 2 * n), fmaf(w1, __ldg(c1 + 2 * n), f2));
             }
     }
     p0 = fmaf(kick, f0, p0);
