@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256) k_deposit_vec_rows(const uint32_t* __rest
 //   mode with a Nyquist component.  The zero mode is zero.
 __global__ void k_adj_combine(const float2* __restrict__ in0, const float2* __restrict__ in1,
                               const float2* __restrict__ in2, float2* __restrict__ out, int n, double kf, double coef,
-                              const double* __restrict__ amp, int mode) {
+                              const float2* __restrict__ amp, int mode) {
     const int M = n / 2;
     const int64_t total = (int64_t)(M + 1) * n * n;
     const float kff = (float)kf, kf2 = kff * kff, coef_f = (float)coef;
@@ -298,7 +298,7 @@ __global__ void k_adj_combine(const float2* __restrict__ in0, const float2* __re
         if (n2 > 0 && !(mode == 1 && nyq_any)) {
             // FP32 arithmetic (no FP64 divide per mode): c = coef / (kf^2 n2) [* amp(n2)]
             float c = coef_f / (kf2 * (float)n2);
-            if (mode == 1) c *= (float)amp[n2];
+            if (mode == 1) c *= amp[n2].x;
             const float kx = (2 * nx == -n) ? 0.f : kff * (float)nx;
             const float ky = (2 * ny == -n) ? 0.f : kff * (float)ny;
             const float kzz = (nz == M) ? 0.f : kff * (float)nz;
@@ -389,7 +389,7 @@ cudaError_t deposit_vec(const uint32_t* x, int np, int n, const float* v, float*
     return cudaGetLastError();
 }
 
-cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const double* amp,
+cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const float2* amp,
                         int mode, cudaStream_t st) {
     const int64_t total = (int64_t)(n / 2 + 1) * n * n;
     k_adj_combine<<<blocks_for(total), 256, 0, st>>>(in[0], in[1], in[2], out, n, kf, coef, amp, mode);

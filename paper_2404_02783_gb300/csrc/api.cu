@@ -276,14 +276,14 @@ pm_status lpt2_displacement(pm_ctx* c, void* const* psi1, void* s, void* a, void
         SpecOp od;
         od.za_filter = ZA_IDENTITY;  // out_j = d_j Psi1_comp
         od.coef = -inv_n3;
-        od.amp = (const double*)c->at(c->L.amp);
+        od.amp = c->at(c->L.amp);
         PM_TRY(za_chain<T>(c, psi1[comp], od, out));
         PM_CK(lpt2_source(comp, out, s, a, c->np3, c->cfg.precision, c->st));
     }
     SpecOp o2;
     o2.za_filter = ZA_INV_LAPLACE;  // out_j = d_j phi2, phi2 = laplacian^-1 S
     o2.coef = inv_n3;
-    o2.amp = (const double*)c->at(c->L.amp);
+    o2.amp = c->at(c->L.amp);
     return za_chain<T>(c, s, o2, out);
 }
 
@@ -787,13 +787,15 @@ pm_status pm_init(const pm_config* cfg, void* workspace, size_t bytes, void* str
     const double V = cfg->box * cfg->box * cfg->box;
     for (size_t n2 = 1; n2 < amp.size(); ++n2)
         amp[n2] = std::sqrt(pmhost::power_linear(c->cosmo, c->kf * std::sqrt((double)n2)) / V);
+    std::vector<double> amp_dev(amp.size());  // 8 bytes an entry in either precision
+    amp_table(amp.data(), amp.size(), c->fp64(), amp_dev.data());
     std::vector<double> wtab(c->n / 2 + 1);
     for (int mq = 0; mq <= c->n / 2; ++mq) {
         const double x = M_PI * mq / c->n;
         const double s = (mq == 0) ? 1.0 : std::sin(x) / x;
         wtab[mq] = s * s;
     }
-    cudaError_t e = cudaMemcpyAsync(c->at(L.amp), amp.data(), amp.size() * 8, cudaMemcpyHostToDevice, c->st);
+    cudaError_t e = cudaMemcpyAsync(c->at(L.amp), amp_dev.data(), amp.size() * 8, cudaMemcpyHostToDevice, c->st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->at(L.wtab), wtab.data(), wtab.size() * 8, cudaMemcpyHostToDevice, c->st);
     if (e == cudaSuccess)
@@ -940,7 +942,7 @@ pm_status pm_ic_zeldovich(pm_ctx* c, uint64_t seed, const void* white_noise, int
     const double E = pmhost::E(c->cosmo, a);
     SpecOp op;
     op.za_filter = ZA_AMP;
-    op.amp = (const double*)c->at(c->L.amp);
+    op.amp = c->at(c->L.amp);
     op.fixed_amp = (flags & PM_IC_FIXED) ? 1 : 0;
     const double sign = paired ? -1.0 : 1.0;
     double scale = 1.0;
@@ -948,8 +950,8 @@ pm_status pm_ic_zeldovich(pm_ctx* c, uint64_t seed, const void* white_noise, int
         if (!op.fixed_amp) scale = std::pow((double)np, -1.5);
     } else {
         void* s0 = c->at(c->L.spec[0]);
-        if (c->fp64()) PM_CK(noise<double>((double2*)s0, np, seed, c->st));
-        else PM_CK(noise<float>((float2*)s0, np, seed, c->st));
+        if (c->fp64()) PM_CK(noise<double>((double2*)s0, np, &seed, 1, c->st));
+        else PM_CK(noise<float>((float2*)s0, np, &seed, 1, c->st));
     }
     op.coef = -sign * scale;
     void* force[3] = {c->at(c->L.force[0]), c->at(c->L.force[1]), c->at(c->L.force[2])};
@@ -1628,7 +1630,7 @@ struct AdjSweep {
             PM_TRY(fft_forward_f32(c, s_j[j], sp[j], np));
         }
         const float2* in[3] = {sp[0], sp[1], sp[2]};
-        PM_CK(adj_combine(in, sp[0], np, c->kf, -std::pow((double)np, -1.5), (const double*)c->at(c->L.amp), 1,
+        PM_CK(adj_combine(in, sp[0], np, c->kf, -std::pow((double)np, -1.5), (const float2*)c->at(c->L.amp), 1,
                           c->st));
         PM_TRY(fft_inverse_f32(c, sp[0], (float*)grad_out, np));
         return PM_OK;
@@ -1923,6 +1925,53 @@ pm_status batch_enqueue_step(pm_batch* b, cudaStream_t s) {
     return PM_OK;
 }
 
+// First-order ICs of every realisation, each pass one launch over a group of them (one launch a
+// realisation and pass took 64 x 100 us for 64^3 lattices: kernels of a few microseconds).
+pm_status batch_zeldovich(pm_batch* b, const uint64_t* seeds, int flags) {
+    if (flags & ~(PM_IC_PAIRED | PM_IC_FIXED)) return fail(PM_ERR_INVALID_ARG, "unknown IC flags");
+    const int np = b->cfg.np;
+    const size_t np3 = (size_t)np * np * np;
+    const double a = b->cfg.a_init;
+    const double D = pmhost::growth_D(b->cosmo, a), f = pmhost::growth_f(b->cosmo, a), E = pmhost::E(b->cosmo, a);
+    // the z passes' grid takes np rows a realisation in its y dimension
+    const int group = std::min(b->B, 65535 / np);
+    for (int r0 = 0; r0 < b->B; r0 += group) {
+        const int c = std::min(group, b->B - r0);
+        const double* kf = (const double*)b->at(b->KF) + r0;
+        float2* s[3];
+        float* psi[3];
+        for (int j = 0; j < 3; ++j) {
+            s[j] = (float2*)b->at(b->SPEC[j]);
+            psi[j] = (float*)b->at(b->FORCE[j]);
+        }
+        PM_CK(noise<float>(s[0], np, seeds + r0, c, b->st));
+        SpecOp op;
+        op.kind = OP_ZA;
+        op.za_filter = ZA_AMP;
+        op.fwd = 0;
+        op.coef = (flags & PM_IC_PAIRED) ? 1.0 : -1.0;
+        op.fixed_amp = (flags & PM_IC_FIXED) ? 1 : 0;
+        op.kf_arr = kf;
+        op.amp = (const char*)b->at(b->AMP) + (size_t)r0 * b->amp_len * 8;
+        op.amp_stride = b->amp_len;
+        const int64_t rows = (int64_t)(np / 2 + 1) * np;
+        PM_CK(x_cols<float>(s[0], s[1], c * (np / 2 + 1), np, op, b->st));
+        PM_CK(y_rows_grad3<float>(s[0], s[1], s[2], c * rows, np, 0.0, b->st, kf, rows));
+        const float2* in[3] = {s[1], s[2], s[0]};
+        PM_CK(z_c2r<float>(in, psi, 3, np, c, 4u, 0.0, b->st, kf));
+        void* ps[3] = {psi[0], psi[1], psi[2]};
+        PM_CK(ic_place((uint32_t*)b->at(b->X) + r0 * 3 * np3, (float*)b->at(b->P) + r0 * 3 * np3, ps, np, PM_FP32_FIXED, D,
+                       a * a * E * f * D, 1.0, b->st, c, (const double*)b->at(b->SCALE) + r0));
+    }
+    for (pm_ctx* v : b->views) {
+        v->step = 0;
+        v->synced = true;
+        v->have_phi = false;
+        v->rho_valid = false;
+    }
+    return PM_OK;
+}
+
 void batch_drop_graph(pm_batch* b) {
     if (b->exec) {
         cudaStreamSynchronize(b->cap);
@@ -2018,7 +2067,9 @@ pm_status pm_batch_init(const pm_config* cfg, int nreal, const double* boxes, vo
         const double sq = (mq == 0) ? 1.0 : std::sin(xq) / xq;
         wtab[mq] = sq * sq;
     }
-    cudaError_t e = cudaMemcpyAsync(b->at(b->AMP), amp.data(), amp.size() * 8, cudaMemcpyHostToDevice, b->st);
+    std::vector<double> amp_dev(amp.size());
+    amp_table(amp.data(), amp.size(), false, amp_dev.data());
+    cudaError_t e = cudaMemcpyAsync(b->at(b->AMP), amp_dev.data(), amp.size() * 8, cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->at(b->KF), kf.data(), kf.size() * 8, cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->at(b->SCALE), scale.data(), scale.size() * 8, cudaMemcpyHostToDevice, b->st);
@@ -2055,7 +2106,11 @@ pm_status pm_batch_context(pm_batch* b, int r, pm_ctx** view) {
 
 pm_status pm_batch_ic(pm_batch* b, const uint64_t* seeds, int flags) {
     if (!b || !seeds) return fail(PM_ERR_INVALID_ARG, "null argument");
-    for (int r = 0; r < b->B; ++r) PM_TRY(pm_ic_zeldovich(b->views[r], seeds[r], nullptr, flags));
+    if (flags & PM_IC_2LPT) {
+        for (int r = 0; r < b->B; ++r) PM_TRY(pm_ic_zeldovich(b->views[r], seeds[r], nullptr, flags));
+    } else {
+        PM_TRY(batch_zeldovich(b, seeds, flags));
+    }
     b->have_ic = true;
     b->step = 0;
     b->synced = true;

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 
+#include "dfloat.cuh"
 #include "fft.cuh"
 #include "internal.h"
 
@@ -400,6 +401,22 @@ __device__ __forceinline__ void gr_modes(const SpecOp& op, cplx<T>* v, int t, in
     }
 }
 
+// The Zel'dovich filter of a mode n2 > 0 (ZaFilter): FP64 for the FP64 path; for FP32 the same
+// value from pairs of FP32 numbers (an FP64 divide a mode made the pass 1.8 ms at 512^3).
+template <typename T>
+__device__ __forceinline__ T za_filter(const SpecOp& op, int n2, int field, double kf) {
+    if (op.za_filter == ZA_IDENTITY) return T(op.coef);
+    const double c = div_mode<double>(op.coef, kf * kf);
+    if constexpr (sizeof(T) == 8) {
+        if (op.za_filter == ZA_INV_LAPLACE) return c / (double)n2;
+        return c * (static_cast<const double*>(op.amp) + (int64_t)field * op.amp_stride)[n2] / (double)n2;
+    } else {
+        df v = df_of(c);
+        if (op.za_filter != ZA_INV_LAPLACE) v = v * (static_cast<const df*>(op.amp) + (int64_t)field * op.amp_stride)[n2];
+        return round_df(df_div(v, (float)(n2 > 0 ? n2 : 1)));
+    }
+}
+
 // The per-mode operator of the x pass on mode (nx, ny, nz), |n|^2 = n2, of field `field`:
 // the Newtonian Green's function (or the potential alone), the Zel'dovich filter, or the
 // linearised Poisson-gauge constraint (which reads and updates its Phi history at `old` and,
@@ -414,16 +431,12 @@ __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx,
         phi = (n2 == 0) ? cmake<C>(T(0), T(0)) : cscale(vv, div_mode(coefT, T(n2)));
     } else if constexpr (KIND == OP_ZA) {
         const bool nyq = (2 * nx == -N) || (2 * ny == -N) || (nz == M);
-        const double* amp = op.amp + (int64_t)field * op.amp_stride;
         C g = vv;
         if (op.fixed_amp) {  // keep the phase, set |g| = 1
             const T r2 = g.x * g.x + g.y * g.y;
             g = (r2 > T(0)) ? cscale(g, rsqrt(r2)) : cmake<C>(T(0), T(0));
         }
-        const double filt = op.za_filter == ZA_IDENTITY  ? op.coef
-                            : op.za_filter == ZA_INV_LAPLACE ? op.coef / (kf * kf * (double)n2)
-                                                             : op.coef / (kf * kf) * amp[n2] / (double)n2;
-        phi = (n2 == 0 || nyq) ? cmake<C>(T(0), T(0)) : cscale(g, T(filt));
+        phi = (n2 == 0 || nyq) ? cmake<C>(T(0), T(0)) : cscale(g, za_filter<T>(op, n2, field, kf));
     } else {  // OP_GR
         if (n2 <= op.n_lo * op.n_lo) {
             phi = gr_island_mode<T>(op, vv, nx, ny, nz, n2, field, kf);

@@ -38,7 +38,7 @@ struct SpecOp {
     void* phi_old = nullptr;  // cplx<T> [kz][kx][ky]
     double2* island = nullptr;  // double2 [(n_lo+1)(2 n_lo+1)^2]
     // Zel'dovich
-    const double* amp = nullptr;  // sqrt(P(k)/V) per integer |n|^2
+    const void* amp = nullptr;    // sqrt(P(k)/V) per integer |n|^2: double, or pairs of FP32 numbers (amp_table)
     int fixed_amp = 0;            // phases scaled to unit modulus first (fixed amplitudes)
     int za_filter = 0;            // ZA_AMP: coef amp[|n|^2] / k^2; ZA_IDENTITY: coef; ZA_INV_LAPLACE: coef / k^2
     // power spectrum
@@ -51,6 +51,9 @@ struct SpecOp {
     int deconv = 0;
     const void* in2 = nullptr;        // second (y-transformed) field for the cross spectrum
 };
+
+// The amplitude table as the kernels of a precision read it, 8 bytes an entry.
+void amp_table(const double* amp, size_t count, bool fp64, void* out);
 
 // Uploads the twiddle tables exp(-2 pi i k / 1024) of both precisions to the current
 // device (once per device).

@@ -15,6 +15,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "dfloat.cuh"
 #include "internal.h"
 #include "particles.h"
 #include "update_dev.cuh"
@@ -392,13 +393,50 @@ cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, in
 }
 
 // ---------------------------------------------------------------- Zel'dovich placement
-// x = q + D Psi(q), p = a^2 E f D Psi(q); q the lattice node of particle id i.
+// x = q + D Psi(q), p = a^2 E f D Psi(q); q the lattice node of particle id i.  The FP32 path
+// multiplies by pairs (dfloat.cuh) instead of in FP64: at 512^3 the FP64 products and their
+// conversions took 3.6 ms for 4.8 GB moved.
+// The displacement in ticks: the pair rounded to the nearest integer; beyond 2^30 ticks (a
+// quarter of the box) in FP64, whose 64-bit conversion wraps like the positions.
+struct TickScale {
+    df f;
+    double d;
+};
+__device__ __forceinline__ uint32_t disp_ticks(float ps, const TickScale& s) {
+    df v = two_prod(ps, s.f.h);
+    if (!(fabsf(v.h) < 1073741824.0f)) return (uint32_t)__double2ll_rn((double)ps * s.d);
+    v.l = fmaf(ps, s.f.l, v.l);
+    return (uint32_t)df2int_rn(v);
+}
+// The two terms of the second-order placement.
+__device__ __forceinline__ uint32_t disp_ticks(float p1, const TickScale& s1, float p2, const TickScale& s2) {
+    df a = two_prod(p1, s1.f.h), b = two_prod(p2, s2.f.h);
+    a.l = fmaf(p1, s1.f.l, a.l);
+    b.l = fmaf(p2, s2.f.l, b.l);
+    const df v = a + b;
+    if (!(fabsf(a.h) < 1073741824.0f && fabsf(b.h) < 1073741824.0f && fabsf(v.h) < 1073741824.0f))
+        return (uint32_t)__double2ll_rn((double)p1 * s1.d + (double)p2 * s2.d);
+    return (uint32_t)df2int_rn(v);
+}
+static TickScale tick_scale(double d) { return TickScale{df_of(d), d}; }
+
+// blockIdx.y selects the field of a batch (particles [field][3][np^3], meshes [field][np^3]),
+// whose displacement in ticks is D scale_arr[field].
 __global__ void k_ic_ticks(uint32_t* __restrict__ x, float* __restrict__ p, const float* __restrict__ psx,
-                           const float* __restrict__ psy, const float* __restrict__ psz, int lognp,
-                           double disp_ticks, double pfac) {
+                           const float* __restrict__ psy, const float* __restrict__ psz, int lognp, TickScale scale,
+                           double D, const double* __restrict__ scale_arr, df pfac) {
     const int64_t count = (int64_t)1 << (3 * lognp);
     const int sh = 32 - lognp;
     const int mask = (1 << lognp) - 1;
+    if (scale_arr) {
+        scale.d = D * scale_arr[blockIdx.y];
+        scale.f = df_of(scale.d);
+        x += blockIdx.y * 3 * count;
+        p += blockIdx.y * 3 * count;
+        psx += blockIdx.y * count;
+        psy += blockIdx.y * count;
+        psz += blockIdx.y * count;
+    }
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t q[3] = {(uint32_t)((i >> (2 * lognp)) & mask) << sh, (uint32_t)((i >> lognp) & mask) << sh,
@@ -406,8 +444,8 @@ __global__ void k_ic_ticks(uint32_t* __restrict__ x, float* __restrict__ p, cons
         const float ps[3] = {psx[i], psy[i], psz[i]};
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            x[j * count + i] = q[j] + (uint32_t)__double2ll_rn((double)ps[j] * disp_ticks);
-            p[j * count + i] = (float)(pfac * (double)ps[j]);
+            x[j * count + i] = q[j] + disp_ticks(ps[j], scale);
+            p[j * count + i] = fmaf(ps[j], pfac.h, ps[j] * pfac.l);
         }
     }
 }
@@ -434,13 +472,13 @@ __global__ void k_ic_frac(double* __restrict__ x, double* __restrict__ p, const 
 }
 
 cudaError_t ic_place(void* x, void* p, void* const* psi, int np, int precision, double D, double pfac, double box,
-                     cudaStream_t st) {
+                     cudaStream_t st, int nfields, const double* scale_arr) {
     const int lognp = ilog2(np);
     const int64_t count = (int64_t)np * np * np;
     if (precision == PM_FP32_FIXED) {
-        k_ic_ticks<<<grid_for(count, 256), 256, 0, st>>>((uint32_t*)x, (float*)p, (const float*)psi[0],
-                                                         (const float*)psi[1], (const float*)psi[2], lognp,
-                                                         D * 4294967296.0 / box, pfac);
+        k_ic_ticks<<<dim3(grid_for(count, 256), nfields), 256, 0, st>>>(
+            (uint32_t*)x, (float*)p, (const float*)psi[0], (const float*)psi[1], (const float*)psi[2], lognp,
+            tick_scale(D * 4294967296.0 / box), D, scale_arr, df_of(pfac));
     } else {
         k_ic_frac<<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, (const double*)psi[0],
                                                         (const double*)psi[1], (const double*)psi[2], lognp, D / box,
@@ -491,8 +529,8 @@ struct Psi3 {
     const void* c[3];
 };
 
-__global__ void k_ic2_ticks(uint32_t* __restrict__ x, float* p, Psi3 ps1, Psi3 ps2, int lognp, double disp1,
-                            double disp2, double pfac1, double pfac2) {
+__global__ void k_ic2_ticks(uint32_t* __restrict__ x, float* p, Psi3 ps1, Psi3 ps2, int lognp, TickScale disp1,
+                            TickScale disp2, df pfac1, df pfac2) {
     const int64_t count = (int64_t)1 << (3 * lognp);
     const int sh = 32 - lognp;
     const int mask = (1 << lognp) - 1;
@@ -500,16 +538,16 @@ __global__ void k_ic2_ticks(uint32_t* __restrict__ x, float* p, Psi3 ps1, Psi3 p
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t q[3] = {(uint32_t)((i >> (2 * lognp)) & mask) << sh, (uint32_t)((i >> lognp) & mask) << sh,
                                (uint32_t)(i & mask) << sh};
-        double a1[3], a2[3];
+        float a1[3], a2[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            a1[j] = (double)((const float*)ps1.c[j])[i];
-            a2[j] = (double)((const float*)ps2.c[j])[i];
+            a1[j] = ((const float*)ps1.c[j])[i];
+            a2[j] = ((const float*)ps2.c[j])[i];
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            x[j * count + i] = q[j] + (uint32_t)__double2ll_rn(a1[j] * disp1 + a2[j] * disp2);
-            p[j * count + i] = (float)(pfac1 * a1[j] + pfac2 * a2[j]);
+            x[j * count + i] = q[j] + disp_ticks(a1[j], disp1, a2[j], disp2);
+            p[j * count + i] = round_df(a1[j] * pfac1 + a2[j] * pfac2);
         }
     }
 }
@@ -546,8 +584,9 @@ cudaError_t ic_place2(void* x, void* p, void* const* psi1, void* const* psi2, in
     const Psi3 a = {{psi1[0], psi1[1], psi1[2]}}, b = {{psi2[0], psi2[1], psi2[2]}};
     if (precision == PM_FP32_FIXED) {
         k_ic2_ticks<<<grid_for(count, 256), 256, 0, st>>>((uint32_t*)x, (float*)p, a, b, lognp,
-                                                          D1 * 4294967296.0 / box, D2 * 4294967296.0 / box, pfac1,
-                                                          pfac2);
+                                                          tick_scale(D1 * 4294967296.0 / box),
+                                                          tick_scale(D2 * 4294967296.0 / box), df_of(pfac1),
+                                                          df_of(pfac2));
     } else {
         k_ic2_frac<<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, a, b, lognp, D1 / box, D2 / box,
                                                          pfac1, pfac2);
@@ -575,17 +614,42 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
+// Unit complex Gaussian of mode draw (r.x, r.y) by the Box-Muller transform: in FP64, and for
+// FP32 phases in pairs of FP32 numbers (dfloat.cuh), which round to the same phases but for 3 in
+// ten thousand (neighbouring FP32 numbers there).  At 512^3 the FP64 logarithm, square root and
+// sine took 9.4 ms of the 16.5 ms of the initial conditions; this is bound by issue instead.
+__device__ __forceinline__ void unit_gaussian(uint4 r, double2& g) {
+    const double u1 = ((double)r.x + 0.5) * 2.3283064365386963e-10;  // 2^-32
+    const double u2 = ((double)r.y + 0.5) * 2.3283064365386963e-10;
+    const double amp = sqrt(-log(u1));
+    double s, c;
+    sincospi(2.0 * u2, &s, &c);
+    g = make_double2(amp * c, amp * s);
+}
+__device__ __forceinline__ void unit_gaussian(uint4 r, float2& g) {
+    const df amp = df_sqrt(neg_log_unit(r.x));
+    df s, c;
+    sincos_unit(r.y, s, c);
+    g = make_float2(round_df(amp * c), round_df(amp * s));
+}
+
 // Unit complex Gaussian per wavevector on the [kz][kx][ky] half grid; Hermitian
 // partners on kz = 0 are conjugates of the canonical draw; Nyquist and zero modes 0.
+// blockIdx.y selects the field of a batch, drawn from seeds.s[field].
+struct Seeds {
+    static constexpr int MAX = 128;
+    uint64_t s[MAX];
+};
 template <typename T>
-__global__ void k_noise(cplx<T>* __restrict__ spec, int n, uint32_t seed_lo, uint32_t seed_hi) {
-    const int M = n >> 1;
-    const int64_t total = (int64_t)(M + 1) * n * n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int kz = (int)(e / ((int64_t)n * n));
-        const int rem = (int)(e - (int64_t)kz * n * n);
-        const int nx = signed_k(rem / n, n), ny = signed_k(rem % n, n), nz = kz;
+__global__ void k_noise(cplx<T>* __restrict__ spec, int logn, Seeds seeds) {
+    const int n = 1 << logn, M = n >> 1;
+    const uint32_t total = (uint32_t)(M + 1) << (2 * logn);  // at most 513 x 2^20
+    const uint64_t seed = seeds.s[blockIdx.y];
+    spec += (size_t)blockIdx.y * total;
+    const uint32_t seed_lo = (uint32_t)seed, seed_hi = (uint32_t)(seed >> 32);
+    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int nz = (int)(e >> (2 * logn));
+        const int nx = signed_k((int)(e >> logn) & (n - 1), n), ny = signed_k((int)e & (n - 1), n);
         cplx<T> g;
         g.x = T(0);
         g.y = T(0);
@@ -594,26 +658,26 @@ __global__ void k_noise(cplx<T>* __restrict__ spec, int n, uint32_t seed_lo, uin
             const bool canonical = nz > 0 || ny > 0 || (ny == 0 && nx > 0);
             const int cx = canonical ? nx : -nx, cy = canonical ? ny : -ny;
             const uint4 r = philox4x32_10(make_uint4((uint32_t)cx, (uint32_t)cy, (uint32_t)nz, 0u), seed_lo, seed_hi);
-            const double u1 = ((double)r.x + 0.5) * 2.3283064365386963e-10;  // 2^-32
-            const double u2 = ((double)r.y + 0.5) * 2.3283064365386963e-10;
-            const double amp = sqrt(-log(u1));
-            double s, c;
-            sincospi(2.0 * u2, &s, &c);
-            g.x = T(amp * c);
-            g.y = T(canonical ? amp * s : -amp * s);
+            unit_gaussian(r, g);
+            if (!canonical) g.y = -g.y;
         }
         spec[e] = g;
     }
 }
 
 template <typename T>
-cudaError_t noise(cplx<T>* spec, int n, uint64_t seed, cudaStream_t st) {
+cudaError_t noise(cplx<T>* spec, int n, const uint64_t* seeds, int nfields, cudaStream_t st) {
     const int64_t total = (int64_t)(n / 2 + 1) * n * n;
-    k_noise<T><<<grid_for(total, 256), 256, 0, st>>>(spec, n, (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32));
+    for (int f0 = 0; f0 < nfields; f0 += Seeds::MAX) {
+        const int c = nfields - f0 < Seeds::MAX ? nfields - f0 : Seeds::MAX;
+        Seeds s = {};
+        for (int i = 0; i < c; ++i) s.s[i] = seeds[f0 + i];
+        k_noise<T><<<dim3(grid_for(total, 256), c), 256, 0, st>>>(spec + (size_t)f0 * total, ilog2(n), s);
+    }
     return cudaGetLastError();
 }
-template cudaError_t noise<float>(float2*, int, uint64_t, cudaStream_t);
-template cudaError_t noise<double>(double2*, int, uint64_t, cudaStream_t);
+template cudaError_t noise<float>(float2*, int, const uint64_t*, int, cudaStream_t);
+template cudaError_t noise<double>(double2*, int, const uint64_t*, int, cudaStream_t);
 
 // ---------------------------------------------------------------- GR displacement combination
 // xi = x_GR - x_N on the coarse lattice (exact minimum image on ticks), trilinear in

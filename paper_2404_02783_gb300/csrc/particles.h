@@ -30,8 +30,9 @@ cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, i
                                       double drift, double box, double mass, void* rho, cudaStream_t st,
                                       int nfields = 1, const double* scale_arr = nullptr, void* x_out = nullptr,
                                       double fd_inv_d = 0.0);
+// nfields > 1 (FP32): a batch stored back to back, box given per field as scale_arr[f] = 2^32 / L_f.
 cudaError_t ic_place(void* x, void* p, void* const* psi, int np, int precision, double D, double pfac, double box,
-                     cudaStream_t st);
+                     cudaStream_t st, int nfields = 1, const double* scale_arr = nullptr);
 // Second-order LPT source, accumulated over three stages, one per displacement component c:
 // d[j] = d Psi1_c / d x_j on the np^3 lattice; s and a are np^3 meshes (ctx precision).
 cudaError_t lpt2_source(int stage, void* const* d, void* s, void* a, int64_t count, int precision, cudaStream_t st);
@@ -39,7 +40,7 @@ cudaError_t lpt2_source(int stage, void* const* d, void* s, void* a, int64_t cou
 cudaError_t ic_place2(void* x, void* p, void* const* psi1, void* const* psi2, int np, int precision, double D1,
                       double D2, double pfac1, double pfac2, double box, cudaStream_t st);
 template <typename T>
-cudaError_t noise(cplx<T>* spec, int n, uint64_t seed, cudaStream_t st);
+cudaError_t noise(cplx<T>* spec, int n, const uint64_t* seeds, int nfields, cudaStream_t st);  // seeds: host, one a field
 cudaError_t combine(void* xt, const void* xg, const void* xn, void* xi_out, int npt, int npc, int precision,
                     cudaStream_t st);
 cudaError_t fill(void* a, int64_t count, int precision, double v, cudaStream_t st);
@@ -82,7 +83,7 @@ cudaError_t adj_kick_particles_fd(const uint32_t* x, int64_t count, int n, float
                                   cudaStream_t st);
 // V_j += CIC deposit of v_j for the np^3 lattice-ordered particles x (V_j zeroed by the caller).
 cudaError_t deposit_vec(const uint32_t* x, int np, int n, const float* v, float* const* V, cudaStream_t st);
-cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const double* amp,
+cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const float2* amp,
                         int mode, cudaStream_t st);
 cudaError_t loss_mse(float* delta, const float* target, int64_t n3, double* acc, cudaStream_t st);
 cudaError_t axpby(float* y, const float* a, const float* b, int64_t m, float alpha, float beta, cudaStream_t st);

@@ -8,6 +8,7 @@
 #include <tuple>
 #include <utility>
 
+#include "dfloat.cuh"
 #include "fft.cuh"
 #include "internal.h"
 
@@ -63,6 +64,13 @@ cudaError_t ensure_device_tables() {
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 128) g_tab_ready[dev] = true;
     return cudaSuccess;
+}
+
+void amp_table(const double* amp, size_t count, bool fp64, void* out) {
+    for (size_t i = 0; i < count; ++i) {
+        if (fp64) static_cast<double*>(out)[i] = amp[i];
+        else static_cast<df*>(out)[i] = df_of(amp[i]);
+    }
 }
 
 static std::mutex g_attr_mutex;
