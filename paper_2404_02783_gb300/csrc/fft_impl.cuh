@@ -111,11 +111,11 @@ __device__ __forceinline__ size_t spec_row(int gl, int kz) {
 // =============================================================== z: r2c
 // sub is subtracted from every input value as it is loaded: the mean of a density mesh (its
 // zero mode, which no operator of the path uses), so that the transform's rounding scales
-// with the fluctuations rather than with the mean.  With sub = 1, v - 1 is exact for v in
+// with the fluctuations rather than with the mean (kz_max: planes beyond it are not written).  With sub = 1, v - 1 is exact for v in
 // [0.5, 2^24] and below 0.5 within half the spacing of the values near 1 (2^-25 in FP32).
 template <typename T, int LOGN>
 __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MINB)
-    k_z_r2c(const T* __restrict__ in, cplx<T>* __restrict__ out, T sub) {
+    k_z_r2c(const T* __restrict__ in, cplx<T>* __restrict__ out, T sub, int kz_max) {
     typedef cplx<T> C;
     typedef ZShape<T, LOGN> S;
     constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MIN
         const C z1 = buf[bb * RS + k], z2 = cconj(buf[bb * RS + ((M - k) & (M - 1))]);
         const C P = cscale(cadd(z1, z2), T(0.5));
         const C O = cmul(cscale(cmul_mi<false>(csub(z1, z2)), T(0.5)), tw_global<T>(k * TWS));
-        out[spec_row<M, LOGN>(gl, k) * N + y0 + bb] = cadd(P, O);
-        if (2 * k != M) out[spec_row<M, LOGN>(gl, M - k) * N + y0 + bb] = cconj(csub(P, O));
+        if (k <= kz_max) out[spec_row<M, LOGN>(gl, k) * N + y0 + bb] = cadd(P, O);
+        if (2 * k != M && M - k <= kz_max) out[spec_row<M, LOGN>(gl, M - k) * N + y0 + bb] = cconj(csub(P, O));
     };
 #pragma unroll
     for (int it = 0; it < E / 2; ++it) pair(k0 + it * Q);
@@ -495,6 +495,11 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
         const double kf = op.kf_arr ? op.kf_arr[field] : op.kf;
         const int c = (int)(blk % NCG) * CB + b;
         const size_t pbase = (size_t)plane * N * N;
+        if constexpr (KIND == OP_BIN) {
+            // every mode of the block beyond the last bin (a fifth of them with the whole sphere)
+            const int c0 = c - b, ymin = c0 < M ? c0 : N - c0 - CB + 1;
+            if (ymin * ymin + kz * kz > op.n2_max) continue;
+        }
         C* base = data + pbase + c;
         C v[1][E];
 #pragma unroll
@@ -561,17 +566,17 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
                 const int nxa = (ia < M) ? ia : ia - N, nxb = (ib < M) ? ib : ib - N;
                 const int n2a = nxa * nxa + nyz2, n2b = nxb * nxb + nyz2;
                 int bin_all = -1;
-                if (n2a > 0 && n2b > 0 && n2a <= M * M && n2b <= M * M) {
+                if (n2a > 0 && n2b > 0 && n2a <= op.n2_max && n2b <= op.n2_max) {
                     const int ba = op.bin_of[n2a], bb = op.bin_of[n2b];
                     if (ba == bb) bin_all = ba;
-                } else if (n2a > M * M && n2b > M * M) {
+                } else if (n2a > op.n2_max && n2b > op.n2_max) {
                     continue;
                 }
 #pragma unroll
                 for (int m = g; m < g + G; ++m) {
                     const int nx = nxa + (m - g);
                     const int n2 = nx * nx + nyz2;
-                    if (n2 == 0 || n2 > M * M) continue;
+                    if (n2 == 0 || n2 > op.n2_max) continue;
                     const int bin = (bin_all >= 0) ? bin_all : op.bin_of[n2];
                     if (bin < 0) continue;
                     const C vv = v[0][m], uu = cross ? u[0][m] : vv;
@@ -1028,11 +1033,11 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, OP_NEW
 
 // =============================================================== launchers
 template <typename T, int LOGN>
-cudaError_t z_r2c_n(const T* in, cplx<T>* out, int rows, cudaStream_t st, double sub = 0.0) {
+cudaError_t z_r2c_n(const T* in, cplx<T>* out, int rows, cudaStream_t st, double sub, int kz_max) {
     typedef ZShape<T, LOGN> S;
     cudaError_t e = set_smem((const void*)k_z_r2c<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    k_z_r2c<T, LOGN><<<dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st>>>(in, out, (T)sub);
+    k_z_r2c<T, LOGN><<<dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st>>>(in, out, (T)sub, kz_max);
     return cudaGetLastError();
 }
 
@@ -1069,11 +1074,13 @@ cudaError_t y_grad3_n(const cplx<T>* A, const cplx<T>* B, cplx<T>* Ao, cplx<T>* 
 }
 
 template <typename T, int LOGN>
-cudaError_t forward_zy_n(const T* in, cplx<T>* spec, int batch, cudaStream_t st, double sub) {
+cudaError_t forward_zy_n(const T* in, cplx<T>* spec, int batch, cudaStream_t st, double sub, int kz_max) {
     constexpr int N = 1 << LOGN, M = N / 2;
-    cudaError_t e = z_r2c_n<T, LOGN>(in, spec, N * batch, st, sub);
+    cudaError_t e = z_r2c_n<T, LOGN>(in, spec, N * batch, st, sub, kz_max);
     if (e != cudaSuccess) return e;
-    return y_rows_n<T, LOGN, false>(spec, spec, (int64_t)batch * (M + 1) * N, st);
+    // one field: its planes up to kz_max come first
+    const int64_t planes = batch == 1 ? std::min(kz_max, M) + 1 : (int64_t)batch * (M + 1);
+    return y_rows_n<T, LOGN, false>(spec, spec, planes * N, st);
 }
 
 // A (phi after the inverse x pass) and B (-i kx phi) in the full layout; scratch holds
@@ -1217,7 +1224,7 @@ cudaError_t x_cols_kind(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp&
 
 template <typename T>
 cudaError_t z_r2c(const T* in, cplx<T>* out, int n, int batch, cudaStream_t st, double sub) {
-    PM_DISPATCH_LOGN(n, (z_r2c_n<T, LG>(in, out, n * batch, st, sub)))
+    PM_DISPATCH_LOGN(n, (z_r2c_n<T, LG>(in, out, n * batch, st, sub, n)))
 }
 
 template <typename T>
@@ -1281,8 +1288,8 @@ cudaError_t x_adj(const cplx<T>* V, cplx<T>* out, int n, double kf, double coef,
 }
 
 template <typename T>
-cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_t st, double sub) {
-    PM_DISPATCH_LOGN(n, (forward_zy_n<T, LG>(in, spec, batch, st, sub)))
+cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_t st, double sub, int kz_max) {
+    PM_DISPATCH_LOGN(n, (forward_zy_n<T, LG>(in, spec, batch, st, sub, kz_max)))
 }
 
 template <typename T>
@@ -1305,7 +1312,7 @@ cudaError_t x_cols(cplx<T>* data, cplx<T>* out2, int nplanes, int n, const SpecO
     template cudaError_t y_rows_grad3<T>(cplx<T>*, cplx<T>*, cplx<T>*, int64_t, int, double,           \
                                          cudaStream_t, const double*, int64_t);                        \
     template cudaError_t x_cols<T>(cplx<T>*, cplx<T>*, int, int, const SpecOp&, cudaStream_t);      \
-    template cudaError_t forward_zy<T>(const T*, cplx<T>*, int, int, cudaStream_t, double);             \
+    template cudaError_t forward_zy<T>(const T*, cplx<T>*, int, int, cudaStream_t, double, int);        \
     template cudaError_t x_adj<T>(const cplx<T>*, cplx<T>*, int, double, double, cudaStream_t, float*, \
                                   int64_t, const AdjGrOp*, bool);                                       \
     template cudaError_t inverse_yz_grad<T>(cplx<T>*, cplx<T>*, cplx<T>*, T* const*, int, int, double,   \

@@ -48,6 +48,7 @@ struct SpecOp {
     double* acc2 = nullptr;           // cross spectra only: the same rows for |in2|^2 (null: not wanted)
     int acc_rows = 0;                 // rows available (the x pass runs at most this many CTAs)
     int nbins = 0;
+    int n2_max = 0;                   // modes |n|^2 beyond it are in no bin (at most (n/2)^2)
     int deconv = 0;
     const void* in2 = nullptr;        // second (y-transformed) field for the cross spectrum
 };
@@ -139,9 +140,10 @@ template <typename T>
 cudaError_t fft_plane(cplx<T>* A, cplx<T>* GX, cplx<T>* GY, int nplanes, int n, const SpecOp& op, cudaStream_t st);
 
 // Forward z (r2c) and y passes of `batch` real meshes into spec ([field][kz][kx][ky]
-// before the x pass).
+// before the x pass).  kz_max: the planes beyond it are left unwritten (their modes are not wanted).
 template <typename T>
-cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_t st, double sub = 0.0);
+cudaError_t forward_zy(const T* in, cplx<T>* spec, int n, int batch, cudaStream_t st, double sub = 0.0,
+                       int kz_max = 1 << 20);
 // The three force meshes from phi and -i kx phi after the inverse x pass (A, B, full
 // layout; both overwritten): out[0] = c2r(IFFT_y(B)), out[1] = c2r(IFFT_y(-i ky A)),
 // out[2] = c2r(-i kz IFFT_y(A)); scratch holds one half spectrum per field.

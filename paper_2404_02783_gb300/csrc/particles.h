@@ -98,6 +98,11 @@ cudaError_t bk_indicators(int n, double2* out, int m, int nbins, const int16_t* 
 // unit[u] = (i, j, lb, t): the triangles (i, j, l), l in [max(j, 8 lb), min(nbins, 8 lb + 8)),
 // whose first has index t in the i <= j <= l order; acc indexed by triangle (zeroed by the caller).
 template <typename T>
-cudaError_t bk_units(const T* fields, int m, int nbins, const int4* unit, int nunit, double* acc, cudaStream_t st);
+cudaError_t bk_units(const T* fields, int64_t npoints, int nbins, const int4* unit, int nunit, double* acc,
+                     cudaStream_t st);
+// The indicator fields on one point of each orbit of the cube group (0 <= x <= y <= z <= m / 2),
+// each value times the cube root of the orbit's size, so that a triple product carries it once.
+int64_t bk_orbit_points(int m);
+cudaError_t bk_orbits(const double* fields, int m, int nbins, double* out, cudaStream_t st);
 
 }  // namespace pm
