@@ -500,6 +500,26 @@ pm_status check_edges(int nbins, const double* edges) {
     return PM_OK;
 }
 
+// Mode counts and sums of |n| per bin from the host's bin table.
+void bin_geometry(int n, const std::vector<int16_t>& tab, std::vector<double>& nm, std::vector<double>& ks) {
+    const std::vector<double>& cnt = mode_counts(n);
+    std::fill(nm.begin(), nm.end(), 0.0);
+    std::fill(ks.begin(), ks.end(), 0.0);
+    for (size_t s = 1; s < cnt.size(); ++s) {
+        const int b = tab[s];
+        if (b < 0) continue;
+        nm[b] += cnt[s];
+        ks[b] += cnt[s] * std::sqrt((double)s);
+    }
+}
+
+// Modes beyond the last edge (or the Nyquist sphere) are in no bin.
+void bin_reach(int n, int nbins, const double* edges, int* n2_max, int* kz_max) {
+    const double last = std::min(edges[nbins], n / 2.0);
+    *n2_max = (int)std::floor(last * last);
+    *kz_max = (int)std::floor(last);
+}
+
 // p2_out (with field2 only): the auto spectrum of field2 from the same pass.
 template <typename T>
 pm_status power_t(pm_ctx* c, const void* field, const void* field2, int nbins, const double* edges, int deconv,
@@ -509,9 +529,8 @@ pm_status power_t(pm_ctx* c, const void* field, const void* field2, int nbins, c
     if (!f1) PM_TRY(current_density(c, &f1));
     void* s0 = c->at(c->L.spec[0]);
     void* s1 = c->at(c->L.spec[1]);
-    // modes beyond the last edge (or the Nyquist sphere) are in no bin: their kz planes are not made
-    const double last = std::min(edges[nbins], n / 2.0);
-    const int n2_max = (int)std::floor(last * last), kz_max = (int)std::floor(last);
+    int n2_max, kz_max;  // the kz planes that no bin reaches are not made
+    bin_reach(n, nbins, edges, &n2_max, &kz_max);
     PM_TRY(forward_to_y<T>(c, f1, s0, n, field ? 0.0 : kDensityMean, kz_max));
     if (field2) PM_TRY(forward_to_y<T>(c, field2, s1, n, 0.0, kz_max));
     std::vector<int16_t> tab;
@@ -542,14 +561,8 @@ pm_status power_t(pm_ctx* c, const void* field, const void* field2, int nbins, c
     if (two) PM_CK(bin_rows_sum(rows2, nrows, nbins, acc + nbins, c->st));
     // mode counts and mean |k| per bin follow from the geometry alone: summed on the host while
     // the device transforms and bins (the copy below waits for it)
-    const std::vector<double>& cnt = mode_counts(n);
-    std::vector<double> nm(nbins, 0.0), ks(nbins, 0.0);
-    for (size_t s = 1; s < cnt.size(); ++s) {
-        const int b = tab[s];
-        if (b < 0) continue;
-        nm[b] += cnt[s];
-        ks[b] += cnt[s] * std::sqrt((double)s);
-    }
+    std::vector<double> nm(nbins), ks(nbins);
+    bin_geometry(n, tab, nm, ks);
     std::vector<double> h((two ? 2 : 1) * nbins);
     PM_CK(cudaMemcpyAsync(h.data(), acc, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->st));
     PM_CK(cudaStreamSynchronize(c->st));
@@ -1852,6 +1865,17 @@ pm_status batch_validate(const pm_config* cfg, int B, const double* boxes) {
     return PM_OK;
 }
 
+// The counting density of every realisation on its rho, unless the last update left it there.
+pm_status batch_density(pm_batch* b) {
+    if (b->rho_valid) return PM_OK;
+    const size_t n = b->cfg.nmesh;
+    PM_CK(cudaMemsetAsync(b->at(b->RHO), 0, sizeof(float) * b->B * n * n * n, b->st));
+    PM_CK(deposit_lattice(b->at(b->X), b->cfg.np, PM_FP32_FIXED, b->cfg.nmesh,
+                          std::pow((double)b->cfg.nmesh / b->cfg.np, 3), b->at(b->RHO), b->st, b->B));
+    b->rho_valid = true;
+    return PM_OK;
+}
+
 // Force meshes of realisations r0 .. r0 + c - 1 from their rho (one launch per pass).
 pm_status batch_forces(pm_batch* b, cudaStream_t s, int r0, int c) {
     const int n = b->cfg.nmesh, M = n / 2;
@@ -2137,10 +2161,7 @@ pm_status pm_batch_step(pm_batch* b, int n_steps, int use_graph) {
     if (n_steps < 0) return fail(PM_ERR_INVALID_ARG, "negative step count");
     if (b->step + n_steps > b->cfg.n_steps) return fail(PM_ERR_STATE, "stepping past a_final");
     if (n_steps == 0) return PM_OK;
-    if (!b->rho_valid) {
-        for (int r = 0; r < b->B; ++r) PM_TRY(deposit_particles(b->views[r], b->at(b->views[r]->L.rho)));
-        b->rho_valid = true;
-    }
+    PM_TRY(batch_density(b));
     if (!use_graph) {
         for (int k = 0; k < n_steps; ++k) PM_TRY(batch_enqueue_step(b, b->st));
         return PM_OK;
@@ -2215,7 +2236,8 @@ pm_status pm_batch_autotune(pm_batch* b, int* chunk_out, double* ms_out) {
         void* zero[3] = {v->at(v->L.force[0]), v->at(v->L.force[0]), v->at(v->L.force[0])};
         PM_CK(ic_place(v->at(v->L.x), v->at(v->L.p), zero, v->np, PM_FP32_FIXED, 0.0, 0.0, v->cfg.box, b->st));
     }
-    for (int r = 0; r < b->B; ++r) PM_TRY(deposit_particles(b->views[r], b->at(b->views[r]->L.rho)));
+    b->rho_valid = false;
+    PM_TRY(batch_density(b));
     PM_CK(cudaEventRecord(b->ev_in, b->st));
     PM_CK(cudaStreamWaitEvent(b->cap, b->ev_in, 0));
     batch_drop_graph(b);
@@ -2287,12 +2309,58 @@ pm_status pm_batch_state(pm_batch* b, int* step, double* a, int* synchronised) {
 pm_status pm_batch_power(pm_batch* b, int nbins, const double* edges, int deconvolve, double* k_out, double* p_out,
                          double* nmodes_out) {
     if (!b) return fail(PM_ERR_INVALID_ARG, "null batch");
+    PM_TRY(check_edges(nbins, edges));
+    // one launch a pass over a group of realisations (one realisation at a time took ten launches
+    // of a few microseconds and two synchronisations each)
+    const int n = b->cfg.nmesh, M = n / 2;
+    const size_t n3 = (size_t)n * n * n, nspec = (size_t)(M + 1) * n * n;
+    // deposited afresh: a caller may hold views and have written their particles
+    b->rho_valid = false;
+    PM_TRY(batch_density(b));
+    b->rho_valid = false;
+    std::vector<int16_t> tab;
+    PM_TRY(upload_bin_table(b->views[0], nbins, edges, &tab));
+    SpecOp op;
+    op.kind = OP_BIN;
+    op.fwd = 1;
+    op.kf = b->views[0]->kf;  // the binning works on integer modes
+    op.bin_of = (const int16_t*)b->at(b->BIN);
+    op.wtab = (const double*)b->at(b->WTAB);
+    op.nbins = nbins;
+    op.deconv = deconvolve ? 1 : 0;
+    int kz_max;
+    bin_reach(n, nbins, edges, &op.n2_max, &kz_max);
+    std::vector<double> nm(nbins), ks(nbins), h((size_t)b->B * nbins);
+    // the z pass's grid takes n rows a realisation in its y dimension
+    const int group = std::min(b->B, 65535 / n);
+    for (int r0 = 0; r0 < b->B; r0 += group) {
+        const int c = std::min(group, b->B - r0);
+        float2* s0 = (float2*)b->at(b->SPEC[0]);
+        PM_CK(forward_zy<float>((const float*)b->at(b->RHO) + r0 * n3, s0, n, c, b->st, kDensityMean));
+        // rows of bin sums in the third spectrum array (free here), the totals after them
+        double* rows = (double*)b->at(b->SPEC[2]);
+        op.bin_fields = c;
+        op.acc_rows = std::max(1, std::min(4 * num_sms() / c + 1, (int)(nspec * 8 / (sizeof(double) * nbins)) - 1));
+        op.acc = rows;
+        double* total = rows + (size_t)c * op.acc_rows * nbins;
+        PM_CK(cudaMemsetAsync(rows, 0, sizeof(double) * c * op.acc_rows * nbins, b->st));
+        PM_CK(x_cols<float>(s0, nullptr, kz_max + 1, n, op, b->st));
+        PM_CK(bin_rows_sum(rows, op.acc_rows, nbins, total, b->st, c));
+        PM_CK(cudaMemcpyAsync(h.data() + (size_t)r0 * nbins, total, sizeof(double) * c * nbins, cudaMemcpyDeviceToHost,
+                              b->st));
+    }
+    bin_geometry(n, tab, nm, ks);
+    PM_CK(cudaStreamSynchronize(b->st));
+    const double n6 = std::pow((double)n, 6);
     for (int r = 0; r < b->B; ++r) {
-        pm_ctx* v = nullptr;
-        PM_TRY(pm_batch_context(b, r, &v));
-        PM_TRY(pm_power(v, nullptr, nullptr, nbins, edges, deconvolve, k_out ? k_out + (size_t)r * nbins : nullptr,
-                        p_out ? p_out + (size_t)r * nbins : nullptr,
-                        nmodes_out ? nmodes_out + (size_t)r * nbins : nullptr));
+        const pm_ctx* v = b->views[r];
+        const double V = v->cfg.box * v->cfg.box * v->cfg.box;
+        for (int q = 0; q < nbins; ++q) {
+            const size_t o = (size_t)r * nbins + q;
+            if (nmodes_out) nmodes_out[o] = nm[q];
+            if (p_out) p_out[o] = nm[q] > 0 ? V / n6 * h[o] / nm[q] : NAN;
+            if (k_out) k_out[o] = nm[q] > 0 ? v->kf * ks[q] / nm[q] : NAN;
+        }
     }
     return PM_OK;
 }

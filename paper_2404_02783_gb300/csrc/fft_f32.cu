@@ -28,6 +28,8 @@ __global__ void k_sum_rows(const double* __restrict__ rows, int nrows, int nbins
     const int lane = threadIdx.x & 31;
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b >= nbins) return;  // whole warps leave together
+    rows += (size_t)blockIdx.y * nrows * nbins;
+    out += (size_t)blockIdx.y * nbins;
     double s = 0.0;
     for (int r = lane; r < nrows; r += 32) s += rows[(size_t)r * nbins + b];
 #pragma unroll
@@ -35,9 +37,9 @@ __global__ void k_sum_rows(const double* __restrict__ rows, int nrows, int nbins
     if (lane == 0) out[b] = s;
 }
 
-cudaError_t bin_rows_sum(const double* rows, int nrows, int nbins, double* out, cudaStream_t st) {
+cudaError_t bin_rows_sum(const double* rows, int nrows, int nbins, double* out, cudaStream_t st, int nfields) {
     if (nbins <= 0) return cudaSuccess;
-    k_sum_rows<<<(nbins + 7) / 8, 256, 0, st>>>(rows, nrows, nbins, out);
+    k_sum_rows<<<dim3((nbins + 7) / 8, nfields), 256, 0, st>>>(rows, nrows, nbins, out);
     return cudaGetLastError();
 }
 

@@ -453,7 +453,7 @@ __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx,
 // Registers of the x passes: kinds that hold a second sequence (phi beside its transform, or
 // the second field of a cross spectrum) take twice the data registers.
 template <typename T, int LOGN, int KIND> struct XRes {
-    static constexpr bool TWO = KIND != OP_FWD_STORE && KIND != OP_INV && KIND != OP_POTENTIAL;
+    static constexpr bool TWO = KIND != OP_FWD_STORE && KIND != OP_INV && KIND != OP_POTENTIAL && KIND != OP_BIN;
     static constexpr int DATA = plan_e(1 << LOGN) * 2 * (int)sizeof(T) / 4 * (TWO ? 2 : 1);  // registers
     static constexpr int REGS = DATA <= 32 ? 64 : DATA <= 64 ? 104 : DATA <= 128 ? 168 : 255;
     static constexpr int MINB = 65536 / (REGS * XShape<T, LOGN>::THREADS);
@@ -473,20 +473,23 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
     C* buf = reinterpret_cast<C*>(smem_raw);
     // OP_BIN: 1 / W^2 of the CIC window per |n_j| (W per axis from the FP64 table), in T
     T* iw2 = reinterpret_cast<T*>(buf + S::COL);
-    const bool cross = (KIND == OP_BIN) && op.in2 != nullptr;
+    constexpr bool BIN = KIND == OP_BIN || KIND == OP_BIN_CROSS, cross = KIND == OP_BIN_CROSS;
     const int tid = threadIdx.x;
     const int b = tid % CB, t = tid / CB;
     const int64_t nblk = (int64_t)nplanes * NCG;
     const auto tw = tw_plan<T, N>();
     CtaColEx<C, E, CB> ex{buf + b};
-    if constexpr (KIND == OP_BIN) {
+    if constexpr (BIN) {
         for (int e = tid; e <= M; e += S::THREADS) iw2[e] = op.deconv ? T(1.0 / (op.wtab[e] * op.wtab[e])) : T(1);
         __syncthreads();
     }
-    // OP_BIN: this CTA's row of per-bin sums in global memory (zeroed by the caller)
-    double* acc_row = (KIND == OP_BIN) ? op.acc + (size_t)blockIdx.x * op.nbins : nullptr;
+    // OP_BIN: this CTA's row of per-bin sums in global memory (zeroed by the caller); blockIdx.y
+    // selects one of several fields, whose rows follow one another
+    const size_t row = (size_t)blockIdx.y * op.acc_rows + blockIdx.x;
+    double* acc_row = BIN ? op.acc + row * op.nbins : nullptr;
+    if constexpr (BIN) data += (size_t)blockIdx.y * (M + 1) * N * N;
     // with a cross spectrum, optionally the auto spectrum of the second field in the same pass
-    double* acc2_row = (KIND == OP_BIN && cross && op.acc2) ? op.acc2 + (size_t)blockIdx.x * op.nbins : nullptr;
+    double* acc2_row = (cross && op.acc2) ? op.acc2 + row * op.nbins : nullptr;
 #pragma unroll 1
     for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
         const int plane = (int)(blk / NCG);
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
         const double kf = op.kf_arr ? op.kf_arr[field] : op.kf;
         const int c = (int)(blk % NCG) * CB + b;
         const size_t pbase = (size_t)plane * N * N;
-        if constexpr (KIND == OP_BIN) {
+        if constexpr (BIN) {
             // every mode of the block beyond the last bin (a fifth of them with the whole sphere)
             const int c0 = c - b, ymin = c0 < M ? c0 : N - c0 - CB + 1;
             if (ymin * ymin + kz * kz > op.n2_max) continue;
@@ -527,9 +530,9 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
         }
         const int ny = (c < M) ? c : c - N;
         const int nyz2 = ny * ny + kz * kz;
-        if constexpr (KIND == OP_BIN) {
-            C u[1][E];
-            if (cross) {
+        if constexpr (BIN) {
+            C u[1][cross ? E : 1];
+            if constexpr (cross) {
                 const C* in2 = reinterpret_cast<const C*>(op.in2) + pbase + c;
 #pragma unroll
                 for (int m = 0; m < E; ++m) u[0][m] = in2[(size_t)(t + m * Q) * N];
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
                 for (int m = 0; m < E; ++m) w[m] = ex.put(t, m);
             };
             regroup(v[0]);
-            if (cross) regroup(u[0]);
+            if constexpr (cross) regroup(u[0]);
             // The thread's modes kx = E t .. E t + E - 1 lie on one side of the Nyquist index, so
             // |n|^2 is monotone over them, and a bin is a contiguous range of |n|^2: when the first
             // and the last mode of a group of eight fall in the same bin (neither the zero mode nor
@@ -579,10 +582,10 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
                     if (n2 == 0 || n2 > op.n2_max) continue;
                     const int bin = (bin_all >= 0) ? bin_all : op.bin_of[n2];
                     if (bin < 0) continue;
-                    const C vv = v[0][m], uu = cross ? u[0][m] : vv;
+                    const C vv = v[0][m], uu = u[0][cross ? m : 0];
                     // w |delta_n|^2 / W^2 (or the cross product), w = 1 on the kz = 0, n/2 planes, 2 elsewhere
                     const T wgt = iw2[nx < 0 ? -nx : nx] * wyz;
-                    const T val = (vv.x * uu.x + vv.y * uu.y) * wgt;
+                    const T val = (cross ? vv.x * uu.x + vv.y * uu.y : vv.x * vv.x + vv.y * vv.y) * wgt;
                     const T val2 = acc2_row ? (uu.x * uu.x + uu.y * uu.y) * wgt : T(0);
                     if (bin != run_bin) {
                         if (run_bin >= 0) {
@@ -1105,18 +1108,19 @@ cudaError_t inverse_yz_grad_n(cplx<T>* A, cplx<T>* B, cplx<T>* scratch, T* const
 template <typename T, int LOGN, int KIND>
 cudaError_t x_cols_n(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp& op, cudaStream_t st) {
     typedef XShape<T, LOGN> S;
-    const size_t smem = sizeof(cplx<T>) * S::COL + (KIND == OP_BIN ? sizeof(T) * (S::N / 2 + 1) : 0);
+    const size_t smem = sizeof(cplx<T>) * S::COL + (op.kind == OP_BIN ? sizeof(T) * (S::N / 2 + 1) : 0);
     const void* fn = (const void*)k_x_cols<T, LOGN, KIND>;
     cudaError_t e = set_smem(fn, smem);
     if (e != cudaSuccess) return e;
     int64_t grid = (int64_t)nplanes * (S::N / S::CB);
-    if (KIND == OP_BIN) {  // one row of bin sums per CTA
+    if (op.kind == OP_BIN) {  // one row of bin sums per CTA
         int per_sm = 1;
         e = resident_ctas(fn, S::THREADS, smem, &per_sm);
         if (e != cudaSuccess) return e;
         grid = std::min<int64_t>(grid, std::min<int64_t>((int64_t)per_sm * num_sms(), op.acc_rows));
     }
-    k_x_cols<T, LOGN, KIND><<<(unsigned)grid, S::THREADS, smem, st>>>(data, out2, op, nplanes);
+    k_x_cols<T, LOGN, KIND><<<dim3((unsigned)grid, op.kind == OP_BIN ? op.bin_fields : 1), S::THREADS, smem, st>>>(
+        data, out2, op, nplanes);
     return cudaGetLastError();
 }
 
@@ -1204,7 +1208,9 @@ cudaError_t x_cols_kind(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp&
         case OP_NEWTON: return x_cols_n<T, LOGN, OP_NEWTON>(data, out2, nplanes, op, st);
         case OP_GR: return x_cols_n<T, LOGN, OP_GR>(data, out2, nplanes, op, st);
         case OP_ZA: return x_cols_n<T, LOGN, OP_ZA>(data, out2, nplanes, op, st);
-        case OP_BIN: return x_cols_n<T, LOGN, OP_BIN>(data, out2, nplanes, op, st);
+        case OP_BIN:
+            return op.in2 ? x_cols_n<T, LOGN, OP_BIN_CROSS>(data, out2, nplanes, op, st)
+                          : x_cols_n<T, LOGN, OP_BIN>(data, out2, nplanes, op, st);
         case OP_POTENTIAL: return x_cols_n<T, LOGN, OP_POTENTIAL>(data, out2, nplanes, op, st);
         default: return cudaErrorInvalidValue;
     }

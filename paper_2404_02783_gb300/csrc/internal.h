@@ -17,7 +17,8 @@ enum OpKind {
     OP_GR = 3,         // linearised Poisson-gauge constraint, same outputs, updates Phi_old
     OP_ZA = 4,         // Zel'dovich displacement potential from unit phases, same outputs
     OP_BIN = 5,        // power-spectrum binning (auto or cross), no output
-    OP_POTENTIAL = 6   // Newtonian potential only: IFFT_x(phi)
+    OP_POTENTIAL = 6,  // Newtonian potential only: IFFT_x(phi)
+    OP_BIN_CROSS = 7   // the instance of OP_BIN with a second field (SpecOp::in2)
 };
 
 // Per-mode filter of OP_ZA (the same three-output gradient chain serves the Zel'dovich
@@ -46,7 +47,8 @@ struct SpecOp {
     const double* wtab = nullptr;     // CIC sinc^2(pi m / n) for m = 0..n/2
     double* acc = nullptr;            // [acc_rows][nbins]: per-CTA sums of w |delta|^2 / W^2 (zeroed)
     double* acc2 = nullptr;           // cross spectra only: the same rows for |in2|^2 (null: not wanted)
-    int acc_rows = 0;                 // rows available (the x pass runs at most this many CTAs)
+    int acc_rows = 0;                 // rows available a field (the x pass runs at most this many CTAs for it)
+    int bin_fields = 1;               // OP_BIN: fields back to back, nplanes planes of each binned
     int nbins = 0;
     int n2_max = 0;                   // modes |n|^2 beyond it are in no bin (at most (n/2)^2)
     int deconv = 0;
@@ -98,8 +100,9 @@ cudaError_t x_cols(cplx<T>* data, cplx<T>* out2, int nplanes, int n, const SpecO
 // tab[s] = bin of |n|^2 = s for s <= nmax from the squared edges e2[0..nbins] (device),
 // e2[b] <= s < e2[b+1], the last edge closed, -1 outside.
 cudaError_t bin_table(int16_t* tab, int64_t nmax, const double* e2, int nbins, cudaStream_t st);
-// out[b] = sum_r rows[r nbins + b] in row order (deterministic), r < nrows.
-cudaError_t bin_rows_sum(const double* rows, int nrows, int nbins, double* out, cudaStream_t st);
+// out[f nbins + b] = sum_r rows[(f nrows + r) nbins + b] in row order (deterministic), r < nrows,
+// for each of nfields fields.
+cudaError_t bin_rows_sum(const double* rows, int nrows, int nbins, double* out, cudaStream_t st, int nfields = 1);
 // Transposed force chain on the x pass (adjoint): V holds the three y-transformed spectra
 // of the deposited adjoint momenta back to back; out = IFFT_x[sum_j i k_j c(k) FFT_x V_j]
 // with c = coef / (kf^2 |n|^2).  Also sets zero[0 .. nzero) to 0 (a buffer the caller is

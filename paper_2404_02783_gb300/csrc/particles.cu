@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restric
     }
 }
 
+// blockIdx.y selects the field of a batch (particles [field][3][np^3], meshes [field][n^3]).
 template <int R, int XC>
 __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restrict__ x, int lognp, int logn,
                                                        float inv_cell_ticks, float mass, float* __restrict__ rho) {
@@ -67,6 +68,8 @@ __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restric
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
     uint32_t* carry = tile_words + D::CELLS;
+    x += (int64_t)blockIdx.y * 3 << (3 * lognp);
+    rho += (int64_t)blockIdx.y << (3 * logn);
     const int ntz = (1 << lognp) / D::TZ, nty = (1 << lognp) / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
@@ -113,6 +116,8 @@ __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __rest
     extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
     uint32_t* lo = tile_words;
     uint32_t* carry = tile_words + D::CELLS;
+    x += (int64_t)blockIdx.y * 3 << (3 * lognp);
+    rho += (int64_t)blockIdx.y << (3 * logn);
     const int np = 1 << lognp;
     const int64_t count = (int64_t)1 << (3 * lognp);
     const int ntz = np / D::TZ, nty = np / D::TY;
@@ -175,7 +180,7 @@ static unsigned grid_for(int64_t count, int threads) {
 }
 
 template <int R, int XC>
-static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, void* rho, cudaStream_t st) {
+static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, void* rho, cudaStream_t st, int nfields) {
     typedef DepTile<R, XC> D;
     const int lognp = ilog2(np), logn = ilog2(n);
     const unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
@@ -187,27 +192,31 @@ static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, vo
     }();
     cudaError_t e = set_smem_once((const void*)fn, smem);
     if (e != cudaSuccess) return e;
-    fn<<<blocks, 512, smem, st>>>((const uint32_t*)x, lognp, logn, inv, (float)mass, (float*)rho);
+    fn<<<dim3(blocks, nfields), 512, smem, st>>>((const uint32_t*)x, lognp, logn, inv, (float)mass, (float*)rho);
     return cudaGetLastError();
 }
 template <int R>
-static cudaError_t deposit_tiled(const void* x, int np, int n, double mass, void* rho, cudaStream_t st) {
-    switch (tile_depth(R, np, 1)) {
-        case 4: return deposit_tiled_r<R, 4>(x, np, n, mass, rho, st);
-        case 8: return deposit_tiled_r<R, 8>(x, np, n, mass, rho, st);
-        default: return deposit_tiled_r<R, 16>(x, np, n, mass, rho, st);
+static cudaError_t deposit_tiled(const void* x, int np, int n, double mass, void* rho, cudaStream_t st, int nfields) {
+    switch (tile_depth(R, np, nfields)) {
+        case 4: return deposit_tiled_r<R, 4>(x, np, n, mass, rho, st, nfields);
+        case 8: return deposit_tiled_r<R, 8>(x, np, n, mass, rho, st, nfields);
+        default: return deposit_tiled_r<R, 16>(x, np, n, mass, rho, st, nfields);
     }
 }
 
-cudaError_t deposit_lattice(const void* x, int np, int precision, int n, double mass, void* rho, cudaStream_t st) {
+cudaError_t deposit_lattice(const void* x, int np, int precision, int n, double mass, void* rho, cudaStream_t st,
+                            int nfields) {
     const int R = n / np;
-    if ((uintptr_t)rho % 16 != 0) return deposit(x, (int64_t)np * np * np, precision, n, mass, rho, st);
     // the tile box (16 + 4) x (16 + 4) x (32 + 8) cells must fit in the mesh without overlapping itself
-    const bool tiled = precision == PM_FP32_FIXED && n >= 64 && (R == 1 || R == 2 || R == 4) && np >= 32 / R;
-    if (!tiled) return deposit(x, (int64_t)np * np * np, precision, n, mass, rho, st);
-    if (R == 1) return deposit_tiled<1>(x, np, n, mass, rho, st);
-    if (R == 2) return deposit_tiled<2>(x, np, n, mass, rho, st);
-    return deposit_tiled<4>(x, np, n, mass, rho, st);
+    const bool tiled = precision == PM_FP32_FIXED && n >= 64 && (R == 1 || R == 2 || R == 4) && np >= 32 / R &&
+                       (uintptr_t)rho % 16 == 0;
+    if (!tiled) {
+        if (nfields != 1) return cudaErrorInvalidValue;
+        return deposit(x, (int64_t)np * np * np, precision, n, mass, rho, st);
+    }
+    if (R == 1) return deposit_tiled<1>(x, np, n, mass, rho, st, nfields);
+    if (R == 2) return deposit_tiled<2>(x, np, n, mass, rho, st, nfields);
+    return deposit_tiled<4>(x, np, n, mass, rho, st, nfields);
 }
 
 cudaError_t deposit(const void* x, int64_t count, int precision, int n, double mass, void* rho,
