@@ -952,8 +952,15 @@ __global__ void __launch_bounds__(PlaneShape<T, LOGN>::THREADS, PlaneShape<T, LO
 // back along x into out ([kz][x][ky], ready for the inverse y and z passes).  GR: the
 // Poisson-gauge operator of AdjGrOp instead of c(k), with the carried spectrum gr.Z.  FD (the
 // first-order gradient): V is one scalar field and W = FFT_x V, without the i k_j factors.
+// Registers: the sum, the field and (AHEAD) the next one.
+template <typename T, int LOGN> struct AdjRes {
+    static constexpr int DATA = plan_e(1 << LOGN) * 2 * (int)sizeof(T) / 4;
+    static constexpr int REGS = DATA <= 16 ? 96 : DATA <= 32 ? 160 : DATA <= 64 ? 168 : 255;
+    static constexpr int MINB = 65536 / (REGS * XShape<T, LOGN>::THREADS);
+};
+
 template <typename T, int LOGN, bool GR, bool FD>
-__global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, OP_NEWTON>::MINB)
+__global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, AdjRes<T, LOGN>::MINB)
     k_x_adj(const cplx<T>* V, cplx<T>* out, double kf, double coef, float4* __restrict__ zero, int64_t nzero4,
             AdjGrOp gr) {
     typedef cplx<T> C;
@@ -979,12 +986,27 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, OP_NEW
     const T kzT = (kz == M) ? T(0) : kfT * T(kz);
     C acc[1][E];
     CtaColEx<C, E, CB> ex{reinterpret_cast<C*>(smem_raw) + b};
-#pragma unroll 1
-    for (int j = 0; j < (FD ? 1 : 3); ++j) {
-        C v[1][E];
-        const C* col = V + j * field + pbase + c;
+    // with 16 elements or fewer a thread, the next field is loaded while this one is transformed
+    constexpr bool AHEAD = !FD && E * sizeof(C) <= 128;
+    C v[1][E];
+    const C* col = V + pbase + c;
+    if constexpr (AHEAD) {
 #pragma unroll
         for (int m = 0; m < E; ++m) v[0][m] = col[(size_t)(t + m * Q) * N];
+    }
+#pragma unroll 1
+    for (int j = 0; j < (FD ? 1 : 3); ++j) {
+        C nx[AHEAD ? E : 1];
+        if constexpr (!AHEAD) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[0][m] = col[j * field + (size_t)(t + m * Q) * N];
+        }
+        if constexpr (AHEAD) {
+            if (j < 2) {
+#pragma unroll
+                for (int m = 0; m < E; ++m) nx[m] = col[(j + 1) * field + (size_t)(t + m * Q) * N];
+            }
+        }
         fft_regs<N, 1, false>(v, t, tw, ex);
 #pragma unroll
         for (int m = 0; m < E; ++m) {
@@ -993,6 +1015,10 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, OP_NEW
             const T kj = FD ? T(1) : (j == 0) ? ((2 * nx == -N) ? T(0) : kfT * T(nx)) : (j == 1 ? kyT : kzT);
             const C a = j == 0 ? cmake<C>(T(0), T(0)) : acc[0][m];
             acc[0][m] = cmake<C>(a.x + kj * v[0][m].x, a.y + kj * v[0][m].y);
+        }
+        if constexpr (AHEAD) {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[0][m] = nx[m];
         }
     }
     if constexpr (GR) {
