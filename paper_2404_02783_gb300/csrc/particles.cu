@@ -23,21 +23,50 @@
 namespace pm {
 
 // ---------------------------------------------------------------- CIC decode (FP64 fractions)
+// Base node, its neighbour and the two weights along one axis of s = x n - 1/2 (n = 2^logn).
+// FP64 arithmetic bounds the FP64 particle kernels (its pipe is 84-87% busy), so for x n >= 1 the
+// decode is done on the bits: x n is its mantissa shifted into units of 2^-52, where subtracting
+// 1/2 and splitting off the fraction are exact, as they are in FP64, and two FP64 subtractions
+// give the weights.  The first half cell, and positions outside [0, 1), take the arithmetic form.
 struct CicD {
     int i0, i1;
-    double w1;
+    double w0, w1;
 };
-__device__ __forceinline__ CicD cic_frac(double x, int n) {
+// (Out of line, so that its FP64 instructions are not issued for the others' predicates.)
+__device__ __noinline__ CicD cic_frac_general(double x, int n) {
+    CicD c;
     const double s = x * (double)n - 0.5;
     const double fl = floor(s);
-    CicD c;
     c.w1 = s - fl;
+    c.w0 = 1.0 - c.w1;
     c.i0 = ((int)fl) & (n - 1);
     c.i1 = (c.i0 + 1) & (n - 1);
     return c;
 }
+__device__ __forceinline__ CicD cic_frac(double x, int logn) {
+    const int n = 1 << logn;
+    CicD c;
+    const long long bits = __double_as_longlong(x);
+    const int e = (int)(bits >> 52) - 1023 + logn;  // exponent of x n (the sign makes it large)
+    if ((unsigned)e < (unsigned)logn) {
+        const long long m = bits & 0xfffffffffffffll;
+        const long long v = ((m | (1ll << 52)) << e) - (1ll << 51);
+        c.i0 = (int)(v >> 52);
+        const double d = __longlong_as_double((v & 0xfffffffffffffll) | 0x3ff0000000000000ll);  // 1 + fraction
+        c.w1 = d - 1.0;
+        c.w0 = 2.0 - d;
+        c.i1 = (c.i0 + 1) & (n - 1);
+    } else {
+        c = cic_frac_general(x, n);
+    }
+    return c;
+}
 
 // ---------------------------------------------------------------- deposit
+// Particles in any order.  Bound by the L2's atomic operations: with V4 (rho 16-byte aligned) the
+// two z corners of a row go in one vector reduction when they share an aligned group of four
+// cells (three rows in four), its other lanes adding 0.
+template <bool V4>
 __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restrict__ x, int64_t count, int logn,
                                                        float inv_cell_ticks, float mass, float* __restrict__ rho) {
     const size_t n = (size_t)1 << logn;
@@ -48,15 +77,29 @@ __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restric
         const CicF cz = cic_ticks(x[2 * count + i], logn, inv_cell_ticks);
         const float wx[2] = {1.0f - cx.w1, cx.w1}, wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};
         const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
+        const int pos = cz.i0 & 3;
+        if (V4 && pos != 3) {
+            const float4 z = make_float4(pos == 0 ? wz[0] : 0.f, pos == 0 ? wz[1] : pos == 1 ? wz[0] : 0.f,
+                                         pos == 1 ? wz[1] : pos == 2 ? wz[0] : 0.f, pos == 2 ? wz[1] : 0.f);
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+            for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const float wab = mass * wx[a] * wy[b];
-                float* row = rho + ((size_t)ix[a] * n + iy[b]) * n;
-                atomicAdd(row + iz[0], wab * wz[0]);
-                atomicAdd(row + iz[1], wab * wz[1]);
-            }
+                for (int b = 0; b < 2; ++b) {
+                    const float wab = mass * wx[a] * wy[b];
+                    red_add_v4(rho + ((size_t)ix[a] * n + iy[b]) * n + (cz.i0 - pos),
+                               make_float4(wab * z.x, wab * z.y, wab * z.z, wab * z.w));
+                }
+        } else {
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const float wab = mass * wx[a] * wy[b];
+                    float* row = rho + ((size_t)ix[a] * n + iy[b]) * n;
+                    atomicAdd(row + iz[0], wab * wz[0]);
+                    atomicAdd(row + iz[1], wab * wz[1]);
+                }
+        }
     }
 }
 
@@ -152,23 +195,64 @@ __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __rest
     });
 }
 
-__global__ void k_deposit_frac(const double* __restrict__ x, int64_t count, int n, double mass,
+__global__ void k_deposit_frac(const double* __restrict__ x, int64_t count, int logn, double mass,
                                double* __restrict__ rho) {
+    const size_t n = (size_t)1 << logn;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const CicD cx = cic_frac(x[i], n), cy = cic_frac(x[count + i], n), cz = cic_frac(x[2 * count + i], n);
-        const double wx[2] = {1.0 - cx.w1, cx.w1}, wy[2] = {1.0 - cy.w1, cy.w1}, wz[2] = {1.0 - cz.w1, cz.w1};
-        const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
+        CicD cx = cic_frac(x[i], logn);
+        const CicD cy = cic_frac(x[count + i], logn), cz = cic_frac(x[2 * count + i], logn);
+        if (mass != 1.0) cx.w0 *= mass, cx.w1 *= mass;
+        const double wx[2] = {cx.w0, cx.w1}, wy[2] = {cy.w0, cy.w1};
+        const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const double wab = mass * wx[a] * wy[b];
+                const double wab = wx[a] * wy[b];
                 double* row = rho + ((size_t)ix[a] * n + iy[b]) * n;
-                atomicAdd(row + iz[0], wab * wz[0]);
-                atomicAdd(row + iz[1], wab * wz[1]);
+                atomicAdd(row + cz.i0, wab * cz.w0);
+                atomicAdd(row + cz.i1, wab * cz.w1);
             }
     }
+}
+
+// The np^3 = n^3 lattice-ordered particles of a context: a thread walks a lattice row along x in
+// runs of `run` and carries the upper plane's weights to the next particle, which usually starts
+// one cell further: 4 atomics a particle instead of 8 (the FP64 atomics bound the plain form).
+__global__ void __launch_bounds__(256) k_deposit_frac_rows(const double* __restrict__ x, int logn, int run,
+                                                           double* __restrict__ rho) {
+    const int n = 1 << logn;
+    const int64_t count = (int64_t)1 << (3 * logn), xstride = (int64_t)1 << (2 * logn);
+    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lx0 = (int)(gid >> (2 * logn)) * run;
+    if (lx0 >= n) return;
+    int64_t i = ((int64_t)lx0 << (2 * logn)) + (gid & (xstride - 1));
+    uint32_t next = 0xffffffffu, o[4] = {0u, 0u, 0u, 0u};  // the carried plane's cell and corners
+    double W[4];
+#pragma unroll 1
+    for (int k = 0; k < run; ++k, i += xstride) {
+        const CicD cx = cic_frac(x[i], logn), cy = cic_frac(x[count + i], logn), cz = cic_frac(x[2 * count + i], logn);
+        const uint32_t yz = ((uint32_t)cy.i0 << logn) | (uint32_t)cz.i0;
+        const bool merge = (((uint32_t)cx.i0 << (2 * logn)) | yz) == next;
+        if (!merge && next != 0xffffffffu) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) atomicAdd(rho + o[q], W[q]);
+        }
+        next = ((uint32_t)cx.i1 << (2 * logn)) | yz;
+        const double wy[2] = {cy.w0, cy.w1}, wz[2] = {cz.w0, cz.w1};
+        const uint32_t iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1}, iz[2] = {(uint32_t)cz.i0, (uint32_t)cz.i1};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double w = wy[q >> 1] * wz[q & 1];
+            const double lower = merge ? fma(cx.w0, w, W[q]) : cx.w0 * w;
+            atomicAdd(rho + ((((uint32_t)cx.i0 << logn) + iy[q >> 1]) << logn) + iz[q & 1], lower);
+            W[q] = cx.w1 * w;
+            o[q] = ((((uint32_t)cx.i1 << logn) + iy[q >> 1]) << logn) + iz[q & 1];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) atomicAdd(rho + o[q], W[q]);
 }
 
 static unsigned grid_for(int64_t count, int threads) {
@@ -212,6 +296,14 @@ cudaError_t deposit_lattice(const void* x, int np, int precision, int n, double 
                        (uintptr_t)rho % 16 == 0;
     if (!tiled) {
         if (nfields != 1) return cudaErrorInvalidValue;
+        if (precision == PM_FP64 && R == 1 && mass == 1.0) {
+            // rows of 16 while they still give every SM two blocks
+            int run = 16;
+            while (run > 1 && (int64_t)np * np * np / run < 2 * 256 * (int64_t)num_sms()) run /= 2;
+            k_deposit_frac_rows<<<(unsigned)((int64_t)np * np * (np / run) / 256), 256, 0, st>>>(
+                (const double*)x, ilog2(n), run, (double*)rho);
+            return cudaGetLastError();
+        }
         return deposit(x, (int64_t)np * np * np, precision, n, mass, rho, st);
     }
     if (R == 1) return deposit_tiled<1>(x, np, n, mass, rho, st, nfields);
@@ -225,16 +317,16 @@ cudaError_t deposit(const void* x, int64_t count, int precision, int n, double m
     const int logn = ilog2(n);
     if (precision == PM_FP32_FIXED) {
         const float inv = (float)ldexp(1.0, -(32 - logn));
-        k_deposit_ticks<<<grid_for(count, 256), 256, 0, st>>>((const uint32_t*)x, count, logn, inv, (float)mass,
-                                                              (float*)rho);
+        const auto fn = (uintptr_t)rho % 16 == 0 ? k_deposit_ticks<true> : k_deposit_ticks<false>;
+        fn<<<grid_for(count, 256), 256, 0, st>>>((const uint32_t*)x, count, logn, inv, (float)mass, (float*)rho);
     } else {
-        k_deposit_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)x, count, n, mass, (double*)rho);
+        k_deposit_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)x, count, logn, mass, (double*)rho);
     }
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- interpolation
-template <typename T, typename X, int ROWS = 1>
+template <typename T>
 __device__ __forceinline__ T gather8(const T* __restrict__ f, size_t n, const int* ix, const int* iy,
                                      const int* iz, const T* wx, const T* wy, const T* wz) {
     T acc = T(0);
@@ -242,12 +334,15 @@ __device__ __forceinline__ T gather8(const T* __restrict__ f, size_t n, const in
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const T* row = f + ((size_t)ix[a] * n + iy[b]) * n * ROWS;
+            const T* row = f + ((size_t)ix[a] * n + iy[b]) * n;
             acc += wx[a] * wy[b] * (wz[0] * __ldg(row + iz[0]) + wz[1] * __ldg(row + iz[1]));
         }
     return acc;
 }
 
+// V4 (field 16-byte aligned): a row's two z corners come in one 16-byte load when they share an
+// aligned group of four cells, which saves requests to L2.
+template <bool V4>
 __global__ void k_interp_ticks(const float* __restrict__ f, int logn, const uint32_t* __restrict__ x,
                                int64_t count, float inv_cell_ticks, float* __restrict__ out) {
     const size_t n = (size_t)1 << logn;
@@ -258,18 +353,39 @@ __global__ void k_interp_ticks(const float* __restrict__ f, int logn, const uint
         const CicF cz = cic_ticks(x[2 * count + i], logn, inv_cell_ticks);
         const float wx[2] = {1.0f - cx.w1, cx.w1}, wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};
         const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
-        out[i] = gather8<float, uint32_t>(f, n, ix, iy, iz, wx, wy, wz);
+        if constexpr (V4) {
+            const int pos = cz.i0 & 3;
+            float4 v[4];
+            float next[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float* row = f + ((size_t)ix[q >> 1] * n + iy[q & 1]) * n;
+                v[q] = __ldg(reinterpret_cast<const float4*>(row + (cz.i0 - pos)));
+                next[q] = pos == 3 ? __ldg(row + cz.i1) : 0.f;
+            }
+            float acc = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float f0 = pos == 0 ? v[q].x : pos == 1 ? v[q].y : pos == 2 ? v[q].z : v[q].w;
+                const float f1 = pos == 0 ? v[q].y : pos == 1 ? v[q].z : pos == 2 ? v[q].w : next[q];
+                acc += wx[q >> 1] * wy[q & 1] * (wz[0] * f0 + wz[1] * f1);
+            }
+            out[i] = acc;
+        } else {
+            out[i] = gather8<float>(f, n, ix, iy, iz, wx, wy, wz);
+        }
     }
 }
 
-__global__ void k_interp_frac(const double* __restrict__ f, int n, const double* __restrict__ x, int64_t count,
+__global__ void k_interp_frac(const double* __restrict__ f, int logn, const double* __restrict__ x, int64_t count,
                               double* __restrict__ out) {
+    const size_t n = (size_t)1 << logn;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const CicD cx = cic_frac(x[i], n), cy = cic_frac(x[count + i], n), cz = cic_frac(x[2 * count + i], n);
-        const double wx[2] = {1.0 - cx.w1, cx.w1}, wy[2] = {1.0 - cy.w1, cy.w1}, wz[2] = {1.0 - cz.w1, cz.w1};
+        const CicD cx = cic_frac(x[i], logn), cy = cic_frac(x[count + i], logn), cz = cic_frac(x[2 * count + i], logn);
+        const double wx[2] = {cx.w0, cx.w1}, wy[2] = {cy.w0, cy.w1}, wz[2] = {cz.w0, cz.w1};
         const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
-        out[i] = gather8<double, double>(f, (size_t)n, ix, iy, iz, wx, wy, wz);
+        out[i] = gather8<double>(f, n, ix, iy, iz, wx, wy, wz);
     }
 }
 
@@ -279,10 +395,10 @@ cudaError_t interp(const void* field, int n, const void* x, int64_t count, int p
     const int logn = ilog2(n);
     if (precision == PM_FP32_FIXED) {
         const float inv = (float)ldexp(1.0, -(32 - logn));
-        k_interp_ticks<<<grid_for(count, 256), 256, 0, st>>>((const float*)field, logn, (const uint32_t*)x, count,
-                                                             inv, (float*)out);
+        const auto fn = (uintptr_t)field % 16 == 0 ? k_interp_ticks<true> : k_interp_ticks<false>;
+        fn<<<grid_for(count, 256), 256, 0, st>>>((const float*)field, logn, (const uint32_t*)x, count, inv, (float*)out);
     } else {
-        k_interp_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)field, n, (const double*)x, count,
+        k_interp_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)field, logn, (const double*)x, count,
                                                             (double*)out);
     }
     return cudaGetLastError();
@@ -336,17 +452,26 @@ __global__ void __launch_bounds__(256) k_ikd_ticks2(uint32_t* __restrict__ x, fl
     }
 }
 
+// A box fraction wrapped into [0, 1): the integer part is only taken off when there is one (out
+// of line, as above).
+__device__ __noinline__ double minus_floor(double x) { return x - floor(x); }
+__device__ __forceinline__ double wrap_fraction(double x) {
+    if ((unsigned)__double2hiint(x) >= 0x3ff00000u) x = minus_floor(x);
+    return x;
+}
+
 template <bool FD>
 __global__ void __launch_bounds__(256) k_ikd_frac(double* __restrict__ x, double* __restrict__ p, int64_t count,
-                                                  int n, const double* __restrict__ g, double kick, double drift_box,
+                                                  int logn, const double* __restrict__ g, double kick, double drift_box,
                                                   double inv_d) {
+    const size_t n = (size_t)1 << logn;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
         double xs[3] = {x[i], x[count + i], x[2 * count + i]};
-        const CicD cx = cic_frac(xs[0], n), cy = cic_frac(xs[1], n), cz = cic_frac(xs[2], n);
-        const double wx[2] = {1.0 - cx.w1, cx.w1}, wy[2] = {1.0 - cy.w1, cy.w1}, wz[2] = {1.0 - cz.w1, cz.w1};
+        const CicD cx = cic_frac(xs[0], logn), cy = cic_frac(xs[1], logn), cz = cic_frac(xs[2], logn);
+        const double wx[2] = {cx.w0, cx.w1}, wy[2] = {cy.w0, cy.w1}, wz[2] = {cz.w0, cz.w1};
         const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
-        double f[3];
+        double f[3] = {0.0, 0.0, 0.0};
         if constexpr (FD) {
             double P[2][4];
 #pragma unroll
@@ -358,16 +483,24 @@ __global__ void __launch_bounds__(256) k_ikd_frac(double* __restrict__ x, double
             fd1_force<double>(P[0], P[1], wx[0], wx[1], wy, wz, inv_d, f[0], f[1], f[2]);
         } else {
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
-                f[j] = gather8<double, double, kForceRows>(g + j * n, (size_t)n, ix, iy, iz, wx, wy, wz);
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const double wab = wx[a] * wy[b];
+                    const double* row = g + ((size_t)ix[a] * n + iy[b]) * n * kForceRows;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const double w = wab * wz[c];
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) f[j] = fma(w, __ldg(row + j * n + iz[c]), f[j]);
+                    }
+                }
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             const double pj = p[j * count + i] + kick * f[j];
             p[j * count + i] = pj;
-            double xj = xs[j] + drift_box * pj;
-            xj -= floor(xj);
-            x[j * count + i] = xj;
+            x[j * count + i] = wrap_fraction(xs[j] + drift_box * pj);
         }
     }
 }
@@ -388,7 +521,7 @@ static cudaError_t interp_kick_drift_t(void* x, void* p, int64_t count, int prec
             k_ikd_ticks<FD><<<grid_for(count, 256), 256, 0, st>>>((uint32_t*)x, (float*)p, count, logn, inv,
                                                                   (const float*)g, (float)kick, dt, (float)inv_d);
     } else {
-        k_ikd_frac<FD><<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, count, n, (const double*)g, kick,
+        k_ikd_frac<FD><<<grid_for(count, 256), 256, 0, st>>>((double*)x, (double*)p, count, logn, (const double*)g, kick,
                                                              drift / box, inv_d);
     }
     return cudaGetLastError();
@@ -914,6 +1047,7 @@ __global__ void k_disp_ticks(const uint32_t* __restrict__ x, float* __restrict__
         for (int j = 0; j < 3; ++j) d[j * count + i] = (float)(int32_t)(x[j * count + i] - q[j]) * tick_mpc;
     }
 }
+__device__ __noinline__ double minus_rint(double x) { return x - rint(x); }
 __global__ void k_disp_frac(const double* __restrict__ x, double* __restrict__ d, int lognp, double box) {
     const int64_t count = (int64_t)1 << (3 * lognp);
     const int mask = (1 << lognp) - 1;
@@ -922,8 +1056,10 @@ __global__ void k_disp_frac(const double* __restrict__ x, double* __restrict__ d
         const int q[3] = {(int)((i >> (2 * lognp)) & mask), (int)((i >> lognp) & mask), (int)(i & mask)};
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const double v = x[j * count + i] - q[j] * inv_np;
-            d[j * count + i] = (v - rint(v)) * box;
+            // the nearest image is only looked for beyond half the box
+            double v = fma((double)q[j], -inv_np, x[j * count + i]);  // q inv_np is exact
+            if (!(((unsigned)__double2hiint(v) & 0x7fffffffu) < 0x3fe00000u)) v = minus_rint(v);
+            d[j * count + i] = v * box;
         }
     }
 }
@@ -964,8 +1100,9 @@ cudaError_t positions_mpc(const void* x, void* out, int64_t count, int precision
 __global__ void k_count_outside(const double* __restrict__ x, int64_t count, unsigned long long* __restrict__ bad) {
     unsigned long long mine = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = x[i];
-        mine += (v >= 0.0 && v < 1.0) ? 0ull : 1ull;  // false for NaN: counted
+        // 0 <= v < 1 on the bits (not the FP64 pipe): -0 passes, NaN does not
+        const unsigned long long v = __double_as_longlong(x[i]);
+        mine += ((unsigned)(v >> 32) < 0x3ff00000u || (v << 1) == 0) ? 0ull : 1ull;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
@@ -981,7 +1118,6 @@ cudaError_t count_outside_box(const double* x, int64_t count, unsigned long long
 // ---------------------------------------------------------------- cell keys and stable order
 __global__ void k_cell_keys(const void* __restrict__ xv, int64_t count, int precision, int logn, float inv_cell_ticks,
                             uint32_t* __restrict__ keys, uint32_t* __restrict__ counts) {
-    const int n = 1 << logn;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
         int b[3];
@@ -990,7 +1126,7 @@ __global__ void k_cell_keys(const void* __restrict__ xv, int64_t count, int prec
             for (int j = 0; j < 3; ++j) b[j] = cic_ticks(x[j * count + i], logn, inv_cell_ticks).i0;
         } else {
             const double* x = (const double*)xv;
-            for (int j = 0; j < 3; ++j) b[j] = cic_frac(x[j * count + i], n).i0;
+            for (int j = 0; j < 3; ++j) b[j] = cic_frac(x[j * count + i], logn).i0;
         }
         const uint32_t key = ((uint32_t)b[0] << (2 * logn)) | ((uint32_t)b[1] << logn) | (uint32_t)b[2];
         keys[i] = key;
@@ -1080,6 +1216,21 @@ __global__ void k_scatter_unstable(const uint32_t* __restrict__ keys, int64_t co
         order[atomicAdd(&cursor[keys[i]], 1u)] = (uint32_t)i;
 }
 
+// Sorts at most MAX distinct ids: loaded together, each placed by the number of smaller ones.
+template <uint32_t MAX>
+__device__ __forceinline__ void sort_in_registers(uint32_t* a, uint32_t len) {
+    uint32_t v[MAX];
+#pragma unroll
+    for (uint32_t k = 0; k < MAX; ++k) v[k] = k < len ? a[k] : 0xffffffffu;
+#pragma unroll
+    for (uint32_t k = 0; k < MAX; ++k) {
+        uint32_t rank = 0;
+#pragma unroll
+        for (uint32_t m = 0; m < MAX; ++m) rank += v[m] < v[k] ? 1u : 0u;
+        if (k < len) a[rank] = v[k];
+    }
+}
+
 // Within each cell the ids were placed in arbitrary order; sort them ascending
 // (Shell sort with gaps 1, 4, 13, ...), which makes the whole order stable in id.
 __global__ void k_sort_buckets(const uint32_t* __restrict__ start, const uint32_t* __restrict__ cursor, int64_t ncell,
@@ -1089,6 +1240,14 @@ __global__ void k_sort_buckets(const uint32_t* __restrict__ start, const uint32_
         const uint32_t len = e - s;
         if (len < 2) continue;
         uint32_t* a = order + s;
+        if (len <= 8) {
+            sort_in_registers<8>(a, len);
+            continue;
+        }
+        if (len <= 16) {
+            sort_in_registers<16>(a, len);
+            continue;
+        }
         uint32_t gap = 1;
         while (gap < len / 3) gap = 3 * gap + 1;
         for (; gap > 0; gap /= 3)
