@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "dfloat.cuh"
 #include "fft.cuh"
@@ -401,25 +402,56 @@ __device__ __forceinline__ void gr_modes(const SpecOp& op, cplx<T>* v, int t, in
     }
 }
 
-// The Zel'dovich filter of a mode n2 > 0 (ZaFilter): FP64 for the FP64 path; for FP32 the same
-// value from pairs of FP32 numbers (an FP64 divide a mode made the pass 1.8 ms at 512^3).
-template <typename T>
-__device__ __forceinline__ T za_filter(const SpecOp& op, int n2, int field, double kf) {
-    if (op.za_filter == ZA_IDENTITY) return T(op.coef);
-    const double c = div_mode<double>(op.coef, kf * kf);
-    if constexpr (sizeof(T) == 8) {
-        if (op.za_filter == ZA_INV_LAPLACE) return c / (double)n2;
-        return c * (static_cast<const double*>(op.amp) + (int64_t)field * op.amp_stride)[n2] / (double)n2;
-    } else {
-        df v = df_of(c);
-        if (op.za_filter != ZA_INV_LAPLACE) v = v * (static_cast<const df*>(op.amp) + (int64_t)field * op.amp_stride)[n2];
-        return round_df(df_div(v, (float)(n2 > 0 ? n2 : 1)));
+// The Zel'dovich filter (ZaFilter) on a thread's E modes kx = t + m Q of the x pass, in place:
+// FP64 for the FP64 path; for FP32 the same value from pairs of FP32 numbers (an FP64 divide a mode
+// made the pass 1.8 ms at 512^3), the amplitudes of eight modes loaded ahead of their use.
+template <typename T, int N, int E, int Q>
+__device__ __forceinline__ void za_modes(const SpecOp& op, cplx<T>* v, int t, int ny, int nz, int field, double kf) {
+    typedef cplx<T> C;
+    constexpr int M = N / 2, G = E < 8 ? E : 8;
+    const int nyz2 = ny * ny + nz * nz;
+    const bool nyq_yz = (2 * ny == -N) || (nz == M);
+    const double c = op.za_filter == ZA_IDENTITY ? op.coef : op.coef / (kf * kf);
+    const df cf = df_of(c);
+    const int64_t tab = (int64_t)field * op.amp_stride;
+#pragma unroll
+    for (int m0 = 0; m0 < E; m0 += G) {
+        typename std::conditional<sizeof(T) == 8, double, df>::type amp[G];
+        if (op.za_filter == ZA_AMP) {
+#pragma unroll
+            for (int m = 0; m < G; ++m) {
+                const int nx = (2 * (m0 + m) < E) ? t + (m0 + m) * Q : t + (m0 + m) * Q - N;
+                if constexpr (sizeof(T) == 8) amp[m] = __ldg(static_cast<const double*>(op.amp) + tab + nx * nx + nyz2);
+                else {
+                    const float2 p = __ldg(static_cast<const float2*>(op.amp) + tab + nx * nx + nyz2);
+                    amp[m] = df{p.x, p.y};
+                }
+            }
+        }
+#pragma unroll
+        for (int m = m0; m < m0 + G; ++m) {
+            const int nx = (2 * m < E) ? t + m * Q : t + m * Q - N;
+            const int n2 = nx * nx + nyz2;
+            C g = v[m];
+            if (op.fixed_amp) {  // keep the phase, set |g| = 1
+                const T r2 = g.x * g.x + g.y * g.y;
+                g = (r2 > T(0)) ? cscale(g, rsqrt(r2)) : cmake<C>(T(0), T(0));
+            }
+            T filt;
+            if (op.za_filter == ZA_IDENTITY) {
+                filt = T(c);
+            } else if constexpr (sizeof(T) == 8) {
+                filt = (op.za_filter == ZA_AMP ? c * amp[m - m0] : c) / (double)n2;
+            } else {
+                filt = round_df(df_div(op.za_filter == ZA_AMP ? cf * amp[m - m0] : cf, (float)(n2 > 0 ? n2 : 1)));
+            }
+            v[m] = (n2 == 0 || nyq_yz || 2 * nx == -N) ? cmake<C>(T(0), T(0)) : cscale(g, filt);
+        }
     }
 }
 
 // The per-mode operator of the x pass on mode (nx, ny, nz), |n|^2 = n2, of field `field`:
-// the Newtonian Green's function (or the potential alone), the Zel'dovich filter, or the
-// linearised Poisson-gauge constraint (which reads and updates its Phi history at `old` and,
+// the Newtonian Green's function (or the potential alone), or the linearised Poisson-gauge constraint (which reads and updates its Phi history at `old` and,
 // for |n| <= n_lo, the FP64 island).  Returns phi for the mode.
 template <typename T, int KIND, int N>
 __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx, int ny, int nz, int n2, int field,
@@ -429,14 +461,6 @@ __device__ __forceinline__ cplx<T> mode_op(const SpecOp& op, cplx<T> vv, int nx,
     C phi;
     if constexpr (KIND == OP_NEWTON || KIND == OP_POTENTIAL) {
         phi = (n2 == 0) ? cmake<C>(T(0), T(0)) : cscale(vv, div_mode(coefT, T(n2)));
-    } else if constexpr (KIND == OP_ZA) {
-        const bool nyq = (2 * nx == -N) || (2 * ny == -N) || (nz == M);
-        C g = vv;
-        if (op.fixed_amp) {  // keep the phase, set |g| = 1
-            const T r2 = g.x * g.x + g.y * g.y;
-            g = (r2 > T(0)) ? cscale(g, rsqrt(r2)) : cmake<C>(T(0), T(0));
-        }
-        phi = (n2 == 0 || nyq) ? cmake<C>(T(0), T(0)) : cscale(g, za_filter<T>(op, n2, field, kf));
     } else {  // OP_GR
         if (n2 <= op.n_lo * op.n_lo) {
             phi = gr_island_mode<T>(op, vv, nx, ny, nz, n2, field, kf);
@@ -615,6 +639,8 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
             if constexpr (KIND == OP_GR) {
                 gr_modes<T, N, E, Q>(op, v[0], t, ny, kz, field, kf, kf2T,
                                      reinterpret_cast<C*>(op.phi_old) + pbase + c);
+            } else if constexpr (KIND == OP_ZA) {
+                za_modes<T, N, E, Q>(op, v[0], t, ny, kz, field, kf);
             } else {
 #pragma unroll
                 for (int m = 0; m < E; ++m) {

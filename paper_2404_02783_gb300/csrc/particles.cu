@@ -544,9 +544,12 @@ struct TickScale {
     df f;
     double d;
 };
+__device__ __noinline__ uint32_t wrapped_ticks(float p1, double s1, float p2, double s2) {
+    return (uint32_t)__double2ll_rn((double)p1 * s1 + (double)p2 * s2);
+}
 __device__ __forceinline__ uint32_t disp_ticks(float ps, const TickScale& s) {
     df v = two_prod(ps, s.f.h);
-    if (!(fabsf(v.h) < 1073741824.0f)) return (uint32_t)__double2ll_rn((double)ps * s.d);
+    if (!(fabsf(v.h) < 1073741824.0f)) return wrapped_ticks(ps, s.d, 0.0f, 0.0);
     v.l = fmaf(ps, s.f.l, v.l);
     return (uint32_t)df2int_rn(v);
 }
@@ -557,7 +560,7 @@ __device__ __forceinline__ uint32_t disp_ticks(float p1, const TickScale& s1, fl
     b.l = fmaf(p2, s2.f.l, b.l);
     const df v = a + b;
     if (!(fabsf(a.h) < 1073741824.0f && fabsf(b.h) < 1073741824.0f && fabsf(v.h) < 1073741824.0f))
-        return (uint32_t)__double2ll_rn((double)p1 * s1.d + (double)p2 * s2.d);
+        return wrapped_ticks(p1, s1.d, p2, s2.d);
     return (uint32_t)df2int_rn(v);
 }
 static TickScale tick_scale(double d) { return TickScale{df_of(d), d}; }
