@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* __restrict__ x
                                                   float K, float Km, float drift_next, float* __restrict__ lam_u) {
     const int n = 1 << logn;
     const float nf = (float)n;
+    launch_next();
+    wait_previous();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t nx0 = 0, nx1 = 0, nx2 = 0;
@@ -218,6 +220,8 @@ __global__ void __launch_bounds__(256) k_deposit_vec_rows(const uint32_t* __rest
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lz = (int)(gid & (np - 1)), ly = (int)((gid >> lognp) & (np - 1));
     const int lx0 = (int)(gid >> (2 * lognp)) * run;
+    launch_next();
+    wait_previous();
     if (lx0 >= np) return;
     const int64_t xstride = (int64_t)1 << (2 * lognp);
     const int64_t id0 = (((int64_t)lx0 << lognp) + ly) * np + lz;
@@ -377,9 +381,8 @@ cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v
                                const float* rho_bar, float K, float Km, float drift_next, float* lam_u,
                                cudaStream_t st) {
     const int logn = ilog2(n);
-    k_adj_kick<<<blocks_for(count), 256, 0, st>>>(x, count, logn, (float)ldexp(1.0, -(32 - logn)), v, G,
-                                                  rho_bar, K, Km, drift_next, lam_u);
-    return cudaGetLastError();
+    return launch_chained(k_adj_kick, dim3(blocks_for(count)), 256, 0, st, x, count, logn, (float)ldexp(1.0, -(32 - logn)), v,
+                          G, rho_bar, K, Km, drift_next, lam_u);
 }
 
 cudaError_t deposit_grad(const uint32_t* x, int64_t count, int n, const float* v, double inv_d, float* V,
@@ -409,11 +412,8 @@ cudaError_t deposit_vec(const uint32_t* x, int np, int n, const float* v, float*
     const int64_t threads = (int64_t)np * np * (np / run);
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     const float inv = (float)ldexp(1.0, -(32 - logn));
-    if (n == np)
-        k_deposit_vec_rows<true><<<blocks, 256, 0, st>>>(x, lognp, logn, run, inv, v, V[0], V[1], V[2]);
-    else
-        k_deposit_vec_rows<false><<<blocks, 256, 0, st>>>(x, lognp, logn, run, inv, v, V[0], V[1], V[2]);
-    return cudaGetLastError();
+    return launch_chained(n == np ? k_deposit_vec_rows<true> : k_deposit_vec_rows<false>, dim3(blocks), 256, 0, st, x, lognp,
+                          logn, run, inv, v, V[0], V[1], V[2]);
 }
 
 cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const float2* amp,

@@ -121,6 +121,8 @@ __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MIN
     typedef ZShape<T, LOGN> S;
     constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x;
     const int y0 = blockIdx.x * YB;
@@ -173,6 +175,8 @@ __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MIN
     typedef ZShape<T, LOGN> S;
     constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     C* buf = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x;
     const int comp = blockIdx.z;
@@ -244,6 +248,8 @@ __global__ void __launch_bounds__(YShape<T, LOGN>::THREADS, YShape<T, LOGN>::MIN
     typedef YShape<T, LOGN> S;
     constexpr int N = S::N, E = S::E, Q = S::Q;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     const int b = row_of<Q>(threadIdx.x), t = threadIdx.x % Q;
     const int64_t r = (int64_t)blockIdx.x * S::RB + b;
     const bool ok = r < nrows;
@@ -273,6 +279,8 @@ __global__ void __launch_bounds__(YShape<T, LOGN>::THREADS, YShape<T, LOGN>::MIN
     typedef YShape<T, LOGN> S;
     constexpr int N = S::N, E = S::E, Q = S::Q;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     const int b = row_of<Q>(threadIdx.x), t = threadIdx.x % Q;
     const int64_t r = (int64_t)blockIdx.x * S::RB + b;
     const bool ok = r < nrows;
@@ -494,6 +502,8 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
     constexpr int N = S::N, M = N / 2, E = S::E, Q = S::Q, CB = S::CB;
     constexpr int NCG = N / CB;  // column groups per plane
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     C* buf = reinterpret_cast<C*>(smem_raw);
     // OP_BIN: 1 / W^2 of the CIC window per |n_j| (W per axis from the FP64 table), in T
     T* iw2 = reinterpret_cast<T*>(buf + S::COL);
@@ -877,6 +887,8 @@ __global__ void __launch_bounds__(PlaneShape<T, LOGN>::THREADS, PlaneShape<T, LO
     C* P = tws + N;
     const int tid = threadIdx.x;
     load_stage_twiddles<T, N>(tws);
+    launch_next();
+    wait_previous();
 #pragma unroll 1
     for (int plane = blockIdx.x; plane < nplanes; plane += gridDim.x) {
         const size_t pbase = (size_t)plane * N * N;
@@ -993,6 +1005,8 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, AdjRes<T, LOGN>::MIN
     typedef XShape<T, LOGN> S;
     constexpr int N = S::N, M = N / 2, E = S::E, Q = S::Q, CB = S::CB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    launch_next();
+    wait_previous();
     const int tid = threadIdx.x;
     const int b = tid % CB, t = tid / CB;
     const int kz = blockIdx.y;
@@ -1092,8 +1106,7 @@ cudaError_t z_r2c_n(const T* in, cplx<T>* out, int rows, cudaStream_t st, double
     typedef ZShape<T, LOGN> S;
     cudaError_t e = set_smem((const void*)k_z_r2c<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    k_z_r2c<T, LOGN><<<dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st>>>(in, out, (T)sub, kz_max);
-    return cudaGetLastError();
+    return launch_chained(k_z_r2c<T, LOGN>, dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st, in, out, (T)sub, kz_max);
 }
 
 template <typename T, int LOGN>
@@ -1102,8 +1115,7 @@ cudaError_t z_c2r_n(const Ptr3<T>& P, int ncomp, int rows, unsigned mask, double
     typedef ZShape<T, LOGN> S;
     cudaError_t e = set_smem((const void*)k_z_c2r<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    k_z_c2r<T, LOGN><<<dim3(S::N / S::YB, rows, ncomp), S::THREADS, S::SMEM, st>>>(P, mask, (T)kf, kf_arr);
-    return cudaGetLastError();
+    return launch_chained(k_z_c2r<T, LOGN>, dim3(S::N / S::YB, rows, ncomp), S::THREADS, S::SMEM, st, P, mask, (T)kf, kf_arr);
 }
 
 template <typename T, int LOGN, bool INV>
@@ -1112,8 +1124,7 @@ cudaError_t y_rows_n(const cplx<T>* in, cplx<T>* out, int64_t nrows, cudaStream_
     cudaError_t e = set_smem((const void*)k_y_rows<T, LOGN, INV>, S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t nblk = (nrows + S::RB - 1) / S::RB;
-    k_y_rows<T, LOGN, INV><<<(unsigned)nblk, S::THREADS, S::SMEM, st>>>(in, out, nrows);
-    return cudaGetLastError();
+    return launch_chained(k_y_rows<T, LOGN, INV>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, in, out, nrows);
 }
 
 template <typename T, int LOGN>
@@ -1123,9 +1134,8 @@ cudaError_t y_grad3_n(const cplx<T>* A, const cplx<T>* B, cplx<T>* Ao, cplx<T>* 
     cudaError_t e = set_smem((const void*)k_y_grad3<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t nblk = (nrows + S::RB - 1) / S::RB;
-    k_y_grad3<T, LOGN><<<(unsigned)nblk, S::THREADS, S::SMEM, st>>>(A, B, Ao, Bo, Co, nrows, (T)kf, kf_arr,
-                                                                    rows_per_field);
-    return cudaGetLastError();
+    return launch_chained(k_y_grad3<T, LOGN>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, A, B, Ao, Bo, Co, nrows, (T)kf,
+                          kf_arr, rows_per_field);
 }
 
 template <typename T, int LOGN>
@@ -1171,9 +1181,8 @@ cudaError_t x_cols_n(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp& op
         if (e != cudaSuccess) return e;
         grid = std::min<int64_t>(grid, std::min<int64_t>((int64_t)per_sm * num_sms(), op.acc_rows));
     }
-    k_x_cols<T, LOGN, KIND><<<dim3((unsigned)grid, op.kind == OP_BIN ? op.bin_fields : 1), S::THREADS, smem, st>>>(
-        data, out2, op, nplanes);
-    return cudaGetLastError();
+    return launch_chained(k_x_cols<T, LOGN, KIND>, dim3((unsigned)grid, op.kind == OP_BIN ? op.bin_fields : 1), S::THREADS,
+                          smem, st, data, out2, op, nplanes);
 }
 
 template <typename T, int LOGN, int THREADS>
@@ -1222,10 +1231,8 @@ cudaError_t plane_n(cplx<T>* A, cplx<T>* GX, cplx<T>* GY, int nplanes, const Spe
     if (e != cudaSuccess) return e;
     const int grid = (int)std::min<int64_t>((int64_t)per_sm * num_sms(), nplanes);
     if (op.kind == OP_GR)
-        k_plane<T, LOGN, OP_GR><<<grid, SH::THREADS, SH::SMEM, st>>>(A, GX, GY, op, nplanes);
-    else
-        k_plane<T, LOGN, OP_NEWTON><<<grid, SH::THREADS, SH::SMEM, st>>>(A, GX, GY, op, nplanes);
-    return cudaGetLastError();
+        return launch_chained(k_plane<T, LOGN, OP_GR>, dim3(grid), SH::THREADS, SH::SMEM, st, A, GX, GY, op, nplanes);
+    return launch_chained(k_plane<T, LOGN, OP_NEWTON>, dim3(grid), SH::THREADS, SH::SMEM, st, A, GX, GY, op, nplanes);
 }
 
 template <typename T, int LOGN, bool GR, bool FD>
@@ -1235,9 +1242,8 @@ cudaError_t x_adj_k(const cplx<T>* V, cplx<T>* out, double kf, double coef, floa
     const size_t smem = sizeof(cplx<T>) * S::COL;
     cudaError_t e = set_smem((const void*)k_x_adj<T, LOGN, GR, FD>, smem);
     if (e != cudaSuccess) return e;
-    k_x_adj<T, LOGN, GR, FD><<<dim3(S::N / S::CB, S::N / 2 + 1), S::THREADS, smem, st>>>(
-        V, out, kf, coef, (float4*)zero, zero ? nzero / 4 : 0, gr);
-    return cudaGetLastError();
+    return launch_chained(k_x_adj<T, LOGN, GR, FD>, dim3(S::N / S::CB, S::N / 2 + 1), S::THREADS, smem, st, V, out, kf, coef,
+                          (float4*)zero, zero ? nzero / 4 : 0, gr);
 }
 
 template <typename T, int LOGN>

@@ -282,6 +282,7 @@ static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, vo
 template <int R>
 static cudaError_t deposit_tiled(const void* x, int np, int n, double mass, void* rho, cudaStream_t st, int nfields) {
     switch (tile_depth(R, np, nfields)) {
+        case 2: return deposit_tiled_r<R, R == 4 ? 4 : 2>(x, np, n, mass, rho, st, nfields);
         case 4: return deposit_tiled_r<R, 4>(x, np, n, mass, rho, st, nfields);
         case 8: return deposit_tiled_r<R, 8>(x, np, n, mass, rho, st, nfields);
         default: return deposit_tiled_r<R, 16>(x, np, n, mass, rho, st, nfields);

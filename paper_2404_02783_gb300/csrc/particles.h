@@ -20,7 +20,7 @@ cudaError_t interp(const void* field, int n, const void* x, int64_t count, int p
 // fd_inv_d > 0: first-order gradient (g is the potential, a plain mesh), inv_d = n / L.
 cudaError_t interp_kick_drift(void* x, void* p, int64_t count, int precision, int n, const void* g, double kick,
                               double drift, double box, cudaStream_t st, double fd_inv_d = 0.0);
-// x extent in mesh cells (16, 8 or 4) of the Lagrangian deposit tiles of nfields lattices.
+// x extent in mesh cells (16, 8, 4 or 2) of the Lagrangian deposit tiles of nfields lattices.
 int tile_depth(int R, int np, int nfields);
 // Kick + drift of the np^3 lattice-ordered particles fused with the deposit of the
 // drifted positions into rho (which must be zero on entry); FP32 ticks, n / np in {1,2,4}.

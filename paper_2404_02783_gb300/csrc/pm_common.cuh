@@ -8,6 +8,32 @@
 
 namespace pm {
 
+// ------------------------------------------------------------------ launches that overlap their ramps
+// The kernels of a step are launched so that each may start while the one before it on the stream
+// drains (programmatic dependent launch): launch_next lets the next one in, and wait_previous
+// holds this one until the kernels before it are complete and their writes visible.  Every such
+// kernel calls it before its first access to global memory, so the order of the stream holds;
+// kernels launched in the ordinary way see the whole of it as before.  On small meshes, where a
+// step is six kernels of a few microseconds, the ramps are a good part of the time: a step took
+// 33.4 us at 32^3 and takes 22.2, 77.5 and 71.0 at 128^3, 470 and 453 at 256^3, 3848 and 3834 at 512^3.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... K, typename... A>
+cudaError_t launch_chained(void (*fn)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, K(args)...);
+}
+
 // ------------------------------------------------------------------ type traits
 template <typename T> struct CT;
 template <> struct CT<float> { typedef float2 type; };

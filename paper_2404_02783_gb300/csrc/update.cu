@@ -39,12 +39,14 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restri
         g += fb * (FD ? 1 : kForceRows) * n3;
         rho += fb * n3;
     }
-    const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
     constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
+    launch_next();
     tile_zero<D::CELLS>(lo);
+    wait_previous();
     __syncthreads();
+    const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
     auto pid = [&](int e) -> int64_t {
         const int lz = e % D::TZ, ly = (e / D::TZ) % D::TY, lx = e / (D::TZ * D::TY);
         return ((((int64_t)(bx * D::TX + lx) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
@@ -127,12 +129,14 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
         g += fb * ROWS * count;
         rho += fb * count;
     }
-    const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
     constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int ox = bx * D::TX - D::H, oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
+    launch_next();
     tile_zero<D::CELLS>(lo);
+    wait_previous();
     __syncthreads();
+    const float drift_ticks = (float)(drift * (scale_arr ? scale_arr[blockIdx.y] : scale0));
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
     const int64_t id0 = ((((int64_t)(bx * D::TX) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
     constexpr int64_t xstride = (int64_t)1 << (2 * LOGN);
@@ -256,10 +260,9 @@ cudaError_t ikd_launch(const UpdateArgs& a) {
     }();
     cudaError_t e = set_smem_once((const void*)fn, smem);
     if (e != cudaSuccess) return e;
-    fn<<<dim3(blocks, a.nfields), 512, smem, a.st>>>((const uint32_t*)a.x, (uint32_t*)a.xo, (float*)a.p,
-                                                     (const float*)a.g, (float)a.kick, a.drift, a.scale0, a.scale_arr,
-                                                     (float)a.mass, (float*)a.rho, (float)a.inv_d);
-    return cudaGetLastError();
+    return launch_chained(fn, dim3(blocks, a.nfields), 512, smem, a.st, (const uint32_t*)a.x, (uint32_t*)a.xo, (float*)a.p,
+                          (const float*)a.g, (float)a.kick, a.drift, a.scale0, a.scale_arr, (float)a.mass, (float*)a.rho,
+                          (float)a.inv_d);
 }
 
 // Meshes of 128^3 and up always fill the SMs with tiles of depth 16.
@@ -268,6 +271,7 @@ cudaError_t ikd_sized(int n, int np, const UpdateArgs& a) {
     switch (n) {
         case 64:
             switch (tile_depth(R, np, a.nfields)) {
+                case 2: return ikd_launch<R, R == 4 ? 4 : 2, 6, FD>(a);  // R = 4: a lattice step is four cells
                 case 4: return ikd_launch<R, 4, 6, FD>(a);
                 case 8: return ikd_launch<R, 8, 6, FD>(a);
                 default: return ikd_launch<R, 16, 6, FD>(a);
@@ -293,12 +297,13 @@ cudaError_t ikd_any(int n, int np, const UpdateArgs& a) {
 }  // namespace
 
 // A tile of XC cells in x brings 4 of its own in halo cells, so the deepest tile is used that
-// still gives every SM one: 64^3 particles on 64^3 cells are 32 tiles of depth 16 and the update
-// takes 25.4 us, 15.5 at depth 8, 11.9 at depth 4; from 152 tiles on depth 16 is as good or
-// better (64^3 on 128^3, 256 tiles: 15.0 us against 16.1 and 18.5; 256^3: 237, 247, 269 us).
+// still gives every SM one: 64^3 particles on 64^3 cells are 32 tiles of depth 16; their update took
+// 25.4 us at depth 16, 15.5 at 8, 11.9 at 4, and a step 27.4 us at depth 4 and 22.5 at 2.  From 152
+// tiles on depth 16 is as good or better (64^3 on 128^3, 256 tiles: 15.0 us against 16.1 and 18.5 at
+// 8 and 4; 256^3: 237, 247, 269 us).
 int tile_depth(int R, int np, int nfields) {
     const int64_t tiles = (int64_t)nfields * (np * R / 16) * (np * R / 16) * (np * R / 32);  // of depth 16
-    return tiles >= num_sms() ? 16 : 2 * tiles >= num_sms() ? 8 : 4;
+    return tiles >= num_sms() ? 16 : 2 * tiles >= num_sms() ? 8 : 4 * tiles >= num_sms() ? 4 : 2;
 }
 
 bool ikd_deposit_supported(int np, int precision, int n) {
