@@ -52,13 +52,18 @@ __device__ __forceinline__ void load_stage_twiddles(cplx<T>* tw) {
     }
 }
 
-// a / d in the per-mode operators.  FP32 divides as written.  FP64 divides are slow on this
-// part, so FP64 computes the reciprocal of d by the Newton-Raphson iteration for 1/d,
-// r <- r + r (1 - d r), started from the FP32 reciprocal of d and run twice (the relative
-// error squares each time: ~2^-23, then ~2^-46, then below the FP64 rounding), and returns
-// a r.  d must lie in the FP32 normal range (about 1.2e-38 .. 3.4e38; the operators' k^2
-// and constraint denominators do).  pm_div_mode_check compares it with the division.
-template <typename T> __device__ __forceinline__ T div_mode(T a, T d) { return a / d; }
+// a / d in the per-mode operators, d positive and in the FP32 normal range (about 1.2e-38 ..
+// 3.4e38; the operators' k^2 and constraint denominators are).  The division's own instruction
+// sequence, with its check for operands out of range, is a good part of what the x pass issues a
+// mode.  FP32: the quotient by the approximate reciprocal and one Newton-Raphson correction from
+// its remainder, which leaves the rounding of the last operation.  FP64 divides are slower still:
+// the reciprocal of d by the iteration for 1/d, r <- r + r (1 - d r), started from the FP32
+// reciprocal of d and run twice (the relative error squares each time: ~2^-23, then ~2^-46, then
+// below the FP64 rounding), times a.  pm_div_mode_check compares it with the division.
+template <typename T> __device__ __forceinline__ T div_mode(T a, T d) {
+    const T r = __fdividef(1.0f, d), q = a * r;
+    return fmaf(fmaf(-q, d, a), r, q);
+}
 template <> __device__ __forceinline__ double div_mode<double>(double a, double d) {
     double r = (double)__frcp_rn((float)d);
     r = fma(r, fma(-d, r, 1.0), r);
@@ -1090,7 +1095,7 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, AdjRes<T, LOGN>::MIN
             const int i = t + m * Q;
             const int nx = (2 * m < E) ? i : i - N;
             const int n2 = nx * nx + ny * ny + kz * kz;
-            const T cc = (n2 == 0) ? T(0) : coefT / T(n2);
+            const T cc = (n2 == 0) ? T(0) : div_mode(coefT, T(n2));
             const C a = acc[0][m];
             acc[0][m] = FD ? cscale(a, cc) : cmake<C>(-cc * a.y, cc * a.x);  // (i) c sum_j k_j V_j
         }

@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(256) k_combine_blocks(uint32_t* __restrict__ x
         }
         // one x plane of the r^3 target block at a time: its r x 3 target vectors are loaded
         // before any arithmetic, so their latencies overlap instead of forming r^2 x 3 chains
-#pragma unroll 1
+#pragma unroll(r <= 2 ? 2 : 1)
         for (int ox = 0; ox < r; ++ox) {
             V v[r][3];
 #pragma unroll
