@@ -105,12 +105,10 @@ __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restric
 
 // blockIdx.y selects the field of a batch (particles [field][3][np^3], meshes [field][n^3]).
 template <int R, int XC>
-__global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restrict__ x, int lognp, int logn,
-                                                       float inv_cell_ticks, float mass, float* __restrict__ rho) {
+__global__ void __launch_bounds__(512, 3) k_deposit_tiled(const uint32_t* __restrict__ x, int lognp, int logn,
+                                                          float inv_cell_ticks, float mass, float* __restrict__ rho) {
     typedef DepTile<R, XC> D;
-    extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
-    uint32_t* lo = tile_words;
-    uint32_t* carry = tile_words + D::CELLS;
+    extern __shared__ __align__(16) uint32_t lo[];  // D::CELLS
     x += (int64_t)blockIdx.y * 3 << (3 * lognp);
     rho += (int64_t)blockIdx.y << (3 * logn);
     const int ntz = (1 << lognp) / D::TZ, nty = (1 << lognp) / D::TY;
@@ -138,12 +136,12 @@ __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restric
             nu1 = x[count + idn];
             nu2 = x[2 * count + idn];
         }
-        tile_deposit<D, false>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
+        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
     }
-    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sum, [&] {
         for (int e = threadIdx.x; e < D::PER; e += 512) {
             const int64_t id = pid(e);
-            tile_deposit<D, true>(lo, carry, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+            tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
                                   oz, quanta, sum);
         }
     });
@@ -152,13 +150,11 @@ __global__ void __launch_bounds__(512) k_deposit_tiled(const uint32_t* __restric
 // R = 1: each thread walks one lattice row of the CTA's block along x and carries the upper-x
 // plane of its CIC stencil to the next particle (the deposit half of the fused update kernel).
 template <int XC>
-__global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __restrict__ x, int lognp, int logn,
+__global__ void __launch_bounds__(512, 3) k_deposit_sweep(const uint32_t* __restrict__ x, int lognp, int logn,
                                                           float inv_cell_ticks, float mass, float* __restrict__ rho) {
     typedef DepTile<1, XC> D;
     static_assert(D::TY * D::TZ == 512, "one thread per (ly, lz); lx runs over the loop");
-    extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
-    uint32_t* lo = tile_words;
-    uint32_t* carry = tile_words + D::CELLS;
+    extern __shared__ __align__(16) uint32_t lo[];  // D::CELLS
     x += (int64_t)blockIdx.y * 3 << (3 * lognp);
     rho += (int64_t)blockIdx.y << (3 * logn);
     const int np = 1 << lognp;
@@ -186,10 +182,10 @@ __global__ void __launch_bounds__(512, 2) k_deposit_sweep(const uint32_t* __rest
         sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);
-    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sc.sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.sum, [&] {
         for (int lx = 0; lx < D::TX; ++lx) {
             const int64_t id = id0 + lx * xstride;
-            tile_deposit<D, true>(lo, carry, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+            tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
                                   oz, quanta, sc.sum);
         }
     });
@@ -269,7 +265,7 @@ static cudaError_t deposit_tiled_r(const void* x, int np, int n, double mass, vo
     const int lognp = ilog2(np), logn = ilog2(n);
     const unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
     const float inv = (float)ldexp(1.0, -(32 - logn));
-    const size_t smem = sizeof(uint32_t) * D::WORDS;
+    const size_t smem = sizeof(uint32_t) * D::CELLS;
     const auto fn = [] {
         if constexpr (R == 1) return k_deposit_sweep<XC>;
         else return k_deposit_tiled<R, XC>;

@@ -66,6 +66,20 @@ template <> __device__ __forceinline__ float2 csub<float2>(float2 a, float2 b) {
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
     return *reinterpret_cast<float2*>(&r);
 }
+// s a, and s a + c
+__device__ __forceinline__ float2 mul2(float s, float2 a) {
+    const float2 s2 = make_float2(s, s);
+    unsigned long long r, x = *reinterpret_cast<const unsigned long long*>(&s2), y = *reinterpret_cast<unsigned long long*>(&a);
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    return *reinterpret_cast<float2*>(&r);
+}
+__device__ __forceinline__ float2 fma2(float s, float2 a, float2 c) {
+    const float2 s2 = make_float2(s, s);
+    unsigned long long r, x = *reinterpret_cast<const unsigned long long*>(&s2), y = *reinterpret_cast<unsigned long long*>(&a),
+                          z = *reinterpret_cast<unsigned long long*>(&c);
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    return *reinterpret_cast<float2*>(&r);
+}
 // multiply by -i (forward) or +i (inverse)
 template <bool INV, typename C> __device__ __forceinline__ C cmul_mi(C a) {
     C c;

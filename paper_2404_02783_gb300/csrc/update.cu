@@ -27,9 +27,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restri
     constexpr int logn = LOGN, lognp = LOGN - (R == 4 ? 2 : R == 2 ? 1 : 0), np = 1 << lognp;
     constexpr int64_t count = (int64_t)1 << (3 * lognp);
     constexpr float inv_cell_ticks = 1.0f / (float)(1u << (32 - LOGN));
-    extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
-    uint32_t* lo = tile_words;
-    uint32_t* carry = tile_words + D::CELLS;
+    extern __shared__ __align__(16) uint32_t lo[];  // D::CELLS
     {
         const int64_t fb = blockIdx.y;
         constexpr int64_t n3 = (int64_t)1 << (3 * LOGN);
@@ -82,15 +80,36 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restri
         xo[id] = u0;
         xo[count + id] = u1;
         xo[2 * count + id] = u2;
-        tile_deposit<D, false>(lo, carry, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
+        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
     }
-    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sum, [&] {
         for (int e = threadIdx.x; e < D::PER; e += 512) {
             const int64_t id = pid(e);
-            tile_deposit<D, true>(lo, carry, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
+            tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
                                   oy, oz, quanta, sum);
         }
     });
+}
+
+// The second accumulation of a sweep's tile (tile_close), from the thread's written positions.
+template <int XC, int LOGN>
+__device__ __forceinline__ void sweep_again(uint32_t* lo, const uint32_t* xo, float* rho, float quanta) {
+    typedef DepTile<1, XC> D;
+    constexpr int np = 1 << LOGN, ntz = np / D::TZ, nty = np / D::TY;
+    constexpr int64_t count = (int64_t)1 << (3 * LOGN);
+    const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
+    const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
+    uint32_t sum = 0;
+    for (int lx = 0; lx < D::TX; ++lx) {
+        const int64_t id = ((((int64_t)(bx * D::TX + lx) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
+        tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], LOGN,
+                              1.0f / (float)(1u << (32 - LOGN)), bx * D::TX - D::H, by * D::TY - D::H,
+                              bz * D::TZ - D::HZ, quanta, sum);
+    }
+}
+template <int XC, int LOGN>
+__device__ __noinline__ void sweep_again_call(uint32_t* lo, const uint32_t* xo, float* rho, float quanta) {
+    sweep_again<XC, LOGN>(lo, xo, rho, quanta);
 }
 
 // x and xo may be the same array (in-place update): every particle's position is read once,
@@ -104,7 +123,10 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restri
 // particle takes the full path, so the result is the same CIC gather and deposit.
 // Bound by issue (about 70% busy) and by the latency of the gather: the upper plane's loads, which
 // every particle needs, are issued before the branch that reloads the lower plane (512^3, early
-// and clustered steps: 1742 and 1953 us; after it 1826 and 2020).  Holding the gather in flight
+// and clustered steps: 1742 and 1953 us; after it 1826 and 2020).  The components are interpolated
+// in packed pairs, and a tile without words for carries leaves the L1 cache 100 KB an SM instead of
+// 68 for the force planes that neighbouring rows share (1733 and 1946 us with both the other way,
+// 1723 and 1902 now; 2783 and 2633 at 2 Mpc/h cells, where particles have moved furthest).  Holding the gather in flight
 // across the previous particle's deposit spills at two 512-thread CTAs an SM (2293 us) and gains
 // nothing at three 256-thread CTAs (1798 and 1958).
 template <int XC, int LOGN, bool FD>
@@ -118,9 +140,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
     constexpr int logn = LOGN, np = 1 << LOGN, NC = FD ? 1 : 3, ROWS = FD ? 1 : kForceRows;
     constexpr int64_t count = (int64_t)1 << (3 * LOGN);
     constexpr float inv_cell_ticks = 1.0f / (float)(1u << (32 - LOGN));
-    extern __shared__ __align__(16) uint32_t tile_words[];  // D::WORDS
-    uint32_t* lo = tile_words;
-    uint32_t* carry = tile_words + D::CELLS;
+    extern __shared__ __align__(16) uint32_t lo[];  // D::CELLS
     {
         const int64_t fb = blockIdx.y;
         x += fb * 3 * count;
@@ -195,16 +215,16 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
                 const float Up[4] = {U[0][0], U[1][0], U[2][0], U[3][0]};
                 fd1_force<float>(Lp, Up, wx0, wx1, wy, wz, inv_d, f0, f1, f2);
             } else {
+                // along x and y on the corner pairs (b, 0), (b, 1), then along z
+                float f[3];
 #pragma unroll
-                for (int b = 0; b < 2; ++b)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const float w = wy[b] * wz[c];
-                        const int q = 2 * b + c;
-                        f0 = fmaf(w, fmaf(wx0, L[q][0], wx1 * U[q][0]), f0);
-                        f1 = fmaf(w, fmaf(wx0, L[q][1], wx1 * U[q][1]), f1);
-                        f2 = fmaf(w, fmaf(wx0, L[q][2], wx1 * U[q][2]), f2);
-                    }
+                for (int j = 0; j < 3; ++j) {
+                    const float2 t0 = fma2(wx1, make_float2(U[0][j], U[1][j]), mul2(wx0, make_float2(L[0][j], L[1][j])));
+                    const float2 t1 = fma2(wx1, make_float2(U[2][j], U[3][j]), mul2(wx0, make_float2(L[2][j], L[3][j])));
+                    const float2 t = fma2(wy[1], t1, mul2(wy[0], t0));
+                    f[j] = fmaf(wz[0], t.x, wz[1] * t.y);
+                }
+                f0 = f[0], f1 = f[1], f2 = f[2];
             }
             p0 = fmaf(kick, f0, p0);
             p1 = fmaf(kick, f1, p1);
@@ -223,12 +243,11 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
         sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);  // the carried plane of the row's last particle
-    tile_close<D>(lo, carry, rho, ox, oy, oz, logn, sc.sum, [&] {
-        for (int lx = 0; lx < D::TX; ++lx) {
-            const int64_t id = id0 + lx * xstride;
-            tile_deposit<D, true>(lo, carry, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
-                                  oy, oz, quanta, sc.sum);
-        }
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.sum, [&] {
+        // a call where the three components fill the registers (in line its values spill in the loop:
+        // 1764 us against 1724); with the potential alone the call costs more (1730 us against 1563)
+        if constexpr (FD) sweep_again<XC, LOGN>(lo, xo, rho, quanta);
+        else sweep_again_call<XC, LOGN>(lo, xo, rho, quanta);
     });
 }
 
@@ -253,7 +272,7 @@ cudaError_t ikd_launch(const UpdateArgs& a) {
     typedef DepTile<R, XC> D;
     constexpr int np = (1 << LOGN) / R;
     constexpr unsigned blocks = (unsigned)((np / D::TX) * (np / D::TY) * (np / D::TZ));
-    const size_t smem = sizeof(uint32_t) * D::WORDS;
+    const size_t smem = sizeof(uint32_t) * D::CELLS;
     const auto fn = [] {
         if constexpr (R == 1) return k_ikd_deposit_sweep<XC, LOGN, FD>;
         else return k_ikd_deposit<R, XC, LOGN, FD>;

@@ -40,9 +40,9 @@ __device__ __forceinline__ CicF cic_ticks(uint32_t u, int logn, float inv_cell_t
 // nothing; instead the sum of all cells is compared with the sum of all additions, both in 64
 // bits, before the tile is flushed: each wrap of a 32-bit cell takes exactly 2^32 from the
 // former.  A tile that fails the comparison (a cell of 256 times the mean density) is
-// accumulated again from the positions just written, with an 8-bit carry per cell caught from
-// the atomics' return values (a tile holds at most 8192 mass units, i.e. 2^37 quanta, so a
-// carry stays below 32).
+// accumulated again from the positions just written, each wrap seen in an addition's return value
+// and added to the global mesh as its 256 mass units (2^32 quanta).  A cell wraps up to 31 times;
+// a whole 256 on a sum in the same binade is exact, so this rounds once a doubling.
 // The box starts HZ = 4 cells below the tile in z so that its rows are made of 16-byte
 // chunks aligned in the mesh: the flush adds four cells per vector reduction.
 template <int R, int XC = 16>
@@ -51,13 +51,11 @@ struct DepTile {
     static constexpr int TX = XC / R, TY = 16 / R, TZ = 32 / R, H = 2, HZ = 4;
     static constexpr int DX = TX * R + 2 * H, DY = TY * R + 2 * H, DZ = TZ * R + 2 * HZ;
     static constexpr int CELLS = DX * DY * DZ, CZ = DZ / 4, PLANE = DY * CZ;  // 16-byte chunks a row, an x plane
-    static constexpr int CARRY_WORDS = CELLS / 4;      // one word of four 8-bit carries per chunk
-    static constexpr int WORDS = CELLS + CARRY_WORDS;  // shared memory: lo[CELLS], carry[CARRY_WORDS]
     static constexpr int PER = TX * TY * TZ;
     static constexpr int PLANES = THREADS / PLANE;     // x planes a pass over the chunks takes at once
     static_assert(TX >= 1 && PER * R * R * R <= 8192, "tile mass bound");
     static_assert(DZ % 4 == 0 && (TZ * R) % 4 == 0 && HZ % 4 == 0, "z box made of aligned 16-byte chunks");
-    static_assert(CELLS % 4 == 0 && CARRY_WORDS % 4 == 0 && PLANES >= 1, "whole vectors");
+    static_assert(CELLS % 4 == 0 && PLANES >= 1, "whole vectors");
 };
 
 __device__ __forceinline__ void red_add_v4(float* dst, float4 v) {
@@ -75,10 +73,18 @@ __device__ __forceinline__ void tile_add(uint32_t* lo, int c, float w, uint32_t&
     atomicAdd(lo + c, v);
     sum += v;
 }
-__device__ __forceinline__ void tile_add_carry(uint32_t* lo, uint32_t* carry, int c, float w) {
+// The mesh cell is found from the tile's only when a cell wraps: its address is not held otherwise.
+template <class D>
+__device__ __forceinline__ void tile_add_wrapping(uint32_t* lo, int c, float w, float* __restrict__ rho, int ox, int oy,
+                                                  int oz, int logn) {
     const uint32_t v = __float2uint_rn(w);
     const uint32_t old = atomicAdd(lo + c, v);
-    if (old + v < old) atomicAdd(carry + (c >> 2), 1u << (8 * (c & 3)));
+    if (old + v < old) {
+        const int nm = (1 << logn) - 1, row = c / D::DZ;
+        atomicAdd(rho + ((((uint32_t)((ox + row / D::DY) & nm) << logn) + (uint32_t)((oy + row % D::DY) & nm)) << logn) +
+                      ((oz + c % D::DZ) & nm),
+                  256.0f);
+    }
 }
 
 template <int WORDS>
@@ -89,9 +95,9 @@ __device__ __forceinline__ void tile_zero(uint32_t* words) {
 
 // One particle's CIC weights into the tile (box origin o*) or, outside it, into rho.  quanta =
 // mass 2^24 (a power of two times the mass: the weights are the same numbers, scaled).
-// CARRY: the second accumulation of a tile, of the particles inside the box alone.
-template <class D, bool CARRY>
-__device__ __forceinline__ void tile_deposit(uint32_t* lo, uint32_t* carry, float* __restrict__ rho, uint32_t u0,
+// AGAIN: the second accumulation of a tile, of the particles inside the box alone.
+template <class D, bool AGAIN>
+__device__ __forceinline__ void tile_deposit(uint32_t* lo, float* __restrict__ rho, uint32_t u0,
                                              uint32_t u1, uint32_t u2, int logn, float inv_cell_ticks, int ox,
                                              int oy, int oz, float quanta, uint32_t& sum) {
     const int nm = (1 << logn) - 1;
@@ -108,15 +114,15 @@ __device__ __forceinline__ void tile_deposit(uint32_t* lo, uint32_t* carry, floa
             for (int b = 0; b < 2; ++b) {
                 const float wab = quanta * wx[a] * wy[b];
                 const int c = c0 + (a * D::DY + b) * D::DZ;
-                if (CARRY) {
-                    tile_add_carry(lo, carry, c, wab * wz[0]);
-                    tile_add_carry(lo, carry, c + 1, wab * wz[1]);
+                if (AGAIN) {
+                    tile_add_wrapping<D>(lo, c, wab * wz[0], rho, ox, oy, oz, logn);
+                    tile_add_wrapping<D>(lo, c + 1, wab * wz[1], rho, ox, oy, oz, logn);
                 } else {
                     tile_add(lo, c, wab * wz[0], sum);
                     tile_add(lo, c + 1, wab * wz[1], sum);
                 }
             }
-    } else if (!CARRY) {
+    } else if (!AGAIN) {
         const uint32_t ix[2] = {(uint32_t)cx.i0, (uint32_t)cx.i1}, iy[2] = {(uint32_t)cy.i0, (uint32_t)cy.i1};
 #pragma unroll
         for (int a = 0; a < 2; ++a)
@@ -142,36 +148,26 @@ __device__ __forceinline__ void for_chunks(F f) {
 
 // Adds the tile's cells (box origin o*, oz a multiple of 4, rho 16-byte aligned) to rho,
 // four z-cells per reduction.
-template <class D, bool CARRY>
-__device__ __forceinline__ void tile_flush(const uint32_t* lo, const uint32_t* carry, float* __restrict__ rho, int ox,
-                                           int oy, int oz, int logn) {
+template <class D>
+__device__ __forceinline__ void tile_flush(const uint32_t* lo, float* __restrict__ rho, int ox, int oy, int oz,
+                                           int logn) {
     const int nm = (1 << logn) - 1;
     for_chunks<D>([&](int c, int lx, int ly, int lz4) {
         const uint4 l = reinterpret_cast<const uint4*>(lo)[c];
-        const uint32_t h = CARRY ? carry[c] : 0u;
-        if (l.x | l.y | l.z | l.w | h) {
-            float4 v = make_float4(__uint2float_rn(l.x) * kTileQuantum, __uint2float_rn(l.y) * kTileQuantum,
-                                   __uint2float_rn(l.z) * kTileQuantum, __uint2float_rn(l.w) * kTileQuantum);
-            if (CARRY) {
-                v.x += (float)(h & 255u) * 256.0f;
-                v.y += (float)((h >> 8) & 255u) * 256.0f;
-                v.z += (float)((h >> 16) & 255u) * 256.0f;
-                v.w += (float)(h >> 24) * 256.0f;
-            }
+        if (l.x | l.y | l.z | l.w)
             red_add_v4(rho + ((((uint32_t)((ox + lx) & nm) << logn) + (uint32_t)((oy + ly) & nm)) << logn) +
                            ((oz + 4 * lz4) & nm),
-                       v);
-        }
+                       make_float4(__uint2float_rn(l.x) * kTileQuantum, __uint2float_rn(l.y) * kTileQuantum,
+                                   __uint2float_rn(l.z) * kTileQuantum, __uint2float_rn(l.w) * kTileQuantum));
     });
 }
 
 // Ends a tile: compares the sum of its cells with the sum of all additions (`sum` of every
-// thread) and flushes it, after accumulating it again with carries when they differ (redo()
-// deposits the thread's particles from their written positions with CARRY).  Every thread of
-// the CTA calls it.
+// thread) and flushes it, after accumulating it again when they differ (redo() deposits the
+// thread's particles from their written positions with AGAIN).  Every thread of the CTA calls it.
 template <class D, class F>
-__device__ __forceinline__ void tile_close(uint32_t* lo, uint32_t* carry, float* __restrict__ rho, int ox, int oy,
-                                           int oz, int logn, uint32_t sum, F redo) {
+__device__ __forceinline__ void tile_close(uint32_t* lo, float* __restrict__ rho, int ox, int oy, int oz, int logn,
+                                           uint32_t sum, F redo) {
     __shared__ unsigned long long missing;
     if (threadIdx.x == 0) missing = 0;
     __syncthreads();
@@ -188,14 +184,14 @@ __device__ __forceinline__ void tile_close(uint32_t* lo, uint32_t* carry, float*
         atomicAdd(&missing, (unsigned long long)l0 + ((unsigned long long)l1 << 16) + ((unsigned long long)l2 << 32));
     __syncthreads();
     if (missing == 0) {
-        tile_flush<D, false>(lo, carry, rho, ox, oy, oz, logn);
+        tile_flush<D>(lo, rho, ox, oy, oz, logn);
         return;
     }
-    tile_zero<D::WORDS>(lo);  // the carries follow the cells
+    tile_zero<D::CELLS>(lo);
     __syncthreads();
     redo();
     __syncthreads();
-    tile_flush<D, true>(lo, carry, rho, ox, oy, oz, logn);
+    tile_flush<D>(lo, rho, ox, oy, oz, logn);
 }
 
 // Deposit of a thread walking its lattice row along x (R = 1).  The next particle usually
