@@ -14,7 +14,7 @@
 // are bound by that pipe and by issue, not by registers.  The threads of a row then fit in one
 // warp (Q <= 32) and its exchange needs only __syncwarp.  With eight elements a thread (three
 // stages at 512, CTA barriers) the passes of a 512^3 force evaluation took 432 (forward z + y),
-// 457 (x) and 1317 us (inverse y + z with the gradients); they take 324, 340 and 976 us, the
+// 457 (x) and 1317 us (inverse y + z with the gradients); they take 320, 313 and 977 us, the
 // first and the last at the copy bandwidth over the bytes they move (2.15 and 6.46 GB).
 //
 // Twiddles come from a per-stage table (tw_stage_offset; values from the host FP64 table
@@ -34,82 +34,104 @@ __device__ __forceinline__ void dft2(C& a, C& b) {
     b = csub(t, b);
 }
 
+// (x + iy) exp(-+ i pi/4) and (x + iy) exp(-+ 3 i pi/4), times sqrt 2.  The factor 1/sqrt 2 is
+// left to the additions that follow, as one fused operation each (add_w8, sub_w8): the compiler does
+// not contract the packed additions with a multiplication, and with the product rounded by itself
+// the 512^3 transform was 2% further from 64 bits, its x pass took 325 us for 316, the inverse y and
+// z passes 992 for 983.
 template <bool INV, typename C>
+__device__ __forceinline__ C rot_w8_1(C a) {
+    return INV ? cmake<C>(a.x - a.y, a.x + a.y) : cmake<C>(a.x + a.y, a.y - a.x);
+}
+template <bool INV, typename C>
+__device__ __forceinline__ C rot_w8_3(C a) {
+    return INV ? cmake<C>(-a.x - a.y, a.x - a.y) : cmake<C>(a.y - a.x, -a.x - a.y);
+}
+// a + b, a - b, b times 1/sqrt 2 when W8
+template <bool W8, typename C>
+__device__ __forceinline__ C add_w8(C a, C b) {
+    if constexpr (W8) return cfma(decltype(a.x)(0.70710678118654752440), b, a);
+    else return cadd(a, b);
+}
+template <bool W8, typename C>
+__device__ __forceinline__ C sub_w8(C a, C b) {
+    if constexpr (W8) return cfma(decltype(a.x)(-0.70710678118654752440), b, a);
+    else return csub(a, b);
+}
+
+// S2: v2 waits for its factor 1/sqrt 2, S13: v1 and v3 do.
+template <bool INV, bool S2 = false, bool S13 = false, typename C>
 __device__ __forceinline__ void dft4(C& v0, C& v1, C& v2, C& v3) {
-    C t0 = cadd(v0, v2), t1 = csub(v0, v2), t2 = cadd(v1, v3);
+    C t0 = add_w8<S2>(v0, v2), t1 = sub_w8<S2>(v0, v2), t2 = cadd(v1, v3);
     C t3 = cmul_mi<INV>(csub(v1, v3));
-    v0 = cadd(t0, t2);
-    v2 = csub(t0, t2);
-    v1 = cadd(t1, t3);
-    v3 = csub(t1, t3);
+    v0 = add_w8<S13>(t0, t2);
+    v2 = sub_w8<S13>(t0, t2);
+    v1 = add_w8<S13>(t1, t3);
+    v3 = sub_w8<S13>(t1, t3);
 }
 
-// (x + iy) exp(-+ i pi/4) and (x + iy) exp(-+ 3 i pi/4)
-template <bool INV, typename C>
-__device__ __forceinline__ C mul_w8_1(C a) {
-    typedef decltype(a.x) T;
-    const T s = T(0.70710678118654752440);
-    return INV ? cmake<C>((a.x - a.y) * s, (a.x + a.y) * s) : cmake<C>((a.x + a.y) * s, (a.y - a.x) * s);
-}
-template <bool INV, typename C>
-__device__ __forceinline__ C mul_w8_3(C a) {
-    typedef decltype(a.x) T;
-    const T s = T(0.70710678118654752440);
-    return INV ? cmake<C>((-a.x - a.y) * s, (a.x - a.y) * s) : cmake<C>((a.y - a.x) * s, (-a.x - a.y) * s);
-}
-
-template <bool INV, typename C>
+// S4: v[4] waits for its factor 1/sqrt 2, S26: v[2] and v[6] do.
+template <bool INV, bool S4 = false, bool S26 = false, typename C>
 __device__ __forceinline__ void dft8(C* v) {
     // even / odd split: E = DFT4(v0 v2 v4 v6), O = DFT4(v1 v3 v5 v7); X_k = E_k + w^k O_k
-    dft4<INV>(v[0], v[2], v[4], v[6]);
+    dft4<INV, S4, S26>(v[0], v[2], v[4], v[6]);
     dft4<INV>(v[1], v[3], v[5], v[7]);
-    const C o1 = mul_w8_1<INV>(v[3]);
+    const C o1 = rot_w8_1<INV>(v[3]);
     const C o2 = cmul_mi<INV>(v[5]);
-    const C o3 = mul_w8_3<INV>(v[7]);
+    const C o3 = rot_w8_3<INV>(v[7]);
     const C e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
     v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
-    v[1] = cadd(e1, o1); v[5] = csub(e1, o1);
+    v[1] = add_w8<true>(e1, o1); v[5] = sub_w8<true>(e1, o1);
     v[2] = cadd(e2, o2); v[6] = csub(e2, o2);
-    v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
+    v[3] = add_w8<true>(e3, o3); v[7] = sub_w8<true>(e3, o3);
 }
 
-// cos(2 pi j / 32), j = 0..16
-__host__ __device__ constexpr double cos32(int j) {
-    return j > 8 ? -cos32(16 - j)
-                 : (j == 0   ? 1.0
-                    : j == 1 ? 0.98078528040323044913
-                    : j == 2 ? 0.92387953251128675613
-                    : j == 3 ? 0.83146961230254523708
-                    : j == 4 ? 0.70710678118654752440
-                    : j == 5 ? 0.55557023301960222474
-                    : j == 6 ? 0.38268343236508977173
-                    : j == 7 ? 0.19509032201612826785
-                             : 0.0);
+// a exp(-+2 pi i J / 32), |J| <= 3, by three shears (the rotation of Paeth 1986): along x by
+// tan(theta / 2), along y by sin(theta), along x again.  Three fused operations instead of two and
+// two products, and the rounded constants are small beside 1: cos(pi/16) and cos(pi/8) are both
+// nearly half a unit low in FP32.  Relative error of the r2c transform of white noise with cos and
+// sin, and now: 1.61e-7 and 1.56e-7 (128^3), 1.77e-7 and 1.64e-7 (256^3), 1.93e-7 and 1.74e-7
+// (512^3).  FP64 at 256^3, us: forward 863 -> 844, x 1331 -> 1293, inverse 2596 -> 2539.
+template <int J, bool INV, typename C>
+__device__ __forceinline__ C shear_w32(C a) {
+    typedef decltype(a.x) T;
+    constexpr int j = J < 0 ? -J : J;
+    constexpr double tan_half = j == 1 ? 0.098491403357164253077 : j == 2 ? 0.19891236737965800691 : 0.30334668360734239168;
+    constexpr double sine = j == 1 ? 0.19509032201612826785 : j == 2 ? 0.38268343236508977173 : 0.55557023301960222474;
+    constexpr T sign = T((J < 0) != INV ? -1 : 1);
+    constexpr T t = sign * T(tan_half), s = sign * T(sine);
+    const T x = fma(t, a.y, a.x), y = fma(-s, x, a.y);
+    return cmake<C>(fma(t, y, x), y);
 }
 
-// a exp(-+2 pi i J / 32), J = 0..31
+// a exp(-+2 pi i J / 32), J = 0..31, times sqrt 2 for J = 4, 12, 20, 28
 template <int J, bool INV, typename C>
 __device__ __forceinline__ C mul_w32(C a) {
-    typedef decltype(a.x) T;
     if constexpr (J >= 16) {
         const C b = mul_w32<J - 16, INV>(a);
         return cmake<C>(-b.x, -b.y);
     } else if constexpr (J == 0) {
         return a;
     } else if constexpr (J == 4) {
-        return mul_w8_1<INV>(a);
+        return rot_w8_1<INV>(a);
+    } else if constexpr (J == 12) {
+        return rot_w8_3<INV>(a);
     } else if constexpr (J == 8) {
         return cmul_mi<INV>(a);
-    } else if constexpr (J == 12) {
-        return mul_w8_3<INV>(a);
+    } else if constexpr (J < 4) {
+        return shear_w32<J, INV>(a);
+    } else if constexpr (J < 12) {
+        return shear_w32<J - 8, INV>(cmul_mi<INV>(a));
     } else {
-        constexpr T c = T(cos32(J)), s = T(J <= 8 ? cos32(8 - J) : cos32(J - 8));
-        return INV ? cmake<C>(a.x * c - a.y * s, a.y * c + a.x * s) : cmake<C>(a.x * c + a.y * s, a.y * c - a.x * s);
+        const C b = shear_w32<J - 16, INV>(a);
+        return cmake<C>(-b.x, -b.y);
     }
 }
 
 // A DFT of size 4 R2 as 4 x R2: DFT4 over the stride-R2 elements, the twiddles
-// exp(-+2 pi i n2 k1 / (4 R2)), then DFT_R2 over n2 for each k1; X_{k1 + 4 k2}.
+// exp(-+2 pi i n2 k1 / (4 R2)), then DFT_R2 over n2 for each k1; X_{k1 + 4 k2}.  The eighth roots
+// among the twiddles are those of n2 = R2 / 2 at k1 = 1, 3 and of n2 = R2 / 4, 3 R2 / 4 at k1 = 2:
+// the elements whose factor the DFT_R2 takes into its first additions.
 template <int R2, int N2, int K1, bool INV, typename C>
 __device__ __forceinline__ void dft4xr_twiddle(C* v) {
     if constexpr (K1 < 4) {
@@ -122,13 +144,20 @@ __device__ __forceinline__ void dft4xr_twiddle(C* v) {
 
 template <int R2, bool INV, typename C>
 __device__ __forceinline__ void dft4xr(C* v) {
+    static_assert(R2 == 4 || R2 == 8, "DFT_R2 below");
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) dft4<INV>(v[n2], v[n2 + R2], v[n2 + 2 * R2], v[n2 + 3 * R2]);
     dft4xr_twiddle<R2, 1, 1, INV>(v);
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-        if constexpr (R2 == 8) dft8<INV>(v + R2 * k1);
-        else dft4<INV>(v[R2 * k1], v[R2 * k1 + 1], v[R2 * k1 + 2], v[R2 * k1 + 3]);
+    if constexpr (R2 == 8) {
+        dft8<INV>(v);
+        dft8<INV, true, false>(v + 8);
+        dft8<INV, false, true>(v + 16);
+        dft8<INV, true, false>(v + 24);
+    } else {
+        dft4<INV>(v[0], v[1], v[2], v[3]);
+        dft4<INV, true, false>(v[4], v[5], v[6], v[7]);
+        dft4<INV, false, true>(v[8], v[9], v[10], v[11]);
+        dft4<INV, true, false>(v[12], v[13], v[14], v[15]);
     }
     C w[4 * R2];
 #pragma unroll

@@ -99,8 +99,9 @@ template <typename T, int LOGN> struct YShape {
 };
 // x passes: CB columns of one plane a CTA, CTAs of 64 to 256 threads with several an SM.  Eight
 // columns (64-byte row segments) beat sixteen where a thread holds 16 or 32 values: 340 against
-// 457 us for the Newtonian pass at 512^3 and 43 against 48 us at 256^3, since the wider CTA
-// halves the CTAs an SM that overlap one another's loads; below that sixteen are better.
+// 457 us for the Newtonian pass at 512^3 and 43 against 48 us at 256^3 when they were compared (313
+// and 41 now), since the wider CTA halves the CTAs an SM that overlap one another's loads; below
+// that sixteen are better.
 template <typename T, int LOGN> struct XShape {
     static constexpr int N = 1 << LOGN, E = plan_e(N), Q = N / E;
     static constexpr int CB = (sizeof(T) == 8) ? (E == 32 ? 4 : 8) : (E >= 16 ? 8 : 16);

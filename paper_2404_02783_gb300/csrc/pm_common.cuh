@@ -80,6 +80,11 @@ __device__ __forceinline__ float2 fma2(float s, float2 a, float2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
     return *reinterpret_cast<float2*>(&r);
 }
+// s a + c, each part rounded once
+__device__ __forceinline__ float2 cfma(float s, float2 a, float2 c) { return fma2(s, a, c); }
+__device__ __forceinline__ double2 cfma(double s, double2 a, double2 c) {
+    return make_double2(fma(s, a.x, c.x), fma(s, a.y, c.y));
+}
 // multiply by -i (forward) or +i (inverse)
 template <bool INV, typename C> __device__ __forceinline__ C cmul_mi(C a) {
     C c;
