@@ -597,10 +597,12 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
             // |n|^2 is monotone over them, and a bin is a contiguous range of |n|^2: when the first
             // and the last mode of a group of eight fall in the same bin (neither the zero mode nor
             // beyond (n/2)^2), so do all eight, and two table lookups replace eight.  Consecutive
-            // modes of a bin are summed in registers, each run added once to the CTA's row (native
+            // modes of a bin are summed in registers, at most eight of them in the working precision
+            // before they join the run's FP64 total; each run is added once to the CTA's row (native
             // FP64 reduction in L2).
             int run_bin = -1;
             T run_sum = T(0), run_sum2 = T(0);
+            double run_tot = 0.0, run_tot2 = 0.0;
             const T wyz = iw2[ny < 0 ? -ny : ny] * iw2[kz] * T((kz == 0 || kz == M) ? 1 : 2);
             constexpr int G = E < 8 ? E : 8;
 #pragma unroll
@@ -629,10 +631,11 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
                     const T val2 = acc2_row ? (uu.x * uu.x + uu.y * uu.y) * wgt : T(0);
                     if (bin != run_bin) {
                         if (run_bin >= 0) {
-                            atomicAdd(acc_row + run_bin, (double)run_sum);
-                            if (acc2_row) atomicAdd(acc2_row + run_bin, (double)run_sum2);
+                            atomicAdd(acc_row + run_bin, run_tot + (double)run_sum);
+                            if (acc2_row) atomicAdd(acc2_row + run_bin, run_tot2 + (double)run_sum2);
                         }
                         run_bin = bin;
+                        run_tot = run_tot2 = 0.0;
                         run_sum = val;
                         run_sum2 = val2;
                     } else {
@@ -640,10 +643,18 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>:
                         run_sum2 += val2;
                     }
                 }
+                if (g + G < E) {
+                    run_tot += (double)run_sum;
+                    run_sum = T(0);
+                    if (acc2_row) {
+                        run_tot2 += (double)run_sum2;
+                        run_sum2 = T(0);
+                    }
+                }
             }
             if (run_bin >= 0) {
-                atomicAdd(acc_row + run_bin, (double)run_sum);
-                if (acc2_row) atomicAdd(acc2_row + run_bin, (double)run_sum2);
+                atomicAdd(acc_row + run_bin, run_tot + (double)run_sum);
+                if (acc2_row) atomicAdd(acc2_row + run_bin, run_tot2 + (double)run_sum2);
             }
             continue;
         } else {
