@@ -15,8 +15,8 @@ namespace pm {
 // k_deposit_tiled would have done from the drifted positions.
 // blockIdx.y selects the field of a batch of independent runs stored back to back
 // (particles [field][3][np^3], force meshes [field][n][n][3][n], density [field][n^3]); scale =
-// 2^32 / L of that field.  The mesh side 2^LOGN is a compile-time constant: the kernels are
-// bound by issue, and its shifts, masks and row strides are then immediates.
+// 2^32 / L of that field.  The mesh side 2^LOGN is a compile-time constant: the kernels were
+// bound by issue without it, and its shifts, masks and row strides are then immediates.
 template <int R, int XC, int LOGN, bool FD>
 __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
                                                         float* __restrict__ p, const float* __restrict__ g, float kick,
@@ -121,14 +121,15 @@ __device__ __noinline__ void sweep_again_call(uint32_t* lo, const uint32_t* xo, 
 // carries the upper-plane weights in registers, adds them to the next particle's
 // lower-plane weights and issues 4 tile atomics a particle instead of 8.  Any other
 // particle takes the full path, so the result is the same CIC gather and deposit.
-// Bound by issue (about 70% busy) and by the latency of the gather: the upper plane's loads, which
-// every particle needs, are issued before the branch that reloads the lower plane (512^3, early
-// and clustered steps: 1742 and 1953 us; after it 1826 and 2020).  The components are interpolated
-// in packed pairs, and a tile without words for carries leaves the L1 cache 100 KB an SM instead of
-// 68 for the force planes that neighbouring rows share (1733 and 1946 us with both the other way,
-// 1723 and 1902 now; 2783 and 2633 at 2 Mpc/h cells, where particles have moved furthest).  Holding the gather in flight
-// across the previous particle's deposit spills at two 512-thread CTAs an SM (2293 us) and gains
-// nothing at three 256-thread CTAs (1798 and 1958).
+// Bound by the latency of the gather (256^3: long scoreboard 7.8 cycles an issue, issue 56% busy, 142 M
+// warp instructions) with two CTAs an SM: the upper plane's loads, which every particle needs, are
+// issued before the branch that reloads the lower plane (512^3, early and clustered steps: 1742 and
+// 1953 us; after it 1826 and 2020).  The components are interpolated in packed pairs, and a tile
+// without words for carries leaves the L1 cache 100 KB an SM instead of 68 for the force planes that
+// neighbouring rows share (1733 and 1946 us with both the other way, 1723 and 1903 now; 2783 and 2633
+// at 2 Mpc/h cells, where particles have moved furthest).  Holding the gather in flight across the
+// previous particle's deposit spills at two 512-thread CTAs an SM (2293 us) and gains nothing at
+// three 256-thread CTAs (1798 and 1958).
 template <int XC, int LOGN, bool FD>
 __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
                                                               float* __restrict__ p, const float* __restrict__ g,
