@@ -446,11 +446,12 @@ pm_status pm_batch_bias(pm_batch* batch, double fraction, int nbins, const doubl
 
 /* CIC deposit (Sec. 4 counting density): rho[n][n][n] += mass * CIC weights of
  * count particles x[3][count] (ticks or fractions, per precision).  rho is NOT
- * cleared first.  n a power of two in 8..1024. */
+ * cleared first.  n a power of two in 2..1024. */
 pm_status pm_cic_deposit(const void* x, int64_t count, int precision, int n, double mass,
                          void* rho, void* stream);
 
-/* CIC interpolation of a scalar mesh field[n][n][n] to count particles: out[count]. */
+/* CIC interpolation of a scalar mesh field[n][n][n] to count particles: out[count].
+ * n a power of two in 2..1024. */
 pm_status pm_cic_interp(const void* field, int n, const void* x, int64_t count, int precision,
                         void* out, void* stream);
 

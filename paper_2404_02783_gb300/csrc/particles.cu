@@ -63,7 +63,11 @@ __device__ __forceinline__ CicD cic_frac(double x, int logn) {
 }
 
 // ---------------------------------------------------------------- deposit
-// Particles in any order.  Bound by the L2's atomic operations: with V4 (rho 16-byte aligned) the
+// The vector forms below read and write aligned groups of four cells of a z row: rows of at least
+// one such group, on 16-byte boundaries.
+static bool quad_rows(const void* mesh, int n) { return n >= 4 && (uintptr_t)mesh % 16 == 0; }
+
+// Particles in any order.  Bound by the L2's atomic operations: with V4 (quad_rows) the
 // two z corners of a row go in one vector reduction when they share an aligned group of four
 // cells (three rows in four), its other lanes adding 0.
 template <bool V4>
@@ -314,7 +318,7 @@ cudaError_t deposit(const void* x, int64_t count, int precision, int n, double m
     const int logn = ilog2(n);
     if (precision == PM_FP32_FIXED) {
         const float inv = (float)ldexp(1.0, -(32 - logn));
-        const auto fn = (uintptr_t)rho % 16 == 0 ? k_deposit_ticks<true> : k_deposit_ticks<false>;
+        const auto fn = quad_rows(rho, n) ? k_deposit_ticks<true> : k_deposit_ticks<false>;
         fn<<<grid_for(count, 256), 256, 0, st>>>((const uint32_t*)x, count, logn, inv, (float)mass, (float*)rho);
     } else {
         k_deposit_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)x, count, logn, mass, (double*)rho);
@@ -337,7 +341,7 @@ __device__ __forceinline__ T gather8(const T* __restrict__ f, size_t n, const in
     return acc;
 }
 
-// V4 (field 16-byte aligned): a row's two z corners come in one 16-byte load when they share an
+// V4 (quad_rows): a row's two z corners come in one 16-byte load when they share an
 // aligned group of four cells, which saves requests to L2.
 template <bool V4>
 __global__ void k_interp_ticks(const float* __restrict__ f, int logn, const uint32_t* __restrict__ x,
@@ -392,7 +396,7 @@ cudaError_t interp(const void* field, int n, const void* x, int64_t count, int p
     const int logn = ilog2(n);
     if (precision == PM_FP32_FIXED) {
         const float inv = (float)ldexp(1.0, -(32 - logn));
-        const auto fn = (uintptr_t)field % 16 == 0 ? k_interp_ticks<true> : k_interp_ticks<false>;
+        const auto fn = quad_rows(field, n) ? k_interp_ticks<true> : k_interp_ticks<false>;
         fn<<<grid_for(count, 256), 256, 0, st>>>((const float*)field, logn, (const uint32_t*)x, count, inv, (float*)out);
     } else {
         k_interp_frac<<<grid_for(count, 256), 256, 0, st>>>((const double*)field, logn, (const double*)x, count,
