@@ -74,10 +74,9 @@ __global__ void k_adj_gather(const uint32_t* __restrict__ x, int64_t count, int 
 // Bound by the latency of its 32 gathers a particle, i.e. by warps in flight: walking the lattice
 // rows with the upper plane's 16 values kept in registers takes 105 registers and 40.5 us at
 // 128^3 against 36.6.
-__global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* __restrict__ x, int64_t count, int logn,
-                                                  float inv_cell_ticks, float* __restrict__ v,
-                                                  const float* __restrict__ G, const float* __restrict__ rho_bar,
-                                                  float K, float Km, float drift_next, float* __restrict__ lam_u) {
+__global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* x, int64_t count, int logn, float inv_cell_ticks,
+                                                  float* __restrict__ v, const float* G, const float* rho_bar, float K,
+                                                  float Km, float drift_next, float* __restrict__ lam_u) {
     const int n = 1 << logn;
     const float nf = (float)n;
     launch_next();
@@ -114,8 +113,8 @@ __global__ void __launch_bounds__(256) k_adj_kick(const uint32_t* __restrict__ x
                     const uint32_t row = ((ix[a] << logn) + iy[b]) << logn, o = row + iz[c];
                     const float* Go = G + (kForceRows * row + iz[c]);
                     // K sum_j v_j G_j + K mass rho_bar at the corner
-                    const float s = K * (v0 * __ldg(Go) + v1 * __ldg(Go + n) + v2 * __ldg(Go + 2 * n)) +
-                                    Km * __ldg(rho_bar + o);
+                    const float s = K * (v0 * load_ordered(Go) + v1 * load_ordered(Go + n) + v2 * load_ordered(Go + 2 * n)) +
+                                    Km * load_ordered(rho_bar + o);
                     g0 = fmaf(dw[a] * wy[b] * wz[c], s, g0);
                     g1 = fmaf(wx[a] * dw[b] * wz[c], s, g1);
                     g2 = fmaf(wx[a] * wy[b] * dw[c], s, g2);
@@ -211,8 +210,8 @@ __global__ void __launch_bounds__(256) k_adj_kick_fd(const uint32_t* __restrict_
 // particles that are neighbours in z, and usually sit one cell apart: a lane then hands its
 // upper-z values to the next lane, which adds them to its lower-z ones (6 atomics a particle).
 template <bool MERGE>
-__global__ void __launch_bounds__(256) k_deposit_vec_rows(const uint32_t* __restrict__ x, int lognp, int logn,
-                                                          int run, float inv_cell_ticks, const float* __restrict__ v,
+__global__ void __launch_bounds__(256) k_deposit_vec_rows(const uint32_t* x, int lognp, int logn,
+                                                          int run, float inv_cell_ticks, const float* v,
                                                           float* __restrict__ V0, float* __restrict__ V1,
                                                           float* __restrict__ V2) {
     const int np = 1 << lognp;

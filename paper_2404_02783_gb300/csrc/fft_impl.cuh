@@ -122,7 +122,7 @@ __device__ __forceinline__ size_t spec_row(int gl, int kz) {
 // [0.5, 2^24] and below 0.5 within half the spacing of the values near 1 (2^-25 in FP32).
 template <typename T, int LOGN>
 __global__ void __launch_bounds__(ZShape<T, LOGN>::THREADS, ZShape<T, LOGN>::MINB)
-    k_z_r2c(const T* __restrict__ in, cplx<T>* __restrict__ out, T sub, int kz_max) {
+    k_z_r2c(const T* in, cplx<T>* __restrict__ out, T sub, int kz_max) {
     typedef cplx<T> C;
     typedef ZShape<T, LOGN> S;
     constexpr int N = S::N, M = S::M, E = S::E, Q = S::Q, YB = S::YB, RS = S::RS;
@@ -502,7 +502,7 @@ template <typename T, int LOGN, int KIND> struct XRes {
 // binning pass runs one CTA for each row of bin sums, the others one for each block.
 template <typename T, int LOGN, int KIND>
 __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, XRes<T, LOGN, KIND>::MINB)
-    k_x_cols(cplx<T>* __restrict__ data, cplx<T>* __restrict__ out2, SpecOp op, int nplanes) {
+    k_x_cols(cplx<T>* data, cplx<T>* __restrict__ out2, SpecOp op, int nplanes) {
     typedef cplx<T> C;
     typedef XShape<T, LOGN> S;
     constexpr int N = S::N, M = N / 2, E = S::E, Q = S::Q, CB = S::CB;

@@ -12,12 +12,23 @@ namespace pm {
 // The kernels of a step are launched so that each may start while the one before it on the stream
 // drains (programmatic dependent launch): launch_next lets the next one in, and wait_previous
 // holds this one until the kernels before it are complete and their writes visible.  Every such
-// kernel calls it before its first access to global memory, so the order of the stream holds;
-// kernels launched in the ordinary way see the whole of it as before.  On small meshes, where a
+// kernel calls it before its first access to anything an earlier kernel writes (the constant
+// tables, uploaded once, may be read before), so the order of the stream holds; kernels launched
+// in the ordinary way see the whole of it as before.  A chained kernel is resident while its
+// predecessor still writes what it will read, so it reads that by plain loads: the non-coherent
+// ones (__ldg, const __restrict__ parameters) ask for data that is constant as long as the kernel
+// runs, which holds for the tables alone.  On small meshes, where a
 // step is six kernels of a few microseconds, the ramps are a good part of the time: a step took
 // 33.4 us at 32^3 and takes 22.2, 77.5 and 71.0 at 128^3, 470 and 453 at 256^3, 3848 and 3834 at 512^3.
 __device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A plain load that keeps its place among the other asm statements: the compiler does not gather
+// many of them ahead of their use, which costs registers (58 for 48 in k_adj_kick).
+__device__ __forceinline__ float load_ordered(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 
 template <typename... K, typename... A>
 cudaError_t launch_chained(void (*fn)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {

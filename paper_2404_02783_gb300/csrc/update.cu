@@ -18,8 +18,8 @@ namespace pm {
 // 2^32 / L of that field.  The mesh side 2^LOGN is a compile-time constant: the kernels were
 // bound by issue without it, and its shifts, masks and row strides are then immediates.
 template <int R, int XC, int LOGN, bool FD>
-__global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
-                                                        float* __restrict__ p, const float* __restrict__ g, float kick,
+__global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* x, uint32_t* __restrict__ xo,
+                                                        float* __restrict__ p, const float* g, float kick,
                                                         double drift, double scale0,
                                                         const double* __restrict__ scale_arr, float mass,
                                                         float* __restrict__ rho, float inv_d) {
@@ -131,8 +131,8 @@ __device__ __noinline__ void sweep_again_call(uint32_t* lo, const uint32_t* xo, 
 // previous particle's deposit spills at two 512-thread CTAs an SM (2293 us) and gains nothing at
 // three 256-thread CTAs (1798 and 1958).
 template <int XC, int LOGN, bool FD>
-__global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __restrict__ x, uint32_t* __restrict__ xo,
-                                                              float* __restrict__ p, const float* __restrict__ g,
+__global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* x, uint32_t* __restrict__ xo,
+                                                              float* __restrict__ p, const float* g,
                                                               float kick, double drift, double scale0,
                                                               const double* __restrict__ scale_arr, float mass,
                                                               float* __restrict__ rho, float inv_d) {
@@ -199,13 +199,13 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* __
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int j = 0; j < NC; ++j) U[q][j] = __ldg(g + ku[q] + j * np);
+                for (int j = 0; j < NC; ++j) U[q][j] = g[ku[q] + j * np];
             if (!same) {
                 const PlaneCorners<ROWS> k(cx.i0, cy, cz, logn);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
-                    for (int j = 0; j < NC; ++j) L[q][j] = __ldg(g + k[q] + j * np);
+                    for (int j = 0; j < NC; ++j) L[q][j] = g[k[q] + j * np];
             }
             next_cell = ((uint32_t)cx.i1 << (2 * LOGN)) | yz;
             const float wy[2] = {1.0f - cy.w1, cy.w1}, wz[2] = {1.0f - cz.w1, cz.w1};

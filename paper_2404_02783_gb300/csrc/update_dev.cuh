@@ -305,7 +305,7 @@ struct PlaneCorners {
 // to first order (fd1_force).
 template <bool FD>
 __device__ __forceinline__ void ikd_particle(uint32_t& u0, uint32_t& u1, uint32_t& u2, float& p0, float& p1,
-                                             float& p2, int logn, float inv_cell_ticks, const float* __restrict__ g,
+                                             float& p2, int logn, float inv_cell_ticks, const float* g,
                                              float kick, float drift_ticks, float inv_d) {
     constexpr int ROWS = FD ? 1 : kForceRows;
     const CicF cx = cic_ticks(u0, logn, inv_cell_ticks);
@@ -319,7 +319,7 @@ __device__ __forceinline__ void ikd_particle(uint32_t& u0, uint32_t& u1, uint32_
 #pragma unroll
         for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) P[a][q] = __ldg(g + k[a][q]);
+            for (int q = 0; q < 4; ++q) P[a][q] = g[k[a][q]];
         fd1_force<float>(P[0], P[1], wx[0], wx[1], wy, wz, inv_d, f0, f1, f2);
     } else {
         const int n = 1 << logn;
@@ -330,9 +330,9 @@ __device__ __forceinline__ void ikd_particle(uint32_t& u0, uint32_t& u1, uint32_
                 const float* c0 = g + k[a][2 * b];
                 const float* c1 = g + k[a][2 * b + 1];
                 const float w0 = wx[a] * wy[b] * wz[0], w1 = wx[a] * wy[b] * wz[1];
-                f0 = fmaf(w0, __ldg(c0), fmaf(w1, __ldg(c1), f0));
-                f1 = fmaf(w0, __ldg(c0 + n), fmaf(w1, __ldg(c1 + n), f1));
-                f2 = fmaf(w0, __ldg(c0 + 2 * n), fmaf(w1, __ldg(c1 + 2 * n), f2));
+                f0 = fmaf(w0, c0[0], fmaf(w1, c1[0], f0));
+                f1 = fmaf(w0, c0[n], fmaf(w1, c1[n], f1));
+                f2 = fmaf(w0, c0[2 * n], fmaf(w1, c1[2 * n], f2));
             }
     }
     p0 = fmaf(kick, f0, p0);
