@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(512, 3) k_deposit_tiled(const uint32_t* __rest
     rho += (int64_t)blockIdx.y << (3 * logn);
     const int ntz = (1 << lognp) / D::TZ, nty = (1 << lognp) / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
-    const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
+    const int ox = D::box_x(bx), oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
     const int64_t count = (int64_t)1 << (3 * lognp);
     tile_zero<D::CELLS>(lo);
     __syncthreads();
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(512, 3) k_deposit_tiled(const uint32_t* __rest
         return ((((int64_t)(bx * D::TX + lx) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
     };
     const float quanta = mass * kTileQuanta;
-    uint32_t sum = 0;
+    TileAdds adds;
     // positions are loaded one iteration ahead (their latency overlaps the deposit)
     int64_t idn = pid(threadIdx.x);
     uint32_t nu0 = 0, nu1 = 0, nu2 = 0;
@@ -140,13 +140,13 @@ __global__ void __launch_bounds__(512, 3) k_deposit_tiled(const uint32_t* __rest
             nu1 = x[count + idn];
             nu2 = x[2 * count + idn];
         }
-        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
+        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, adds);
     }
-    tile_close<D>(lo, rho, ox, oy, oz, logn, sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, adds, [&] {
         for (int e = threadIdx.x; e < D::PER; e += 512) {
             const int64_t id = pid(e);
             tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
-                                  oz, quanta, sum);
+                                  oz, quanta, adds);
         }
     });
 }
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(512, 3) k_deposit_sweep(const uint32_t* __rest
     const int64_t count = (int64_t)1 << (3 * lognp);
     const int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
-    const int ox = bx * D::TX - D::H, oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
+    const int ox = D::box_x(bx), oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
     tile_zero<D::CELLS>(lo);
     __syncthreads();
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
@@ -186,11 +186,11 @@ __global__ void __launch_bounds__(512, 3) k_deposit_sweep(const uint32_t* __rest
         sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);
-    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.adds, [&] {
         for (int lx = 0; lx < D::TX; ++lx) {
             const int64_t id = id0 + lx * xstride;
             tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
-                                  oz, quanta, sc.sum);
+                                  oz, quanta, sc.adds);
         }
     });
 }

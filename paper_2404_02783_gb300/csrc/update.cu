@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* x, uint3
     }
     constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
-    const int ox = bx * D::TX * R - D::H, oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
+    const int ox = D::box_x(bx), oy = by * D::TY * R - D::H, oz = bz * D::TZ * R - D::HZ;
     launch_next();
     tile_zero<D::CELLS>(lo);
     wait_previous();
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* x, uint3
         return ((((int64_t)(bx * D::TX + lx) << lognp) + by * D::TY + ly) << lognp) + bz * D::TZ + lz;
     };
     const float quanta = mass * kTileQuanta;
-    uint32_t sum = 0;
+    TileAdds adds;
     // the next particle is loaded one iteration ahead (its latency overlaps this one's work)
     int64_t idn = pid(threadIdx.x);
     uint32_t nu0 = 0, nu1 = 0, nu2 = 0;
@@ -80,13 +80,13 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* x, uint3
         xo[id] = u0;
         xo[count + id] = u1;
         xo[2 * count + id] = u2;
-        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sum);
+        tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, adds);
     }
-    tile_close<D>(lo, rho, ox, oy, oz, logn, sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, adds, [&] {
         for (int e = threadIdx.x; e < D::PER; e += 512) {
             const int64_t id = pid(e);
             tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
-                                  oy, oz, quanta, sum);
+                                  oy, oz, quanta, adds);
         }
     });
 }
@@ -99,12 +99,12 @@ __device__ __forceinline__ void sweep_again(uint32_t* lo, const uint32_t* xo, fl
     constexpr int64_t count = (int64_t)1 << (3 * LOGN);
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
-    uint32_t sum = 0;
+    TileAdds adds;
     for (int lx = 0; lx < D::TX; ++lx) {
         const int64_t id = ((((int64_t)(bx * D::TX + lx) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
         tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], LOGN,
-                              1.0f / (float)(1u << (32 - LOGN)), bx * D::TX - D::H, by * D::TY - D::H,
-                              bz * D::TZ - D::HZ, quanta, sum);
+                              1.0f / (float)(1u << (32 - LOGN)), D::box_x(bx), by * D::TY - D::H,
+                              bz * D::TZ - D::HZ, quanta, adds);
     }
 }
 template <int XC, int LOGN>
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* x,
     }
     constexpr int ntz = np / D::TZ, nty = np / D::TY;
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
-    const int ox = bx * D::TX - D::H, oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
+    const int ox = D::box_x(bx), oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
     launch_next();
     tile_zero<D::CELLS>(lo);
     wait_previous();
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* x,
         sweep_deposit<D>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, sc);
     }
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);  // the carried plane of the row's last particle
-    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.sum, [&] {
+    tile_close<D>(lo, rho, ox, oy, oz, logn, sc.adds, [&] {
         // a call where the three components fill the registers (in line its values spill in the loop:
         // 1764 us against 1724); with the potential alone the call costs more (1730 us against 1563)
         if constexpr (FD) sweep_again<XC, LOGN>(lo, xo, rho, quanta);
