@@ -143,11 +143,13 @@ __global__ void __launch_bounds__(512, 3) k_deposit_tiled(const uint32_t* __rest
         tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, adds);
     }
     tile_close<D>(lo, rho, ox, oy, oz, logn, adds, [&] {
-        for (int e = threadIdx.x; e < D::PER; e += 512) {
-            const int64_t id = pid(e);
-            tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
-                                  oz, quanta, adds);
-        }
+        tile_again<D>(lo, rho, ox, oy, oz, logn, [&] {
+            for (int e = threadIdx.x; e < D::PER; e += 512) {
+                const int64_t id = pid(e);
+                tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+                                      oz, quanta, adds);
+            }
+        });
     });
 }
 
@@ -187,11 +189,13 @@ __global__ void __launch_bounds__(512, 3) k_deposit_sweep(const uint32_t* __rest
     }
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);
     tile_close<D>(lo, rho, ox, oy, oz, logn, sc.adds, [&] {
-        for (int lx = 0; lx < D::TX; ++lx) {
-            const int64_t id = id0 + lx * xstride;
-            tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
-                                  oz, quanta, sc.adds);
-        }
+        tile_again<D>(lo, rho, ox, oy, oz, logn, [&] {
+            for (int lx = 0; lx < D::TX; ++lx) {
+                const int64_t id = id0 + lx * xstride;
+                tile_deposit<D, true>(lo, rho, x[id], x[count + id], x[2 * count + id], logn, inv_cell_ticks, ox, oy,
+                                      oz, quanta, sc.adds);
+            }
+        });
     });
 }
 

@@ -83,11 +83,13 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit(const uint32_t* x, uint3
         tile_deposit<D, false>(lo, rho, u0, u1, u2, logn, inv_cell_ticks, ox, oy, oz, quanta, adds);
     }
     tile_close<D>(lo, rho, ox, oy, oz, logn, adds, [&] {
-        for (int e = threadIdx.x; e < D::PER; e += 512) {
-            const int64_t id = pid(e);
-            tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
-                                  oy, oz, quanta, adds);
-        }
+        tile_again<D>(lo, rho, ox, oy, oz, logn, [&] {
+            for (int e = threadIdx.x; e < D::PER; e += 512) {
+                const int64_t id = pid(e);
+                tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], logn, inv_cell_ticks, ox,
+                                      oy, oz, quanta, adds);
+            }
+        });
     });
 }
 
@@ -98,14 +100,16 @@ __device__ __forceinline__ void sweep_again(uint32_t* lo, const uint32_t* xo, fl
     constexpr int np = 1 << LOGN, ntz = np / D::TZ, nty = np / D::TY;
     constexpr int64_t count = (int64_t)1 << (3 * LOGN);
     const int bz = blockIdx.x % ntz, by = (blockIdx.x / ntz) % nty, bx = blockIdx.x / (ntz * nty);
+    const int ox = D::box_x(bx), oy = by * D::TY - D::H, oz = bz * D::TZ - D::HZ;
     const int lz = threadIdx.x % D::TZ, ly = threadIdx.x / D::TZ;
     TileAdds adds;
-    for (int lx = 0; lx < D::TX; ++lx) {
-        const int64_t id = ((((int64_t)(bx * D::TX + lx) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
-        tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], LOGN,
-                              1.0f / (float)(1u << (32 - LOGN)), D::box_x(bx), by * D::TY - D::H,
-                              bz * D::TZ - D::HZ, quanta, adds);
-    }
+    tile_again<D>(lo, rho, ox, oy, oz, LOGN, [&] {
+        for (int lx = 0; lx < D::TX; ++lx) {
+            const int64_t id = ((((int64_t)(bx * D::TX + lx) << LOGN) + by * D::TY + ly) << LOGN) + bz * D::TZ + lz;
+            tile_deposit<D, true>(lo, rho, xo[id], xo[count + id], xo[2 * count + id], LOGN,
+                                  1.0f / (float)(1u << (32 - LOGN)), ox, oy, oz, quanta, adds);
+        }
+    });
 }
 template <int XC, int LOGN>
 __device__ __noinline__ void sweep_again_call(uint32_t* lo, const uint32_t* xo, float* rho, float quanta) {
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(512, 2) k_ikd_deposit_sweep(const uint32_t* x,
     if (sc.dnext >= 0) sweep_carried<D>(lo, sc);  // the carried plane of the row's last particle
     tile_close<D>(lo, rho, ox, oy, oz, logn, sc.adds, [&] {
         // a call where the three components fill the registers (in line its values spill in the loop:
-        // 1764 us against 1724); with the potential alone the call costs more (1730 us against 1563)
+        // 1764 us against 1724); with the potential alone the call costs more (1680 us against 1501)
         if constexpr (FD) sweep_again<XC, LOGN>(lo, xo, rho, quanta);
         else sweep_again_call<XC, LOGN>(lo, xo, rho, quanta);
     });

@@ -42,10 +42,10 @@ __device__ __forceinline__ CicF cic_ticks(uint32_t u, int logn, float inv_cell_t
 // additions as long as no cell reaches 256 mass units.  The additions return nothing and test
 // nothing; instead the sum of all cells is compared with the sum of all additions, both in 64
 // bits, before the tile is flushed: each wrap of a 32-bit cell takes exactly 2^32 from the
-// former.  A tile that fails the comparison (a cell of 256 times the mean density) is
-// accumulated again from the positions just written, each wrap seen in an addition's return value
-// and added to the global mesh as its 256 mass units (2^32 quanta).  A cell wraps up to 31 times;
-// a whole 256 on a sum in the same binade is exact, so this rounds once a doubling.
+// former.  In a tile that fails the comparison (a cell of 256 times the mean density) the words
+// are the cells' totals modulo 2^32 and go to the mesh as such; the particles are added again from
+// the positions just written, in steps of 2^12 quanta, which gives the wraps (tile_wraps), and a
+// cell's h wraps, 256 h mass units, are added to the mesh at once.
 // The box starts HZ = 4 cells below the tile in z so that its rows are made of 16-byte
 // chunks aligned in the mesh: the flush adds four cells per vector reduction.
 template <int R, int XC = 16>
@@ -91,18 +91,14 @@ __device__ __forceinline__ void tile_add(uint32_t* lo, int c, float w, TileAdds&
     atomicAdd(lo + c, v);
     t.sum += v;
 }
-// The mesh cell is found from the tile's only when a cell wraps: its address is not held otherwise.
-template <class D>
-__device__ __forceinline__ void tile_add_wrapping(uint32_t* lo, int c, float w, float* __restrict__ rho, int ox, int oy,
-                                                  int oz, int logn) {
-    const uint32_t v = __float2uint_rn(w);
-    const uint32_t old = atomicAdd(lo + c, v);
-    if (old + v < old) {
-        const int nm = (1 << logn) - 1, row = c / D::DZ;
-        atomicAdd(rho + ((((uint32_t)((ox + row / D::DY) & nm) << logn) + (uint32_t)((oy + row % D::DY) & nm)) << logn) +
-                      ((oz + c % D::DZ) & nm),
-                  256.0f);
-    }
+// The second accumulation of a tile counts in steps of 2^kCoarse quanta.  A cell of total T, made
+// of N <= 8192 additions, then holds S with T - S 2^12 in [0, N 2^12), at most 2^25, widened by the
+// few quanta an addition by which the sweeps' merged weights may round apart from the particles'
+// own.  The first accumulation's word is T mod 2^32; with its top bit the number of wraps,
+// floor(T / 2^32) <= 32, is that of S 2^12 - top 2^31 + 2^30, which stays 2^29 clear of either end.
+constexpr int kCoarse = 12;
+__device__ __forceinline__ float tile_wraps(uint32_t S, unsigned top) {
+    return 256.0f * (float)(((int)S - (int)(top << (31 - kCoarse)) + (1 << (30 - kCoarse))) >> (32 - kCoarse));
 }
 
 template <int WORDS>
@@ -134,8 +130,8 @@ __device__ __forceinline__ void tile_deposit(uint32_t* lo, float* __restrict__ r
                 const float wab = quanta * wx[a] * wy[b];
                 const int c = c0 + (a * D::DY + b) * D::DZ;
                 if (AGAIN) {
-                    tile_add_wrapping<D>(lo, c, wab * wz[0], rho, ox, oy, oz, logn);
-                    tile_add_wrapping<D>(lo, c + 1, wab * wz[1], rho, ox, oy, oz, logn);
+                    atomicAdd(lo + c, __float2uint_rn(wab * wz[0]) >> kCoarse);
+                    atomicAdd(lo + c + 1, __float2uint_rn(wab * wz[1]) >> kCoarse);
                 } else {
                     tile_add(lo, c, wab * wz[0], t);
                     tile_add(lo, c + 1, wab * wz[1], t);
@@ -165,28 +161,61 @@ __device__ __forceinline__ void for_chunks(int first, int last, F f) {
     for (int lx = first + l0; lx <= last; lx += D::PLANES) f((lx * D::DY + ly) * D::CZ + lz4, lx, ly, lz4);
 }
 
-// Adds the cells of the tile's planes first..last (box origin o*, oz a multiple of 4, rho 16-byte
-// aligned) to rho, four z-cells per reduction.
+// Mesh cell of the first of the tile's chunk (lx, ly, lz4); box origin o*, oz a multiple of 4.
+__device__ __forceinline__ uint32_t chunk_cell(int lx, int ly, int lz4, int ox, int oy, int oz, int logn) {
+    const int nm = (1 << logn) - 1;
+    return ((((uint32_t)((ox + lx) & nm) << logn) + (uint32_t)((oy + ly) & nm)) << logn) + ((oz + 4 * lz4) & nm);
+}
+
+// Adds the cells of the tile's planes first..last to rho (16-byte aligned), four z-cells per
+// reduction.
 template <class D>
 __device__ __forceinline__ void tile_flush(const uint32_t* lo, float* __restrict__ rho, int ox, int oy, int oz,
                                            int logn, int first, int last) {
-    const int nm = (1 << logn) - 1;
     for_chunks<D>(first, last, [&](int c, int lx, int ly, int lz4) {
         const uint4 l = reinterpret_cast<const uint4*>(lo)[c];
         if (l.x | l.y | l.z | l.w)
-            red_add_v4(rho + ((((uint32_t)((ox + lx) & nm) << logn) + (uint32_t)((oy + ly) & nm)) << logn) +
-                           ((oz + 4 * lz4) & nm),
+            red_add_v4(rho + chunk_cell(lx, ly, lz4, ox, oy, oz, logn),
                        make_float4(__uint2float_rn(l.x) * kTileQuantum, __uint2float_rn(l.y) * kTileQuantum,
                                    __uint2float_rn(l.z) * kTileQuantum, __uint2float_rn(l.w) * kTileQuantum));
     });
 }
 
+// Ends a tile in which cells passed 2^32 quanta: the words are added to rho, their top bits kept
+// (four a chunk; a thread has at most DX / PLANES of them), the tile is accumulated again in coarse
+// steps (add() deposits the thread's particles from their written positions with AGAIN) and the
+// wraps are added.
+template <class D, class F>
+__device__ __forceinline__ void tile_again(uint32_t* lo, float* __restrict__ rho, int ox, int oy, int oz, int logn,
+                                           F add) {
+    static_assert(4 * ((D::DX + D::PLANES - 1) / D::PLANES) <= 64, "top bits of a thread's chunks");
+    tile_flush<D>(lo, rho, ox, oy, oz, logn, 0, D::DX - 1);
+    unsigned long long tops = 0;
+    for_chunks<D>(0, D::DX - 1, [&](int c, int, int, int) {
+        const uint4 l = reinterpret_cast<const uint4*>(lo)[c];
+        tops = tops << 4 | (l.x >> 31) << 3 | (l.y >> 31) << 2 | (l.z >> 31) << 1 | l.w >> 31;
+        reinterpret_cast<uint4*>(lo)[c] = make_uint4(0u, 0u, 0u, 0u);
+    });
+    __syncthreads();
+    add();
+    __syncthreads();
+    int left = 0;  // chunks of the thread that follow
+    for_chunks<D>(0, D::DX - 1, [&](int, int, int, int) { ++left; });
+    for_chunks<D>(0, D::DX - 1, [&](int c, int lx, int ly, int lz4) {
+        const uint4 s = reinterpret_cast<const uint4*>(lo)[c];
+        const unsigned t = (unsigned)(tops >> (4 * --left));
+        const float4 v = make_float4(tile_wraps(s.x, t >> 3 & 1u), tile_wraps(s.y, t >> 2 & 1u),
+                                     tile_wraps(s.z, t >> 1 & 1u), tile_wraps(s.w, t & 1u));
+        if (v.x + v.y + v.z + v.w > 0.0f) red_add_v4(rho + chunk_cell(lx, ly, lz4, ox, oy, oz, logn), v);
+    });
+}
+
 // Ends a tile: compares the sum of its cells with the sum of all additions (`adds` of every
-// thread) and flushes it, after accumulating it again when they differ (redo() deposits the
-// thread's particles from their written positions with AGAIN).  Every thread of the CTA calls it.
+// thread) and flushes it, or calls again(), which ends in tile_again, when they differ.  Every
+// thread of the CTA calls it.
 template <class D, class F>
 __device__ __forceinline__ void tile_close(uint32_t* lo, float* __restrict__ rho, int ox, int oy, int oz, int logn,
-                                           const TileAdds& adds, F redo) {
+                                           const TileAdds& adds, F again) {
     __shared__ unsigned long long missing;
     __shared__ int span[2];
     if (threadIdx.x == 0) {
@@ -216,15 +245,8 @@ __device__ __forceinline__ void tile_close(uint32_t* lo, float* __restrict__ rho
     if ((threadIdx.x & 31) == 0)
         atomicAdd(&missing, (unsigned long long)l0 + ((unsigned long long)l1 << 16) + ((unsigned long long)l2 << 32));
     __syncthreads();
-    if (missing == 0) {
-        tile_flush<D>(lo, rho, ox, oy, oz, logn, first, last);
-        return;
-    }
-    tile_zero<D::CELLS>(lo);
-    __syncthreads();
-    redo();
-    __syncthreads();
-    tile_flush<D>(lo, rho, ox, oy, oz, logn, first, last);
+    if (missing == 0) tile_flush<D>(lo, rho, ox, oy, oz, logn, first, last);
+    else again();
 }
 
 // Deposit of a thread walking its lattice row along x (R = 1).  The next particle usually
