@@ -92,15 +92,14 @@ __global__ void __launch_bounds__(256) k_deposit_ticks(const uint32_t* __restric
         const int ix[2] = {cx.i0, cx.i1}, iy[2] = {cy.i0, cy.i1}, iz[2] = {cz.i0, cz.i1};
         const int pos = cz.i0 & 3;
         if (V4 && pos != 3) {
-            const float4 z = make_float4(pos == 0 ? wz[0] : 0.f, pos == 0 ? wz[1] : pos == 1 ? wz[0] : 0.f,
-                                         pos == 1 ? wz[1] : pos == 2 ? wz[0] : 0.f, pos == 2 ? wz[1] : 0.f);
 #pragma unroll
             for (int a = 0; a < 2; ++a)
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
-                    const float wab = mass * wx[a] * wy[b];
+                    const float wab = mass * wx[a] * wy[b], v0 = wab * wz[0], v1 = wab * wz[1];
                     red_add_v4(rho + ((size_t)ix[a] * n + iy[b]) * n + (cz.i0 - pos),
-                               make_float4(wab * z.x, wab * z.y, wab * z.z, wab * z.w));
+                               make_float4(pos == 0 ? v0 : 0.f, pos == 0 ? v1 : pos == 1 ? v0 : 0.f,
+                                           pos == 1 ? v1 : pos == 2 ? v0 : 0.f, pos == 2 ? v1 : 0.f));
                 }
         } else {
 #pragma unroll
