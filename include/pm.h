@@ -486,6 +486,9 @@ pm_status pm_cell_sort_static(const void* x, int64_t count, int precision, int n
  * Newton-Raphson iteration for 1/d from the FP32 reciprocal, two steps, times a.  d must
  * be in the FP32 normal range.  Exposed so that it can be compared with the division. */
 pm_status pm_div_mode_check(const double* a, const double* d, int64_t count, double* out, void* stream);
+/* The same for the FP32 divide (device float arrays): the quotient by the approximate reciprocal
+ * and one correction from its remainder.  d in 2^-126 .. 2^126, |a| above 2^-100 (or 0). */
+pm_status pm_div_mode_check_f32(const float* a, const float* d, int64_t count, float* out, void* stream);
 
 /* 3D real-to-complex FFT of real[n][n][n] into spec (layout above), unnormalised. */
 pm_status pm_fft_r2c(const void* real, void* spec, int n, int precision, void* stream);

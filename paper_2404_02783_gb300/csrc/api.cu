@@ -2445,6 +2445,13 @@ pm_status pm_div_mode_check(const double* a, const double* d, int64_t count, dou
     return PM_OK;
 }
 
+pm_status pm_div_mode_check_f32(const float* a, const float* d, int64_t count, float* out, void* stream) {
+    if (count < 0 || (count > 0 && (!a || !d || !out))) return fail(PM_ERR_INVALID_ARG, "bad arguments");
+    PM_TRY(check_device());
+    PM_CK(div_mode_check(a, d, count, out, (cudaStream_t)stream));
+    return PM_OK;
+}
+
 pm_status pm_fft_r2c(const void* real, void* spec, int n, int precision, void* stream) {
     if (!real || !spec) return fail(PM_ERR_INVALID_ARG, "null pointer");
     if (!pow2(n) || n < 16 || n > 1024) return fail(PM_ERR_INVALID_ARG, "n must be a power of two in 16..1024");

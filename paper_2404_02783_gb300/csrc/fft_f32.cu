@@ -21,6 +21,19 @@ template cudaError_t fft_plane<float>(float2*, float2*, float2*, int, int, const
 template cudaError_t fft_middle<float>(float2*, float2*, float2*, int, int, const SpecOp&, unsigned*, int,
                                        cudaStream_t);
 
+// div_mode<float> applied element by element (the check of its corrected quotient).
+__global__ void k_div_mode_f32(const float* __restrict__ a, const float* __restrict__ d, int64_t count,
+                               float* __restrict__ out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = div_mode<float>(a[i], d[i]);
+}
+cudaError_t div_mode_check(const float* a, const float* d, int64_t count, float* out, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    const int64_t blocks = std::min<int64_t>((count + 255) / 256, 152 * 8);
+    k_div_mode_f32<<<(unsigned)blocks, 256, 0, st>>>(a, d, count, out);
+    return cudaGetLastError();
+}
+
 // out[b] = sum over rows r of rows[r nbins + b]: the per-CTA bin sums of the binning x pass,
 // combined in a fixed order (one warp a bin: lane l sums rows l, l + 32, ... in turn, then a
 // fixed shuffle tree), so the result does not depend on the scheduling.

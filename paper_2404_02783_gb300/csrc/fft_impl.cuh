@@ -52,14 +52,16 @@ __device__ __forceinline__ void load_stage_twiddles(cplx<T>* tw) {
     }
 }
 
-// a / d in the per-mode operators, d positive and in the FP32 normal range (about 1.2e-38 ..
-// 3.4e38; the operators' k^2 and constraint denominators are).  The division's own instruction
-// sequence, with its check for operands out of range, is a good part of what the x pass issues a
-// mode.  FP32: the quotient by the approximate reciprocal and one Newton-Raphson correction from
-// its remainder, which leaves the rounding of the last operation.  FP64 divides are slower still:
-// the reciprocal of d by the iteration for 1/d, r <- r + r (1 - d r), started from the FP32
-// reciprocal of d and run twice (the relative error squares each time: ~2^-23, then ~2^-46, then
-// below the FP64 rounding), times a.  pm_div_mode_check compares it with the division.
+// a / d in the per-mode operators.  The division's own instruction sequence, with its check for
+// operands out of range, is a good part of what the x pass issues a mode.  FP32: the quotient by
+// the approximate reciprocal and one Newton-Raphson correction from its remainder, which leaves
+// the rounding of the last operation: the correctly rounded quotient but for a few in a million,
+// neighbours of it.  d in 2^-126 .. 2^126 (the approximate reciprocal of more is 0) and |a| above
+// 2^-100, or 0 (the remainder is a's last bits); the operators' k^2, constraint denominators and
+// numerators lie far inside.  FP64 divides are slower still: the reciprocal of d by the iteration
+// for 1/d, r <- r + r (1 - d r), started from the FP32 reciprocal of d, which must be normal, and
+// run twice (the relative error squares each time: ~2^-23, then ~2^-46, then below the FP64
+// rounding), times a.  pm_div_mode_check and pm_div_mode_check_f32 compare both with the division.
 template <typename T> __device__ __forceinline__ T div_mode(T a, T d) {
     const T r = __fdividef(1.0f, d), q = a * r;
     return fmaf(fmaf(-q, d, a), r, q);
