@@ -490,6 +490,12 @@ pm_status pm_div_mode_check(const double* a, const double* d, int64_t count, dou
  * and one correction from its remainder.  d in 2^-126 .. 2^126, |a| above 2^-100 (or 0). */
 pm_status pm_div_mode_check_f32(const float* a, const float* d, int64_t count, float* out, void* stream);
 
+/* The unit complex Gaussians that an FP32 context draws from pairs of Philox words (Box-Muller in
+ * pairs of FP32 numbers), out[i] = (re, im) of words[i] = (w0, w1), count of each, 8-byte aligned:
+ * sqrt(-ln((w0 + 1/2) 2^-32)) exp(2 pi i (w1 + 1/2) 2^-32).  Exposed so that they can be compared
+ * with the FP64 values. */
+pm_status pm_phase_check(const uint32_t* words, int64_t count, float* out, void* stream);
+
 /* 3D real-to-complex FFT of real[n][n][n] into spec (layout above), unnormalised. */
 pm_status pm_fft_r2c(const void* real, void* spec, int n, int precision, void* stream);
 

@@ -35,7 +35,7 @@ EXPORTS = ("pm_workspace_size", "pm_init", "pm_destroy", "pm_ic_zeldovich", "pm_
            "pm_bispectrum_scratch_size", "pm_bispectrum", "pm_triangle_index", "pm_b1_gr_theory", "pm_step_factors", "pm_linear_power", "pm_cic_deposit", "pm_cic_interp",
            "pm_adjoint_scratch_size", "pm_adjoint_record", "pm_adjoint_run", "pm_loss_grad", "pm_displacement", "pm_positions", "pm_gr_history", "pm_set_state_gr", "pm_batch_workspace_size", "pm_batch_init", "pm_batch_destroy", "pm_batch_context", "pm_batch_ic",
            "pm_batch_step", "pm_batch_state", "pm_batch_power", "pm_batch_bias", "pm_batch_set_chunk", "pm_batch_autotune", "pm_batch_set_fft", "pm_batch_tuning",
-           "pm_cell_sort_scratch_size", "pm_cell_sort", "pm_cell_sort_static", "pm_div_mode_check", "pm_div_mode_check_f32", "pm_fft_r2c", "pm_fft_c2r", "pm_version", "pm_last_error")
+           "pm_cell_sort_scratch_size", "pm_cell_sort", "pm_cell_sort_static", "pm_div_mode_check", "pm_div_mode_check_f32", "pm_phase_check", "pm_fft_r2c", "pm_fft_c2r", "pm_version", "pm_last_error")
 
 
 class PMError(RuntimeError):
@@ -130,6 +130,7 @@ def lib():
         "pm_cell_sort_static": (vp, i64, i, i, vp, vp, vp),
         "pm_div_mode_check": (vp, vp, i64, vp, vp),
         "pm_div_mode_check_f32": (vp, vp, i64, vp, vp),
+        "pm_phase_check": (vp, i64, vp, vp),
         "pm_fft_r2c": (vp, vp, i, i, vp),
         "pm_fft_c2r": (vp, vp, i, i, vp),
     }
@@ -418,6 +419,10 @@ def pm_div_mode_check(a, d, out, stream=None):
 
 def pm_div_mode_check_f32(a, d, out, stream=None):
     _check(lib().pm_div_mode_check_f32(_ptr(a), _ptr(d), int(a.numel()), _ptr(out), _stream(stream)))
+
+
+def pm_phase_check(words, out, stream=None):
+    _check(lib().pm_phase_check(_ptr(words), int(words.numel()) // 2, _ptr(out), _stream(stream)))
 
 
 def pm_fft_r2c(real, spec, n, precision, stream=None):

@@ -2452,6 +2452,14 @@ pm_status pm_div_mode_check_f32(const float* a, const float* d, int64_t count, f
     return PM_OK;
 }
 
+pm_status pm_phase_check(const uint32_t* words, int64_t count, float* out, void* stream) {
+    if (count < 0 || (count > 0 && (!words || !out)) || (uintptr_t)words % 8 || (uintptr_t)out % 8)
+        return fail(PM_ERR_INVALID_ARG, "bad arguments");
+    PM_TRY(check_device());
+    PM_CK(phase_check(words, count, out, (cudaStream_t)stream));
+    return PM_OK;
+}
+
 pm_status pm_fft_r2c(const void* real, void* spec, int n, int precision, void* stream) {
     if (!real || !spec) return fail(PM_ERR_INVALID_ARG, "null pointer");
     if (!pow2(n) || n < 16 || n > 1024) return fail(PM_ERR_INVALID_ARG, "n must be a power of two in 16..1024");

@@ -776,7 +776,7 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 }
 
 // Unit complex Gaussian of mode draw (r.x, r.y) by the Box-Muller transform: in FP64, and for
-// FP32 phases in pairs of FP32 numbers (dfloat.cuh), which round to the same phases but for 3 in
+// FP32 phases in pairs of FP32 numbers (dfloat.cuh), which round to the same phases but for one in
 // ten thousand (neighbouring FP32 numbers there).  At 512^3 the FP64 logarithm, square root and
 // sine took 9.4 ms of the 16.5 ms of the initial conditions; this is bound by issue instead.
 __device__ __forceinline__ void unit_gaussian(uint4 r, double2& g) {
@@ -839,6 +839,21 @@ cudaError_t noise(cplx<T>* spec, int n, const uint64_t* seeds, int nfields, cuda
 }
 template cudaError_t noise<float>(float2*, int, const uint64_t*, int, cudaStream_t);
 template cudaError_t noise<double>(double2*, int, const uint64_t*, int, cudaStream_t);
+
+// The FP32 phases of pairs of Philox words, by themselves.
+__global__ void k_phase_check(const uint2* __restrict__ words, int64_t count, float2* __restrict__ out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint2 w = words[i];
+        float2 g;
+        unit_gaussian(make_uint4(w.x, w.y, 0u, 0u), g);
+        out[i] = g;
+    }
+}
+cudaError_t phase_check(const uint32_t* words, int64_t count, float* out, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    k_phase_check<<<grid_for(count, 256), 256, 0, st>>>((const uint2*)words, count, (float2*)out);
+    return cudaGetLastError();
+}
 
 // ---------------------------------------------------------------- GR displacement combination
 // xi = x_GR - x_N on the coarse lattice (exact minimum image on ticks), trilinear in

@@ -43,6 +43,8 @@ cudaError_t ic_place2(void* x, void* p, void* const* psi1, void* const* psi2, in
                       double D2, double pfac1, double pfac2, double box, cudaStream_t st);
 template <typename T>
 cudaError_t noise(cplx<T>* spec, int n, const uint64_t* seeds, int nfields, cudaStream_t st);  // seeds: host, one a field
+// out[2 i], out[2 i + 1] = the FP32 unit complex Gaussian of the words[2 i], words[2 i + 1].
+cudaError_t phase_check(const uint32_t* words, int64_t count, float* out, cudaStream_t st);
 cudaError_t combine(void* xt, const void* xg, const void* xn, void* xi_out, int npt, int npc, int precision,
                     cudaStream_t st);
 cudaError_t fill(void* a, int64_t count, int precision, double v, cudaStream_t st);
