@@ -1973,6 +1973,7 @@ pm_status batch_zeldovich(pm_batch* b, const uint64_t* seeds, int flags) {
     const double D = pmhost::growth_D(b->cosmo, a), f = pmhost::growth_f(b->cosmo, a), E = pmhost::E(b->cosmo, a);
     // the z passes' grid takes np rows a realisation in its y dimension
     const int group = std::min(b->B, 65535 / np);
+    std::vector<double> boxes(group);
     for (int r0 = 0; r0 < b->B; r0 += group) {
         const int c = std::min(group, b->B - r0);
         const double* kf = (const double*)b->at(b->KF) + r0;
@@ -1998,8 +1999,9 @@ pm_status batch_zeldovich(pm_batch* b, const uint64_t* seeds, int flags) {
         const float2* in[3] = {s[1], s[2], s[0]};
         PM_CK(z_c2r<float>(in, psi, 3, np, c, 4u, 0.0, b->st, kf));
         void* ps[3] = {psi[0], psi[1], psi[2]};
+        for (int r = 0; r < c; ++r) boxes[r] = b->views[r0 + r]->cfg.box;
         PM_CK(ic_place((uint32_t*)b->at(b->X) + r0 * 3 * np3, (float*)b->at(b->P) + r0 * 3 * np3, ps, np, PM_FP32_FIXED, D,
-                       a * a * E * f * D, 1.0, b->st, c, (const double*)b->at(b->SCALE) + r0));
+                       a * a * E * f * D, 1.0, b->st, c, boxes.data()));
     }
     for (pm_ctx* v : b->views) {
         v->step = 0;

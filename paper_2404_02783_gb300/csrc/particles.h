@@ -32,9 +32,9 @@ cudaError_t interp_kick_drift_deposit(void* x, void* p, int np, int precision, i
                                       double drift, double box, double mass, void* rho, cudaStream_t st,
                                       int nfields = 1, const double* scale_arr = nullptr, void* x_out = nullptr,
                                       double fd_inv_d = 0.0);
-// nfields > 1 (FP32): a batch stored back to back, box given per field as scale_arr[f] = 2^32 / L_f.
+// nfields > 1 (FP32): a batch stored back to back, boxes (host) giving each field's box.
 cudaError_t ic_place(void* x, void* p, void* const* psi, int np, int precision, double D, double pfac, double box,
-                     cudaStream_t st, int nfields = 1, const double* scale_arr = nullptr);
+                     cudaStream_t st, int nfields = 1, const double* boxes = nullptr);
 // Second-order LPT source, accumulated over three stages, one per displacement component c:
 // d[j] = d Psi1_c / d x_j on the np^3 lattice; s and a are np^3 meshes (ctx precision).
 cudaError_t lpt2_source(int stage, void* const* d, void* s, void* a, int64_t count, int precision, cudaStream_t st);
