@@ -2012,6 +2012,14 @@ pm_status batch_zeldovich(pm_batch* b, const uint64_t* seeds, int flags) {
     return PM_OK;
 }
 
+// A view as the batch stands: its place on the a-grid, and no density of its own kept (the batch's
+// passes and other views' may have written it).
+void batch_refresh_view(pm_batch* b, int r) {
+    b->views[r]->step = b->step;
+    b->views[r]->synced = b->synced;
+    b->views[r]->rho_valid = false;
+}
+
 void batch_drop_graph(pm_batch* b) {
     if (b->exec) {
         cudaStreamSynchronize(b->cap);
@@ -2135,9 +2143,7 @@ pm_status pm_batch_destroy(pm_batch* b) {
 
 pm_status pm_batch_context(pm_batch* b, int r, pm_ctx** view) {
     if (!b || !view || r < 0 || r >= b->B) return fail(PM_ERR_INVALID_ARG, "bad batch index");
-    b->views[r]->step = b->step;
-    b->views[r]->synced = b->synced;
-    b->views[r]->rho_valid = false;
+    batch_refresh_view(b, r);
     // operations on a view may overwrite its slice of the batch density
     b->rho_valid = false;
     *view = b->views[r];
@@ -2312,6 +2318,7 @@ pm_status pm_batch_power(pm_batch* b, int nbins, const double* edges, int deconv
                          double* nmodes_out) {
     if (!b) return fail(PM_ERR_INVALID_ARG, "null batch");
     PM_TRY(check_edges(nbins, edges));
+    for (int r = 0; r < b->B; ++r) batch_refresh_view(b, r);
     // one launch a pass over a group of realisations (one realisation at a time took ten launches
     // of a few microseconds and two synchronisations each)
     const int n = b->cfg.nmesh, M = n / 2;
