@@ -728,7 +728,7 @@ template <typename T, int LOGN, int THREADS_> struct MidShape {
     static constexpr int CB = THREADS / QN;  // columns of an x item
     static constexpr int ITEMS = N / RB;     // items of each phase per plane
     static constexpr int MINB = 1024 / THREADS;  // 64 registers a thread
-    typedef RowLayout<N, false> LAY;
+    typedef RowLayout<N> LAY;
     // twiddles + the larger of the y exchange (two rows buffers of RB rows) and the x exchange
     // (two sequences of N x (CB + 1))
     static constexpr int XWORDS = 2 * N * (CB + 1), YWORDS = 2 * RB * LAY::RS;
@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(PlaneShape<T, LOGN>::THREADS, PlaneShape<T, LO
     typedef cplx<T> C;
     typedef PlaneShape<T, LOGN> SH;
     constexpr int N = SH::N, M = SH::M, Q = SH::Q, SEQ = SH::SEQ, ROUNDS = SH::ROUNDS;
-    typedef RowLayout<N, false> LAY;  // a permutation within each row's N slots
+    typedef RowLayout<N> LAY;  // a permutation within each row's N slots
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tws = reinterpret_cast<C*>(smem_raw);
     const TwShared<C> tw{tws};
@@ -1334,8 +1334,6 @@ cudaError_t y_rows_grad3(cplx<T>* A, cplx<T>* B, cplx<T>* Cc, int64_t nrows, int
     PM_DISPATCH_LOGN(n, (y_grad3_n<T, LG>(A, B, A, B, Cc, nrows, kf, st, kf_arr, rows_per_field)))
 }
 
-// The fused middle passes (forward y, x with op, inverse y with the y gradient) on meshes of
-// 256^3 and up; cudaErrorNotSupported for other sizes (the caller runs the separate passes).
 // The fused middle passes (forward y, x with op, inverse y with the y gradient) on meshes of
 // 256^3 and up with CTAs of `threads` (256, 512 or 1024); cudaErrorNotSupported for other sizes
 // (the caller runs the separate passes).

@@ -112,10 +112,6 @@ __host__ __device__ __forceinline__ int ilog2(int n) {
     return l;
 }
 
-// Padded shared-memory index: one spare slot every 8 complex elements keeps the
-// strided Stockham stores free of shared-memory bank conflicts.
-__host__ __device__ __forceinline__ int spad(int i) { return i + (i >> 3); }
-
 // Signed wavenumber of FFT index i on an n-point axis: 0..n/2-1, -n/2..-1.
 __device__ __forceinline__ int signed_k(int i, int n) { return i < (n >> 1) ? i : i - n; }
 
