@@ -380,8 +380,8 @@ cudaError_t adj_kick_particles(const uint32_t* x, int64_t count, int n, float* v
                                const float* rho_bar, float K, float Km, float drift_next, float* lam_u,
                                cudaStream_t st) {
     const int logn = ilog2(n);
-    return launch_chained(k_adj_kick, dim3(blocks_for(count)), 256, 0, st, x, count, logn, (float)ldexp(1.0, -(32 - logn)), v,
-                          G, rho_bar, K, Km, drift_next, lam_u);
+    return launch_chained(k_adj_kick, dim3(blocks_for(count)), 256, 0, st, true, x, count, logn,
+                          (float)ldexp(1.0, -(32 - logn)), v, G, rho_bar, K, Km, drift_next, lam_u);
 }
 
 cudaError_t deposit_grad(const uint32_t* x, int64_t count, int n, const float* v, double inv_d, float* V,
@@ -411,8 +411,8 @@ cudaError_t deposit_vec(const uint32_t* x, int np, int n, const float* v, float*
     const int64_t threads = (int64_t)np * np * (np / run);
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     const float inv = (float)ldexp(1.0, -(32 - logn));
-    return launch_chained(n == np ? k_deposit_vec_rows<true> : k_deposit_vec_rows<false>, dim3(blocks), 256, 0, st, x, lognp,
-                          logn, run, inv, v, V[0], V[1], V[2]);
+    return launch_chained(n == np ? k_deposit_vec_rows<true> : k_deposit_vec_rows<false>, dim3(blocks), 256, 0, st, true,
+                          x, lognp, logn, run, inv, v, V[0], V[1], V[2]);
 }
 
 cudaError_t adj_combine(const float2* const* in, float2* out, int n, double kf, double coef, const float2* amp,

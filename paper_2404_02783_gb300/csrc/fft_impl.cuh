@@ -1120,12 +1120,20 @@ __global__ void __launch_bounds__(XShape<T, LOGN>::THREADS, AdjRes<T, LOGN>::MIN
 }
 
 // =============================================================== launchers
+// Passes whose launches overlap (launch_chained).  Not the FP64 ones of 64^3 and 128^3: blocks that are
+// placed while others still run pile up on the SMs that are free first, and these passes are bound by
+// each SM's few FP64 units (potential of a 64^3 mesh 53 us in order and 156 overlapping, 128^3 334
+// and 383; first-order step 102 and 109, 648 and 698).  At 32^3 every block finds an SM of its own (43
+// and 33 us), from 256^3 on there are many blocks for each (2576 and 2566).
+template <typename T, int LOGN> constexpr bool kOverlap = sizeof(T) == 4 || LOGN <= 5 || LOGN >= 8;
+
 template <typename T, int LOGN>
 cudaError_t z_r2c_n(const T* in, cplx<T>* out, int rows, cudaStream_t st, double sub, int kz_max) {
     typedef ZShape<T, LOGN> S;
     cudaError_t e = set_smem((const void*)k_z_r2c<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_z_r2c<T, LOGN>, dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st, in, out, (T)sub, kz_max);
+    return launch_chained(k_z_r2c<T, LOGN>, dim3(S::N / S::YB, rows), S::THREADS, S::SMEM, st, kOverlap<T, LOGN>, in, out,
+                          (T)sub, kz_max);
 }
 
 template <typename T, int LOGN>
@@ -1134,7 +1142,8 @@ cudaError_t z_c2r_n(const Ptr3<T>& P, int ncomp, int rows, unsigned mask, double
     typedef ZShape<T, LOGN> S;
     cudaError_t e = set_smem((const void*)k_z_c2r<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_z_c2r<T, LOGN>, dim3(S::N / S::YB, rows, ncomp), S::THREADS, S::SMEM, st, P, mask, (T)kf, kf_arr);
+    return launch_chained(k_z_c2r<T, LOGN>, dim3(S::N / S::YB, rows, ncomp), S::THREADS, S::SMEM, st, kOverlap<T, LOGN>, P,
+                          mask, (T)kf, kf_arr);
 }
 
 template <typename T, int LOGN, bool INV>
@@ -1143,7 +1152,8 @@ cudaError_t y_rows_n(const cplx<T>* in, cplx<T>* out, int64_t nrows, cudaStream_
     cudaError_t e = set_smem((const void*)k_y_rows<T, LOGN, INV>, S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t nblk = (nrows + S::RB - 1) / S::RB;
-    return launch_chained(k_y_rows<T, LOGN, INV>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, in, out, nrows);
+    return launch_chained(k_y_rows<T, LOGN, INV>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, kOverlap<T, LOGN>, in,
+                          out, nrows);
 }
 
 template <typename T, int LOGN>
@@ -1153,8 +1163,8 @@ cudaError_t y_grad3_n(const cplx<T>* A, const cplx<T>* B, cplx<T>* Ao, cplx<T>* 
     cudaError_t e = set_smem((const void*)k_y_grad3<T, LOGN>, S::SMEM);
     if (e != cudaSuccess) return e;
     const int64_t nblk = (nrows + S::RB - 1) / S::RB;
-    return launch_chained(k_y_grad3<T, LOGN>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, A, B, Ao, Bo, Co, nrows, (T)kf,
-                          kf_arr, rows_per_field);
+    return launch_chained(k_y_grad3<T, LOGN>, dim3((unsigned)nblk), S::THREADS, S::SMEM, st, kOverlap<T, LOGN>, A, B,
+                          Ao, Bo, Co, nrows, (T)kf, kf_arr, rows_per_field);
 }
 
 template <typename T, int LOGN>
@@ -1201,7 +1211,7 @@ cudaError_t x_cols_n(cplx<T>* data, cplx<T>* out2, int nplanes, const SpecOp& op
         grid = std::min<int64_t>(grid, std::min<int64_t>((int64_t)per_sm * num_sms(), op.acc_rows));
     }
     return launch_chained(k_x_cols<T, LOGN, KIND>, dim3((unsigned)grid, op.kind == OP_BIN ? op.bin_fields : 1), S::THREADS,
-                          smem, st, data, out2, op, nplanes);
+                          smem, st, kOverlap<T, LOGN>, data, out2, op, nplanes);
 }
 
 template <typename T, int LOGN, int THREADS>
@@ -1250,8 +1260,10 @@ cudaError_t plane_n(cplx<T>* A, cplx<T>* GX, cplx<T>* GY, int nplanes, const Spe
     if (e != cudaSuccess) return e;
     const int grid = (int)std::min<int64_t>((int64_t)per_sm * num_sms(), nplanes);
     if (op.kind == OP_GR)
-        return launch_chained(k_plane<T, LOGN, OP_GR>, dim3(grid), SH::THREADS, SH::SMEM, st, A, GX, GY, op, nplanes);
-    return launch_chained(k_plane<T, LOGN, OP_NEWTON>, dim3(grid), SH::THREADS, SH::SMEM, st, A, GX, GY, op, nplanes);
+        return launch_chained(k_plane<T, LOGN, OP_GR>, dim3(grid), SH::THREADS, SH::SMEM, st, kOverlap<T, LOGN>, A, GX,
+                              GY, op, nplanes);
+    return launch_chained(k_plane<T, LOGN, OP_NEWTON>, dim3(grid), SH::THREADS, SH::SMEM, st, kOverlap<T, LOGN>, A, GX,
+                          GY, op, nplanes);
 }
 
 template <typename T, int LOGN, bool GR, bool FD>
@@ -1261,8 +1273,8 @@ cudaError_t x_adj_k(const cplx<T>* V, cplx<T>* out, double kf, double coef, floa
     const size_t smem = sizeof(cplx<T>) * S::COL;
     cudaError_t e = set_smem((const void*)k_x_adj<T, LOGN, GR, FD>, smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(k_x_adj<T, LOGN, GR, FD>, dim3(S::N / S::CB, S::N / 2 + 1), S::THREADS, smem, st, V, out, kf, coef,
-                          (float4*)zero, zero ? nzero / 4 : 0, gr);
+    return launch_chained(k_x_adj<T, LOGN, GR, FD>, dim3(S::N / S::CB, S::N / 2 + 1), S::THREADS, smem, st, kOverlap<T, LOGN>, V,
+                          out, kf, coef, (float4*)zero, zero ? nzero / 4 : 0, gr);
 }
 
 template <typename T, int LOGN>

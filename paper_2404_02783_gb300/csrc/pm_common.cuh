@@ -30,8 +30,10 @@ __device__ __forceinline__ float load_ordered(const float* p) {
     return v;
 }
 
+// overlap = false: an ordinary launch.
 template <typename... K, typename... A>
-cudaError_t launch_chained(void (*fn)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+cudaError_t launch_chained(void (*fn)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool overlap,
+                           A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -39,7 +41,7 @@ cudaError_t launch_chained(void (*fn)(K...), dim3 grid, unsigned threads, size_t
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, fn, K(args)...);

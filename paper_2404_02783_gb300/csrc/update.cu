@@ -284,9 +284,9 @@ cudaError_t ikd_launch(const UpdateArgs& a) {
     }();
     cudaError_t e = set_smem_once((const void*)fn, smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(fn, dim3(blocks, a.nfields), 512, smem, a.st, (const uint32_t*)a.x, (uint32_t*)a.xo, (float*)a.p,
-                          (const float*)a.g, (float)a.kick, a.drift, a.scale0, a.scale_arr, (float)a.mass, (float*)a.rho,
-                          (float)a.inv_d);
+    return launch_chained(fn, dim3(blocks, a.nfields), 512, smem, a.st, true, (const uint32_t*)a.x, (uint32_t*)a.xo,
+                          (float*)a.p, (const float*)a.g, (float)a.kick, a.drift, a.scale0, a.scale_arr, (float)a.mass,
+                          (float*)a.rho, (float)a.inv_d);
 }
 
 // Meshes of 128^3 and up always fill the SMs with tiles of depth 16.
