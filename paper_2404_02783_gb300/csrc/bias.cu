@@ -7,8 +7,10 @@
 // (histograms of the cells that still match the chosen prefix), and of the cells equal to the
 // threshold the lowest-index ones fill the remaining places.  The digits are chosen on the
 // device, so nothing waits for the host between the passes.  When every cell equal to the
-// threshold is selected, which is the rule, the last pass only compares; otherwise the equal
-// cells are ranked by index (per-chunk counts, their scan, and warp ballots within each chunk).
+// threshold is selected the last pass only compares; otherwise the equal cells are ranked by
+// index (per-chunk counts, their scan, and warp ballots within each chunk), as in many 256^3
+// fields, where FP32 values near the threshold repeat (halo proxy and bias fit 305 us without the
+// ranking and 330 with it).
 //
 // Bound by the reads of the field: at 256^3 three histogram passes and one comparing pass.  With
 // eight-bit digits chosen on the host (four passes, four synchronisations) and a ranking pass

@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_bk_units(const 
 
 // The indicator fields I_b(x) = sum of exp(2 pi i n.x / m) over a bin's modes are even along every
 // axis and symmetric under the exchange of axes (a bin is a shell of |n|^2), so their triple sums
-// need one point of each orbit: 45,760 of the 2.1 million at m = 128.  The FP64 sums over all of
+// need one point of each orbit: 47,905 of the 2.1 million at m = 128.  The FP64 sums over all of
 // them took 20 ms of a first call's 24.
 int64_t bk_orbit_points(int m) {
     const int64_t h = m / 2 + 1;

@@ -320,11 +320,11 @@ cudaError_t ikd_any(int n, int np, const UpdateArgs& a) {
 
 }  // namespace
 
-// A tile of XC cells in x brings 4 of its own in halo cells, so the deepest tile is used that
-// still gives every SM one: 64^3 particles on 64^3 cells are 32 tiles of depth 16; their update took
-// 25.4 us at depth 16, 15.5 at 8, 11.9 at 4, and a step 27.4 us at depth 4 and 22.5 at 2.  From 152
-// tiles on depth 16 is as good or better (64^3 on 128^3, 256 tiles: 15.0 us against 16.1 and 18.5 at
-// 8 and 4; 256^3: 237, 247, 269 us).
+// Every slice of a block brings the block's box, so the deepest tile is used that still gives every SM
+// one: 64^3 particles on 64^3 cells are 32 blocks, 256 slices of depth 2.  A step takes 24.4 us with
+// those and 29.0 with 128 of depth 4; the update alone took 25.4 us with whole blocks and takes 10.6.
+// From 152 blocks on whole ones are as good or better (64^3 on 128^3, 256 blocks: 15.0 us against 16.1
+// and 18.5 at depths 8 and 4, with boxes of their own; 256^3: 237, 247, 269 us).
 int tile_depth(int R, int np, int nfields) {
     const int64_t tiles = (int64_t)nfields * (np * R / 16) * (np * R / 16) * (np * R / 32);  // of depth 16
     return tiles >= num_sms() ? 16 : 2 * tiles >= num_sms() ? 8 : 4 * tiles >= num_sms() ? 4 : 2;
